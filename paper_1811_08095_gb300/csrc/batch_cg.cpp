@@ -81,15 +81,16 @@ int BatchCG::init(Engine* e, int capacity, const odwf_solve_params& prm, cudaStr
         return rc;
     if (fsp == Sp::FF && (rc = E->ensure_links(Lk::FF18, s))) return rc;
     if (!mixed) {
-        if ((rc = E->alloc_half("cg.P64", Sp::F64, cap, &P64)) || (rc = E->alloc_half("cg.T64", Sp::F64, cap, &T64)) ||
-            (rc = E->alloc_half("cg.A64", Sp::F64, cap, &A64)) || (rc = E->alloc_half("cg.C64", Sp::F64, cap, &C64)))
+        if ((rc = E->alloc_half("cg.P64", Sp::F64, cap, &P64)) || (rc = E->alloc_half("cg.A64", Sp::FX, cap, &A64)) ||
+            (rc = E->alloc_half("cg.C64", Sp::FX, cap, &C64)))
             return rc;
     } else {
         const std::string tag = "cg.lo" + std::to_string((int)low);
         if ((rc = E->alloc_half("cg.Rin", Sp::F32, cap, &Rin)) || (rc = E->alloc_half("cg.Xin", Sp::F32, cap, &Xin)) ||
             (rc = E->alloc_half(tag + ".P", low, cap, &Pl)) || (rc = E->alloc_half(tag + ".T", low, cap, &Tl)) ||
             (rc = E->alloc_half(tag + ".A", low, cap, &Al)) || (rc = E->alloc_half(tag + ".C", low, cap, &Cl)) ||
-            (rc = E->alloc_half("cg.A1", fsp, 1, &A1)) || (rc = E->alloc_half("cg.C1", fsp, 1, &C1)))
+            (rc = E->alloc_half("cg.A1", fsp == Sp::FF ? Sp::FF : Sp::FX, 1, &A1)) ||
+            (rc = E->alloc_half("cg.C1", fsp == Sp::FF ? Sp::FF : Sp::FX, 1, &C1)))
             return rc;
         if ((rc = E->ensure_links(lk, s))) return rc;
         v2 = hop2_supported(E->ns, low, E->vh());
@@ -313,37 +314,29 @@ int BatchCG::launch_iterations(int k, int lo, int n, cudaStream_t s) {
     const size_t n5 = E->sites5();
     for (int it = 0; it < k; ++it) {
         if (!mixed) {
-            // as in the reliable update: the non-dagger hops read chi = B psi, shifted once per
-            // site into C64 (free until the third hop writes it)
-            ODWF_CK(launch_m5_f64(P64.ref(), C64.ref(), E->vh(), E->ns, r_dev, lo, n, 4, E->cf64, s, st, kRunning));
-            auto P = params<double>(1);
-            P.gate = 1;
-            P.need_status = kRunning;
-            P.sys_base = lo;
-            P.preshifted = 1;
-            P.in = C64.ref();
-            P.out = T64.ref();
-            { auto pb_ = prof_begin(pcls[0], s); P.prof_count = pb_.dev_count; ODWF_CK(launch_hop_f64(P, Epi::MINV, n, s)); prof_end(pb_, s); P.prof_count = nullptr; }
-            ODWF_CK(launch_m5_f64(T64.ref(), C64.ref(), E->vh(), E->ns, r_dev, lo, n, 4, E->cf64, s, st, kRunning));
-            P.p_out = 0;
-            P.in = C64.ref();
-            P.z = P64.ref();
-            P.out = A64.ref();
-            { auto pb_ = prof_begin(pcls[1], s); P.prof_count = pb_.dev_count; ODWF_CK(launch_hop_f64(P, Epi::SCHUR_NORM_MDINV, n, s)); prof_end(pb_, s); P.prof_count = nullptr; }
-            P.preshifted = 0;
-            P.p_out = 1;
-            P.in = A64.ref();
-            P.z = FieldRef{};
-            P.out = C64.ref();
-            { auto pb_ = prof_begin(pcls[2], s); P.prof_count = pb_.dev_count; ODWF_CK(launch_hop_f64(P, Epi::D_MINVDAG, n, s)); prof_end(pb_, s); P.prof_count = nullptr; }
-            P.p_out = 0;
-            P.in = C64.ref();
-            P.z = A64.ref();
-            P.out = FieldRef{};
-            P.cg_r = R64.ref();
-            P.cg_x = X64.ref();
-            P.cg_p = P64.ref();
-            { auto pb_ = prof_begin(pcls[3], s); P.prof_count = pb_.dev_count; ODWF_CK(launch_hop_f64(P, Epi::D_NORMAL_CG, n, s)); prof_end(pb_, s); P.prof_count = nullptr; }
+            ODWF_CK(launch_m5_fx(P64.ref(), C64.ref(), E->vh(), E->ns, r_dev, lo, n, FxOp::B, E->cf64, s, st, kRunning));
+            const FieldRef f[5] = {C64.ref(), A64.ref(), C64.ref(), A64.ref(), FieldRef{}};
+            const Epi e[4] = {Epi::MINV, Epi::SCHUR_NORM_MDINV, Epi::D_MINVDAG, Epi::D_NORMAL_CG};
+            for (int h = 0; h < 4; ++h) {
+                auto P = params<double>(1 - (h & 1));
+                P.gate = 1;
+                P.need_status = kRunning;
+                P.sys_base = lo;
+                P.in = f[h];
+                P.out = f[h + 1];
+                if (h == 1) P.z = P64.ref();
+                if (h == 3) {
+                    P.z = C64.ref();
+                    P.cg_r = R64.ref();
+                    P.cg_x = X64.ref();
+                    P.cg_p = P64.ref();
+                }
+                auto pb_ = prof_begin(pcls[h], s);
+                P.prof_count = pb_.dev_count;
+                const cudaError_t e_ = launch_hop_fx(P, e[h], n, s);
+                prof_end(pb_, s);
+                ODWF_CK(e_);
+            }
             {
                 auto pb_ = prof_begin(pcls[4], s);
                 set_vec_prof(pb_.dev_count);
@@ -555,45 +548,26 @@ int BatchCG::ff_residual(int slot, cudaStream_t s) {
 
 int BatchCG::fp64_residual(int slot, cudaStream_t s) {
     if (fsp == Sp::FF) return ff_residual(slot, s);
-    const HalfField& X = X64;
-    FieldRef t, a, c;
-    if (mixed) {
-        t = Rref();  // R is rewritten by the last hop; it holds t = M^-1 H_oe x until then
-        a = A1.ref_shared();
-        c = C1.ref_shared();
-    } else {
-        t = T64.ref();
-        a = A64.ref();
-        c = C64.ref();
+    const FieldRef a = mixed ? A1.ref_shared() : A64.ref(), c = mixed ? C1.ref_shared() : C64.ref();
+    ODWF_CK(launch_m5_fx(X64.ref(), c, E->vh(), E->ns, r_dev, slot, 1, FxOp::B, E->cf64, s));
+    const FieldRef f[5] = {c, a, c, a, Rref()};
+    const Epi e[4] = {Epi::MINV, Epi::SCHUR_MDINV, Epi::D_MINVDAG, Epi::D_NORMAL_RESID};
+    for (int h = 0; h < 4; ++h) {
+        auto P = params<double>(1 - (h & 1));
+        P.sys_base = slot;
+        P.in = f[h];
+        P.out = f[h + 1];
+        if (h == 1) P.z = X64.ref();
+        if (h == 3) {
+            P.z = c;
+            P.b = Bref();
+        }
+        auto pb_ = prof_begin(pcls_rel[h], s);
+        P.prof_count = pb_.dev_count;
+        const cudaError_t e_ = launch_hop_fx(P, e[h], 1, s);
+        prof_end(pb_, s);
+        ODWF_CK(e_);
     }
-    // The non-dagger hops read chi = B psi, shifted once per site beforehand into c (free
-    // until the third hop writes it) instead of once per neighbour inside the hop.
-    const size_t vh = E->vh();
-    ODWF_CK(launch_m5_f64(X.ref(), c, vh, E->ns, r_dev, slot, 1, 4, E->cf64, s));
-    auto P = params<double>(1);
-    P.sys_base = slot;
-    P.preshifted = 1;
-    P.in = c;
-    P.out = t;
-    { auto pb_ = prof_begin(pcls_rel[0], s); P.prof_count = pb_.dev_count; ODWF_CK(launch_hop_f64(P, Epi::MINV, 1, s)); prof_end(pb_, s); P.prof_count = nullptr; }
-    ODWF_CK(launch_m5_f64(t, c, vh, E->ns, r_dev, slot, 1, 4, E->cf64, s));
-    P.p_out = 0;
-    P.in = c;
-    P.z = X.ref();
-    P.out = a;
-    { auto pb_ = prof_begin(pcls_rel[1], s); P.prof_count = pb_.dev_count; ODWF_CK(launch_hop_f64(P, Epi::SCHUR_MDINV, 1, s)); prof_end(pb_, s); P.prof_count = nullptr; }
-    P.preshifted = 0;
-    P.p_out = 1;
-    P.in = a;
-    P.z = FieldRef{};
-    P.out = c;
-    { auto pb_ = prof_begin(pcls_rel[2], s); P.prof_count = pb_.dev_count; ODWF_CK(launch_hop_f64(P, Epi::D_MINVDAG, 1, s)); prof_end(pb_, s); P.prof_count = nullptr; }
-    P.p_out = 0;
-    P.in = c;
-    P.z = a;
-    P.b = Bref();
-    P.out = Rref();
-    { auto pb_ = prof_begin(pcls_rel[3], s); P.prof_count = pb_.dev_count; ODWF_CK(launch_hop_f64(P, Epi::D_NORMAL_RESID, 1, s)); prof_end(pb_, s); P.prof_count = nullptr; }
     return ODWF_OK;
 }
 

@@ -50,7 +50,7 @@ struct BatchCG {
 
     // per-slot fields (slabs of `cap`); in mixed mode R64 and B64 are one shared system
     HalfField X64, R64, B64;       // FP64 solution, residual, right-hand side
-    HalfField P64, T64, A64, C64;  // FP64 CG (mixed = false) operator fields
+    HalfField P64, A64, C64;       // FP64 CG (mixed = false): p and the hops' fixed-point fields
     HalfField Rin, Xin;            // mixed: FP32 inner residual / solution
     HalfField Pl, Tl, Al, Cl;      // mixed: low-precision operator fields
     HalfField Chil;                // mixed (second-generation kernels): chi_p = B p

@@ -130,6 +130,7 @@ int Engine::bounds_status(cudaStream_t st) {
 size_t Engine::half_bytes(Sp sp) const {
     switch (sp) {
         case Sp::F64: return sites5() * 192;
+        case Sp::FX: return sites5() * 192;
         case Sp::FF: return sites5() * 192;
         case Sp::F32: return sites5() * 96;
         default: return sites5() * 48;
@@ -163,7 +164,7 @@ int Engine::alloc_half(const std::string& name, Sp sp, int nsys, HalfField* f) {
     f->stride = half_bytes(sp);
     f->data = get_ws(name, f->stride * nsys, &rc);
     if (rc) return rc;
-    if (sp == Sp::F16 || sp == Sp::BF16) {
+    if (sp == Sp::F16 || sp == Sp::BF16 || sp == Sp::FX) {  // one 4-byte scale or exponent per 5D site
         f->norm_stride = norm_count();
         f->norm = (float*)get_ws(name + ".n", f->norm_stride * sizeof(float) * nsys, &rc);
         if (rc) return rc;
@@ -202,6 +203,10 @@ int Engine::set_gauge(const void* U, cudaStream_t st) {
     }
     const size_t nl = 8 * vh();
     if (!links_d18) ODWF_CK(cudaMalloc(&links_d18, nl * 144));
+    if (!nbr) {
+        ODWF_CK(cudaMalloc(&nbr, 2 * nl * sizeof(int)));
+        ODWF_CK(launch_build_neighbours(nbr, g, st));
+    }
     ODWF_CK(launch_pack_links(Ud, links_d18, nullptr, nullptr, g, st));
     // FP32 copies are derived from the FP64 ones on first use (ensure_links)
     have_f12 = have_f18 = have_h12 = have_ff18 = false;
@@ -221,10 +226,6 @@ int Engine::set_gauge(const void* U, cudaStream_t st) {
 int Engine::ensure_links(Lk lk, cudaStream_t st) {
     if (!gauge_set) return fail(ODWF_EINVAL, "gauge field not set");
     const size_t nl = 8 * vh();
-    if (!nbr) {
-        ODWF_CK(cudaMalloc(&nbr, 2 * nl * sizeof(int)));
-        ODWF_CK(launch_build_neighbours(nbr, g, st));
-    }
     if (lk == Lk::F12 && !have_f12) {
         if (!links_f12) ODWF_CK(cudaMalloc(&links_f12, nl * 48));
         ODWF_CK(launch_links_from_d18(links_d18, nullptr, links_f12, nl, st));
@@ -266,6 +267,7 @@ HopParams<double> Engine::hop_params<double>(int p_out, const double* r_dev) con
     P.lg_ns = lg_ns;
     P.p_out = p_out;
     P.links = links_d18;
+    P.nbr = nbr;
     P.r_sys = r_dev;
     P.cf = cf64;
     P.bounds_flag = bounds_flag;
@@ -306,45 +308,53 @@ HopParams<float> Engine::hop_params<float>(int p_out, const double* r_dev) const
 int Engine::apply_schur64(const HalfField& in, const HalfField& out, bool dag, const double* r_dev, cudaStream_t st) {
     int rc = 0;
     HalfField T, A;
-    if ((rc = alloc_half("op.T", Sp::F64, 1, &T)) || (rc = alloc_half("op.A", Sp::F64, 1, &A))) return rc;
-    if (!dag) {
-        auto P = hop_params<double>(1, r_dev);
-        P.in = in.ref_sys(0);
-        P.out = T.ref_sys(0);
-        ODWF_CK(launch_hop_f64(P, Epi::MINV, 1, st));
-        P = hop_params<double>(0, r_dev);
-        P.in = T.ref_sys(0);
-        P.z = in.ref_sys(0);
-        P.out = out.ref_sys(0);
-        ODWF_CK(launch_hop_f64(P, Epi::SCHUR, 1, st));
-    } else {
-        ODWF_CK(launch_m5_f64(in.ref_sys(0), A.ref_sys(0), vh(), ns, r_dev, 0, 1, 3, cf64, st));
-        auto P = hop_params<double>(1, r_dev);
-        P.in = A.ref_sys(0);
-        P.out = T.ref_sys(0);
-        ODWF_CK(launch_hop_f64(P, Epi::D_MINVDAG, 1, st));
-        P = hop_params<double>(0, r_dev);
-        P.in = T.ref_sys(0);
-        P.z = in.ref_sys(0);
-        P.out = out.ref_sys(0);
-        ODWF_CK(launch_hop_f64(P, Epi::D_ZMINUS, 1, st));
-    }
+    if ((rc = alloc_half("op.T", Sp::FX, 1, &T)) || (rc = alloc_half("op.A", Sp::FX, 1, &A))) return rc;
+    ODWF_CK(launch_m5_fx(in.ref_sys(0), A.ref_sys(0), vh(), ns, r_dev, 0, 1, dag ? FxOp::MINVDAG : FxOp::B, cf64, st));
+    auto P = hop_params<double>(1, r_dev);
+    P.in = A.ref_sys(0);
+    P.out = T.ref_sys(0);
+    ODWF_CK(launch_hop_fx(P, dag ? Epi::D_MINVDAG : Epi::MINV, 1, st));
+    P = hop_params<double>(0, r_dev);
+    P.in = T.ref_sys(0);
+    P.z = in.ref_sys(0);
+    P.out = out.ref_sys(0);
+    ODWF_CK(launch_hop_fx(P, dag ? Epi::D_ZMINUS : Epi::SCHUR, 1, st));
     return ODWF_OK;
 }
 
 int Engine::apply_full64(const HalfField& in_e, const HalfField& in_o, const HalfField& out_e,
                          const HalfField& out_o, bool dag, const double* r_dev, cudaStream_t st) {
-    const Epi e = dag ? Epi::D_FULL : Epi::FULL;
-    auto P = hop_params<double>(0, r_dev);
-    P.in = in_o.ref_sys(0);
-    P.z = in_e.ref_sys(0);
-    P.out = out_e.ref_sys(0);
-    ODWF_CK(launch_hop_f64(P, e, 1, st));
-    P = hop_params<double>(1, r_dev);
-    P.in = in_e.ref_sys(0);
-    P.z = in_o.ref_sys(0);
-    P.out = out_o.ref_sys(0);
-    ODWF_CK(launch_hop_f64(P, e, 1, st));
+    int rc = 0;
+    HalfField A;
+    if ((rc = alloc_half("op.A", Sp::FX, 1, &A))) return rc;
+    for (int p = 0; p < 2; ++p) {
+        const HalfField& other = p == 0 ? in_o : in_e;
+        ODWF_CK(launch_m5_fx(other.ref_sys(0), A.ref_sys(0), vh(), ns, r_dev, 0, 1, dag ? FxOp::ID : FxOp::B, cf64, st));
+        auto P = hop_params<double>(p, r_dev);
+        P.in = A.ref_sys(0);
+        P.z = (p == 0 ? in_e : in_o).ref_sys(0);
+        P.out = (p == 0 ? out_e : out_o).ref_sys(0);
+        ODWF_CK(launch_hop_fx(P, dag ? Epi::D_FULL : Epi::FULL, 1, st));
+    }
+    return ODWF_OK;
+}
+
+// out = S^dag S in through the four fused hops
+int Engine::apply_normal64(const HalfField& in, const HalfField& out, const double* r_dev, cudaStream_t st) {
+    int rc = 0;
+    HalfField T, A;
+    if ((rc = alloc_half("op.T", Sp::FX, 1, &T)) || (rc = alloc_half("op.A", Sp::FX, 1, &A))) return rc;
+    ODWF_CK(launch_m5_fx(in.ref_sys(0), A.ref_sys(0), vh(), ns, r_dev, 0, 1, FxOp::B, cf64, st));
+    const HalfField* f[5] = {&A, &T, &A, &T, &out};
+    const Epi e[4] = {Epi::MINV, Epi::SCHUR_MDINV, Epi::D_MINVDAG, Epi::D_NORMAL};
+    for (int k = 0; k < 4; ++k) {
+        auto P = hop_params<double>(1 - (k & 1), r_dev);
+        P.in = f[k]->ref_sys(0);
+        P.out = f[k + 1]->ref_sys(0);
+        if (k == 1) P.z = in.ref_sys(0);
+        if (k == 3) P.z = A.ref_sys(0);
+        ODWF_CK(launch_hop_fx(P, e[k], 1, st));
+    }
     return ODWF_OK;
 }
 
@@ -411,31 +421,11 @@ int Engine::apply_normal(void* out, const void* in, int system, cudaStream_t st)
     double2* dout = out_dev ? (double2*)out : (double2*)get_ws("ext.out", eb, &rc);
     if (rc) return rc;
     const double* rd = (const double*)ws["r_handle"].p;
-    HalfField Xe, Ye, T, A, C;
+    HalfField Xe, Ye;
     if ((rc = alloc_half("io.Xe", Sp::F64, 1, &Xe)) || (rc = alloc_half("io.Ye", Sp::F64, 1, &Ye))) return rc;
     if (system == ODWF_SYS_SCHUR_NORMAL) {
-        if ((rc = alloc_half("op.T", Sp::F64, 1, &T)) || (rc = alloc_half("op.A", Sp::F64, 1, &A)) ||
-            (rc = alloc_half("op.C", Sp::F64, 1, &C)))
-            return rc;
         ODWF_CK(launch_pack(Sp::F64, din, Xe.ref_sys(0), g, 0, ns, 1, st));
-        auto P = hop_params<double>(1, rd);
-        P.in = Xe.ref_sys(0);
-        P.out = T.ref_sys(0);
-        ODWF_CK(launch_hop_f64(P, Epi::MINV, 1, st));
-        P = hop_params<double>(0, rd);
-        P.in = T.ref_sys(0);
-        P.z = Xe.ref_sys(0);
-        P.out = A.ref_sys(0);
-        ODWF_CK(launch_hop_f64(P, Epi::SCHUR_MDINV, 1, st));
-        P = hop_params<double>(1, rd);
-        P.in = A.ref_sys(0);
-        P.out = C.ref_sys(0);
-        ODWF_CK(launch_hop_f64(P, Epi::D_MINVDAG, 1, st));
-        P = hop_params<double>(0, rd);
-        P.in = C.ref_sys(0);
-        P.z = A.ref_sys(0);
-        P.out = Ye.ref_sys(0);
-        ODWF_CK(launch_hop_f64(P, Epi::D_NORMAL, 1, st));
+        if ((rc = apply_normal64(Xe, Ye, rd, st))) return rc;
         ODWF_CK(launch_unpack(Sp::F64, Ye.ref_sys(0), dout, g, 0, ns, 1, st));
     } else {
         HalfField Xo, Yo, Ze, Zo;

@@ -69,7 +69,7 @@ struct Engine {
     void* links_ff18 = nullptr;  // the FP64 links as float-float pairs (reliable updates)
     void* links_site[4] = {nullptr, nullptr, nullptr, nullptr};  // site-major copies by Lk (second-generation hops)
     bool have_site[4] = {false, false, false, false};
-    int* nbr = nullptr;  // neighbour table of the second-generation hops (launch_build_neighbours)
+    int* nbr = nullptr;  // neighbour table of the hops (launch_build_neighbours), built by set_gauge
     unsigned* bounds_flag = nullptr;  // device word for the debug build's index checks
     bool gauge_set = false;
     bool have_f12 = false, have_f18 = false, have_h12 = false;  // low-precision copies of the FP64 links
@@ -110,6 +110,7 @@ struct Engine {
     int apply_schur64(const HalfField& in, const HalfField& out, bool dag, const double* r_dev, cudaStream_t st);
     int apply_full64(const HalfField& in_e, const HalfField& in_o, const HalfField& out_e, const HalfField& out_o,
                      bool dag, const double* r_dev, cudaStream_t st);
+    int apply_normal64(const HalfField& in, const HalfField& out, const double* r_dev, cudaStream_t st);  // S^dag S
 
     // C-ABI level operations
     int apply(void* out, const void* in, int mode, bool dag, cudaStream_t st);

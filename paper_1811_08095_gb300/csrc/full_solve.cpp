@@ -70,12 +70,13 @@ int Engine::solve_full(void* x, const void* b, const odwf_solve_params* prm, odw
     double2* dx = x_dev ? (double2*)x : (double2*)get_ws("ext.out", eb, &rc);
     if (rc) return rc;
 
-    HalfField Be, Bo, Re, Ro, Ye, Yo, Xe, Xo, Ee, Eo, W, U, Ze, Zo;
+    HalfField Be, Bo, Re, Ro, Ye, Yo, Xe, Xo, Ee, Eo, W, U, Ze, Zo, F;  // F: a hop's fixed-point input
     const char* names[] = {"fs.Be", "fs.Bo", "fs.Re", "fs.Ro", "fs.Ye", "fs.Yo", "fs.Xe",
                            "fs.Xo", "fs.Ee", "fs.Eo", "fs.W", "fs.U", "fs.Ze", "fs.Zo"};
     HalfField* fields[] = {&Be, &Bo, &Re, &Ro, &Ye, &Yo, &Xe, &Xo, &Ee, &Eo, &W, &U, &Ze, &Zo};
     for (int k = 0; k < 14; ++k)
         if ((rc = alloc_half(names[k], Sp::F64, 1, fields[k]))) return rc;
+    if ((rc = alloc_half("op.A", Sp::FX, 1, &F))) return rc;
     ODWF_CK(launch_pack(Sp::F64, db, Be.ref_sys(0), g, 0, ns, 0, st));
     ODWF_CK(launch_pack(Sp::F64, db, Bo.ref_sys(0), g, 1, ns, 0, st));
 
@@ -103,17 +104,24 @@ int Engine::solve_full(void* x, const void* b, const odwf_solve_params* prm, odw
         return ODWF_OK;
     };
 
+    auto to_fx = [&](const HalfField& a, FxOp op) {  // F = op(a)
+        return launch_m5_fx(a.ref_sys(0), F.ref_sys(0), vh(), ns, rd, 0, 1, op, cf64, st);
+    };
+    auto hop = [&](int p_out, Epi e, const HalfField& z, const HalfField& out) {  // out from F and z
+        auto P = hop_params<double>(p_out, rd);
+        P.in = F.ref_sys(0);
+        P.z = z.ref_sys(0);
+        P.out = out.ref_sys(0);
+        return launch_hop_fx(P, e, 1, st);
+    };
+
     // One pass of the Schur pipeline: E = A^-1 R (approximately, to the CG tolerance).
     auto solve_once = [&]() -> int {
         // Y = right-hand side of the D solve (R itself for FULL_DIRAC, D^-dag R for FULL_NORMAL)
         if (system == ODWF_SYS_FULL_NORMAL) {
-            // W = M^-dag r_o;  bc.B64 = z_e = r_e - H_oe^dag W
-            ODWF_CK(launch_m5_f64(Ro.ref_sys(0), W.ref_sys(0), vh(), ns, rd, 0, 1, 3, cf64, st));
-            auto P = hop_params<double>(0, rd);
-            P.in = W.ref_sys(0);
-            P.z = Re.ref_sys(0);
-            P.out = bc.B64.ref_sys(0);
-            ODWF_CK(launch_hop_f64(P, Epi::D_ZMINUS, 1, st));
+            // bc.B64 = z_e = r_e - H_oe^dag M^-dag r_o
+            ODWF_CK(to_fx(Ro, FxOp::MINVDAG));
+            ODWF_CK(hop(0, Epi::D_ZMINUS, Re, bc.B64));
             int s1 = 0, r1 = run_cg(bc, mqv, st, every, &iters, &nrel, &s1);
             if (r1) return r1;
             if (s1 != kDone) status = s1;
@@ -121,22 +129,15 @@ int Engine::solve_full(void* x, const void* b, const odwf_solve_params* prm, odw
             if ((r1 = apply_schur64(bc.X64, U, false, rd, st))) return r1;
             ODWF_CK(launch_m5_f64(U.ref_sys(0), Ye.ref_sys(0), vh(), ns, rd, 0, 1, 3, cf64, st));
             // y_o = M^-dag (r_o - H_eo^dag y_e)
-            P = hop_params<double>(1, rd);
-            P.in = Ye.ref_sys(0);
-            P.z = Ro.ref_sys(0);
-            P.out = Yo.ref_sys(0);
-            ODWF_CK(launch_hop_f64(P, Epi::D_ZMINUS_POSTMINVDAG, 1, st));
+            ODWF_CK(to_fx(Ye, FxOp::ID));
+            ODWF_CK(hop(1, Epi::D_ZMINUS_POSTMINVDAG, Ro, Yo));
         } else {
             ODWF_CK(copy(Re, Ye));
             ODWF_CK(copy(Ro, Yo));
         }
-        // D e = y:  W = M^-1 y_o;  U = eta~_e = M^-1 (y_e - H_eo W);  bc.B64 = S^dag U
-        ODWF_CK(launch_m5_f64(Yo.ref_sys(0), W.ref_sys(0), vh(), ns, rd, 0, 1, 2, cf64, st));
-        auto P = hop_params<double>(0, rd);
-        P.in = W.ref_sys(0);
-        P.z = Ye.ref_sys(0);
-        P.out = U.ref_sys(0);
-        ODWF_CK(launch_hop_f64(P, Epi::ZMINUS_POSTMINV, 1, st));
+        // D e = y:  U = eta~_e = M^-1 (y_e - H_eo M^-1 y_o);  bc.B64 = S^dag U
+        ODWF_CK(to_fx(Yo, FxOp::B_MINV));
+        ODWF_CK(hop(0, Epi::ZMINUS_POSTMINV, Ye, U));
         int r2 = apply_schur64(U, bc.B64, true, rd, st);
         if (r2) return r2;
         int s2 = 0;
@@ -144,11 +145,8 @@ int Engine::solve_full(void* x, const void* b, const odwf_solve_params* prm, odw
         if (s2 != kDone) status = s2;
         ODWF_CK(copy(bc.X64, Ee));
         // e_o = M^-1 (y_o - H_oe e_e)
-        P = hop_params<double>(1, rd);
-        P.in = Ee.ref_sys(0);
-        P.z = Yo.ref_sys(0);
-        P.out = Eo.ref_sys(0);
-        ODWF_CK(launch_hop_f64(P, Epi::ZMINUS_POSTMINV, 1, st));
+        ODWF_CK(to_fx(Ee, FxOp::B));
+        ODWF_CK(hop(1, Epi::ZMINUS_POSTMINV, Yo, Eo));
         return ODWF_OK;
     };
 

@@ -49,7 +49,6 @@ constexpr int EPI_SCHUR_NORM_MDINV_STORE =
 constexpr int EPI_FULL = mkflags(false, ZOP_M, OP_ID, false, 0, false, false, false, 0);           // M z + H p
 constexpr int EPI_PLAIN = mkflags(false, ZOP_NONE, OP_ID, false, 0, false, false, false, 0);       // H p
 constexpr int EPI_ZMINUS_POSTMINV = mkflags(false, ZOP_ID, OP_ID, true, OP_MINV, false, false, false, 0);  // M^-1 (z - H p)
-constexpr int EPI_ZMINUS = mkflags(false, ZOP_ID, OP_ID, true, 0, false, false, false, 0);         // z - H p
 constexpr int EPID_MINVDAG = mkflags(true, ZOP_NONE, OP_MINVDAG, false, 0, false, false, false, 0);  // M^-dag H^dag a
 constexpr int EPID_NORMAL = mkflags(true, ZOP_MDAG, OP_ID, true, 0, false, false, false, 0);         // M^dag z - H^dag c
 constexpr int EPID_NORMAL_CG =                                                                        // fused CG update
@@ -59,7 +58,6 @@ constexpr int EPID_NORMAL_RESID =                                               
 constexpr int EPID_ZMINUS = mkflags(true, ZOP_ID, OP_ID, true, 0, false, false, false, 0);           // z - H^dag c
 constexpr int EPID_FULL = mkflags(true, ZOP_MDAG, OP_ID, false, 0, false, false, false, 0);          // M^dag z + H^dag p
 constexpr int EPID_PLAIN = mkflags(true, ZOP_NONE, OP_ID, false, 0, false, false, false, 0);         // H^dag p
-constexpr int EPID_SCHUR2 = mkflags(true, ZOP_ID, OP_MINVDAG, true, 0, false, false, false, 0);      // z - M^-dag H^dag t
 constexpr int EPID_ZMINUS_POSTMINVDAG = mkflags(true, ZOP_ID, OP_ID, true, OP_MINVDAG, false, false, false, 0);
 
 // ---------------------------------------------------------------- kernel parameters

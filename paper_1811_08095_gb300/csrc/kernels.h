@@ -12,7 +12,7 @@ namespace odwf {
 constexpr int kMinReduceBlock = 64;
 
 
-enum class Sp { F64 = 0, F32 = 1, F16 = 2, BF16 = 3, FF = 4 };  // FF: float-float pairs (ff.cuh)
+enum class Sp { F64 = 0, F32 = 1, F16 = 2, BF16 = 3, FF = 4, FX = 5 };  // FF: float-float pairs (ff.cuh), FX: fx.cuh
 enum class Lk { D18 = 0, F18 = 1, F12 = 2, H12 = 3, FF18 = 4 };
 
 struct FieldRef;
@@ -28,7 +28,6 @@ enum class Epi {
     FULL,                 // M z + H p
     PLAIN,                // H p
     ZMINUS_POSTMINV,      // M^-1 (z - H p)
-    ZMINUS,               // z - H p
     D_MINVDAG,            // M^-dag H^dag a
     D_NORMAL,             // M^dag z - H^dag c
     D_NORMAL_CG,          // fused CG update (r, x, |r|^2 -> beta)
@@ -36,12 +35,19 @@ enum class Epi {
     D_ZMINUS,             // z - H^dag c
     D_FULL,               // M^dag z + H^dag p
     D_PLAIN,              // H^dag p
-    D_SCHUR2,             // z - M^-dag H^dag t
     D_ZMINUS_POSTMINVDAG, // M^-dag (z - H^dag p)
 };
 
-// FP64 path (double spinors, 18-real double links, FP64 arithmetic)
-cudaError_t launch_hop_f64(const HopParams<double>& P, Epi e, int nsys, cudaStream_t st);
+// FP64-accuracy path (kernels_fx.cuh): hops in block fixed point with FP64 links and epilogues.  P.in is
+// a fixed-point field (Sp::FX; chi = B psi for the non-dagger epilogues), P.nbr the neighbour table.
+// MINV writes B M^-1 H p, the next hop's input; MINV, SCHUR_NORM_MDINV, SCHUR_MDINV and D_MINVDAG write
+// fixed point, the others FP64; z is FP64 except for D_NORMAL, D_NORMAL_CG and D_NORMAL_RESID.
+cudaError_t launch_hop_fx(const HopParams<double>& P, Epi e, int nsys, cudaStream_t st);
+// op(in) of an FP64 field into fixed point
+enum class FxOp { ID, B, MINVDAG, B_MINV };
+cudaError_t launch_m5_fx(const FieldRef& in, const FieldRef& out, size_t n_sites, int ns, const double* r_sys,
+                         int sys_base, int nsys, FxOp op, const Coef5<double>& cf, cudaStream_t st,
+                         const SysState* gate_st = nullptr, int need = 0);
 // Float-float path (float-float fields and links, float-float arithmetic on the FP32 pipe): the
 // reliable updates of the mixed-precision CG.  Epilogues MINV, SCHUR_MDINV, D_MINVDAG, D_NORMAL,
 // D_NORMAL_RESID.

@@ -1,4 +1,4 @@
-// FP64 kernels, layout conversion, vector and gauge-packing kernels.
+// Site-local FP64 kernels, layout conversion, vector and gauge-packing kernels.
 #include "kernels.cuh"
 #include "kernels.h"
 
@@ -20,37 +20,7 @@ int lg2(int v) {
 namespace {
 constexpr int kBS = 256;
 
-template <int F>
-cudaError_t hop64(const HopParams<double>& P, int nsys, cudaStream_t st) {
-    const size_t n = (size_t)P.g.Vh * P.ns;
-    dim3 grid(blocks_for(n, kBS), nsys);
-    note_launch(); hop_kernel<SpF64, SpF64, SpF64, SpF64, LinkD18, double, F><<<grid, kBS, 0, st>>>(P);
-    return cudaGetLastError();
-}
 }  // namespace
-
-cudaError_t launch_hop_f64(const HopParams<double>& P, Epi e, int nsys, cudaStream_t st) {
-    switch (e) {
-        case Epi::MINV: return hop64<EPI_MINV>(P, nsys, st);
-        case Epi::SCHUR: return hop64<EPI_SCHUR>(P, nsys, st);
-        case Epi::SCHUR_NORM_MDINV: return hop64<EPI_SCHUR_NORM_MDINV>(P, nsys, st);
-        case Epi::SCHUR_MDINV: return hop64<EPI_SCHUR_NORM_MDINV_STORE>(P, nsys, st);
-        case Epi::FULL: return hop64<EPI_FULL>(P, nsys, st);
-        case Epi::PLAIN: return hop64<EPI_PLAIN>(P, nsys, st);
-        case Epi::ZMINUS_POSTMINV: return hop64<EPI_ZMINUS_POSTMINV>(P, nsys, st);
-        case Epi::ZMINUS: return hop64<EPI_ZMINUS>(P, nsys, st);
-        case Epi::D_MINVDAG: return hop64<EPID_MINVDAG>(P, nsys, st);
-        case Epi::D_NORMAL: return hop64<EPID_NORMAL>(P, nsys, st);
-        case Epi::D_NORMAL_CG: return hop64<EPID_NORMAL_CG>(P, nsys, st);
-        case Epi::D_NORMAL_RESID: return hop64<EPID_NORMAL_RESID>(P, nsys, st);
-        case Epi::D_ZMINUS: return hop64<EPID_ZMINUS>(P, nsys, st);
-        case Epi::D_FULL: return hop64<EPID_FULL>(P, nsys, st);
-        case Epi::D_PLAIN: return hop64<EPID_PLAIN>(P, nsys, st);
-        case Epi::D_SCHUR2: return hop64<EPID_SCHUR2>(P, nsys, st);
-        case Epi::D_ZMINUS_POSTMINVDAG: return hop64<EPID_ZMINUS_POSTMINVDAG>(P, nsys, st);
-    }
-    return cudaErrorInvalidValue;
-}
 
 cudaError_t launch_m5_f64(const FieldRef& in, const FieldRef& out, size_t n_sites, int ns, const double* r_sys,
                           int sys_base, int nsys, int op, const Coef5<double>& cf, cudaStream_t st,
@@ -72,6 +42,7 @@ cudaError_t launch_pack(Sp sp, const double2* ext, const FieldRef& out, const Ge
         case Sp::F16: note_launch(); pack_kernel<SpF16><<<grid, kBS, 0, st>>>(ext, out, g, p, ns, lg, ext_mode); break;
         case Sp::BF16: note_launch(); pack_kernel<SpBF16><<<grid, kBS, 0, st>>>(ext, out, g, p, ns, lg, ext_mode); break;
         case Sp::FF: note_launch(); pack_kernel<SpFF><<<grid, kBS, 0, st>>>(ext, out, g, p, ns, lg, ext_mode); break;
+        default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }
@@ -86,6 +57,7 @@ cudaError_t launch_unpack(Sp sp, const FieldRef& in, double2* ext, const Geom& g
         case Sp::F16: note_launch(); unpack_kernel<SpF16><<<grid, kBS, 0, st>>>(in, ext, g, p, ns, lg, ext_mode); break;
         case Sp::BF16: note_launch(); unpack_kernel<SpBF16><<<grid, kBS, 0, st>>>(in, ext, g, p, ns, lg, ext_mode); break;
         case Sp::FF: note_launch(); unpack_kernel<SpFF><<<grid, kBS, 0, st>>>(in, ext, g, p, ns, lg, ext_mode); break;
+        default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }
@@ -129,6 +101,7 @@ cudaError_t vec_y(Sp spy, const FieldRef& x, const FieldRef& y, size_t n5, int n
             if (dx) return vec_t<SX, SpBF16, double>(x, y, n5, ns, kind, coef, st, gate, need, partials, counters, part_stride, sys_base, nsys, stream);
             return vec_t<SX, SpBF16, float>(x, y, n5, ns, kind, coef, st, gate, need, partials, counters,
                                             part_stride, sys_base, nsys, stream);
+        default: break;
     }
     return cudaErrorInvalidValue;
 }
@@ -143,6 +116,7 @@ cudaError_t launch_vec(Sp spx, Sp spy, const FieldRef& x, const FieldRef& y, siz
         case Sp::F16: return vec_y<SpF16>(spy, x, y, n5, ns, kind, coef, st, gate, need, partials, counters, part_stride, sys_base, nsys, stream);
         case Sp::BF16: return vec_y<SpBF16>(spy, x, y, n5, ns, kind, coef, st, gate, need, partials, counters, part_stride, sys_base, nsys, stream);
         case Sp::FF: return vec_y<SpFF>(spy, x, y, n5, ns, kind, coef, st, gate, need, partials, counters, part_stride, sys_base, nsys, stream);
+        default: break;
     }
     return cudaErrorInvalidValue;
 }
