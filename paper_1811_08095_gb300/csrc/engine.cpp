@@ -52,6 +52,7 @@ Engine::~Engine() {
     if (links_f12) cudaFree(links_f12);
     if (links_h12) cudaFree(links_h12);
     if (links_ff18) cudaFree(links_ff18);
+    if (links_fx) cudaFree(links_fx);
     for (void* p : links_site)
         if (p) cudaFree(p);
     if (nbr) cudaFree(nbr);
@@ -107,6 +108,26 @@ int Engine::init(const odwf_lattice* l, int Ns, double m0_, double mq_, const do
     if (rc) return rc;
     const double r = mq / (2.0 * m0);
     ODWF_CK(cudaMemcpy(rd, &r, sizeof(double), cudaMemcpyHostToDevice));
+    // scan tables of the fixed-point hops' M^-1 (fx_minv): 1/d, then al and its running product for
+    // M^-1 up (forward, e_s), M^-1 down (backward, e_s), M^-dag up (backward, e_{s+1}), down (forward, e_{s-1})
+    std::vector<double> tab(cf64.inv_d, cf64.inv_d + Ns);
+    for (int v = 0; v < 4; ++v) {
+        std::vector<double> al(Ns), A(Ns);
+        for (int s = 0; s < Ns; ++s)
+            al[s] = -cf64.e[v == 2 ? (s + 1) % Ns : v == 3 ? (s + Ns - 1) % Ns : s] * cf64.inv_d[s];
+        const bool fwd = v == 0 || v == 3;
+        double prod = 1.0;
+        for (int n = 0; n < Ns; ++n) {
+            const int s = fwd ? n : Ns - 1 - n;
+            prod *= al[s];
+            A[s] = prod;
+        }
+        tab.insert(tab.end(), al.begin(), al.end());
+        tab.insert(tab.end(), A.begin(), A.end());
+    }
+    fx_tab = (double*)get_ws("fx_tab", tab.size() * sizeof(double), &rc);
+    if (rc) return rc;
+    ODWF_CK(cudaMemcpy(fx_tab, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice));
     bounds_flag = (unsigned*)get_ws("bounds_flag", sizeof(unsigned), &rc);
     if (rc) return rc;
     ODWF_CK(cudaMemset(bounds_flag, 0, sizeof(unsigned)));
@@ -207,7 +228,9 @@ int Engine::set_gauge(const void* U, cudaStream_t st) {
         ODWF_CK(cudaMalloc(&nbr, 2 * nl * sizeof(int)));
         ODWF_CK(launch_build_neighbours(nbr, g, st));
     }
+    if (!links_fx) ODWF_CK(cudaMalloc(&links_fx, nl * 148));
     ODWF_CK(launch_pack_links(Ud, links_d18, nullptr, nullptr, g, st));
+    ODWF_CK(launch_links_fx(links_d18, links_fx, nl, st));
     // FP32 copies are derived from the FP64 ones on first use (ensure_links)
     have_f12 = have_f18 = have_h12 = have_ff18 = false;
     for (bool& b : have_site) b = false;
@@ -266,7 +289,10 @@ HopParams<double> Engine::hop_params<double>(int p_out, const double* r_dev) con
     P.ns = ns;
     P.lg_ns = lg_ns;
     P.p_out = p_out;
-    P.links = links_d18;
+    P.links = links_fx;
+    P.link_ex = reinterpret_cast<const int*>(static_cast<const char*>(links_fx) + 8 * vh() * 144);
+    P.links_d = links_d18;
+    P.tab5 = fx_tab;
     P.nbr = nbr;
     P.r_sys = r_dev;
     P.cf = cf64;
@@ -309,7 +335,7 @@ int Engine::apply_schur64(const HalfField& in, const HalfField& out, bool dag, c
     int rc = 0;
     HalfField T, A;
     if ((rc = alloc_half("op.T", Sp::FX, 1, &T)) || (rc = alloc_half("op.A", Sp::FX, 1, &A))) return rc;
-    ODWF_CK(launch_m5_fx(in.ref_sys(0), A.ref_sys(0), vh(), ns, r_dev, 0, 1, dag ? FxOp::MINVDAG : FxOp::B, cf64, st));
+    ODWF_CK(launch_m5_fx(in.ref_sys(0), A.ref_sys(0), vh(), ns, r_dev, 0, 1, dag ? FxOp::MINVDAG : FxOp::B, cf64, fx_tab, st));
     auto P = hop_params<double>(1, r_dev);
     P.in = A.ref_sys(0);
     P.out = T.ref_sys(0);
@@ -329,7 +355,7 @@ int Engine::apply_full64(const HalfField& in_e, const HalfField& in_o, const Hal
     if ((rc = alloc_half("op.A", Sp::FX, 1, &A))) return rc;
     for (int p = 0; p < 2; ++p) {
         const HalfField& other = p == 0 ? in_o : in_e;
-        ODWF_CK(launch_m5_fx(other.ref_sys(0), A.ref_sys(0), vh(), ns, r_dev, 0, 1, dag ? FxOp::ID : FxOp::B, cf64, st));
+        ODWF_CK(launch_m5_fx(other.ref_sys(0), A.ref_sys(0), vh(), ns, r_dev, 0, 1, dag ? FxOp::ID : FxOp::B, cf64, fx_tab, st));
         auto P = hop_params<double>(p, r_dev);
         P.in = A.ref_sys(0);
         P.z = (p == 0 ? in_e : in_o).ref_sys(0);
@@ -344,7 +370,7 @@ int Engine::apply_normal64(const HalfField& in, const HalfField& out, const doub
     int rc = 0;
     HalfField T, A;
     if ((rc = alloc_half("op.T", Sp::FX, 1, &T)) || (rc = alloc_half("op.A", Sp::FX, 1, &A))) return rc;
-    ODWF_CK(launch_m5_fx(in.ref_sys(0), A.ref_sys(0), vh(), ns, r_dev, 0, 1, FxOp::B, cf64, st));
+    ODWF_CK(launch_m5_fx(in.ref_sys(0), A.ref_sys(0), vh(), ns, r_dev, 0, 1, FxOp::B, cf64, fx_tab, st));
     const HalfField* f[5] = {&A, &T, &A, &T, &out};
     const Epi e[4] = {Epi::MINV, Epi::SCHUR_MDINV, Epi::D_MINVDAG, Epi::D_NORMAL};
     for (int k = 0; k < 4; ++k) {

@@ -61,8 +61,11 @@ struct Engine {
     Coef5<ff> cfff{};  // the FP64 coefficients as float-float pairs (reliable updates)
     int device = 0;
 
+    double* fx_tab = nullptr;  // fifth-dimension scan tables of the fixed-point hops (in ws)
+
     // packed links
     void* links_d18 = nullptr;
+    void* links_fx = nullptr;  // the FP64 links in fixed point (fx.cuh)
     void* links_f18 = nullptr;
     void* links_f12 = nullptr;
     void* links_h12 = nullptr;

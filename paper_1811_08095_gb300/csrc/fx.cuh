@@ -11,10 +11,15 @@
 // bits beyond FP64's own rounding of it.  Components more than 2^kFxSpread below the largest of
 // their 5D site, non-finite values and denormals keep their FP64 bits instead (exponent kFxRaw);
 // sites that read such a neighbour take the FP64 arithmetic (fx_hop_slow), so nothing is lost on
-// fields of extreme range and NaN and Inf propagate as in FP64.
+// fields of extreme range and NaN and Inf propagate as in FP64.  (Components below 2^-1042 beside
+// one above 2^-958 count as zero.)
 //
-// Storage of a field: the 16-byte chunks of the FP64 layout (SpF64) holding integers, and one
-// int32 exponent per 5D site at ex[h * Ns + s].
+// A link array holds nine (re1, re0, im1, im0) records per link, rows first, in the order of the FP64
+// links ((p * 4 + mu) * Vh + h), and one exponent each behind them (kFxRaw: a non-finite link).
+//
+// Storage of a field: the 16-byte chunks of the FP64 layout (SpF64), each a complex number as
+// (re1, re0, im1, im0), and one int32 exponent per 5D site at ex[h * Ns + s].  Limbs of a sum of two
+// spins fit 32 bits without a carry.
 #pragma once
 
 #include "kernels.cuh"
@@ -26,62 +31,20 @@ constexpr int kFxZero = -(1 << 24);  // exponent of an all-zero site (never the 
 constexpr int kFxSpread = 32;        // largest exponent range of a site's nonzero components
 constexpr int kFxMinField = 64;      // smallest biased exponent of a site's largest component
 
-// (m << up) >> down of the 53-bit significand of d, down = emax - exponent of d, with d's sign
+// (m << UP) >> (emax - exponent of d) of the 53-bit significand m of d, with d's sign.  A zero has
+// exponent field 0 and is shifted out (shr.u64 clamps), emax being at least kFxMinField.
 template <int UP>
 __device__ __forceinline__ long long fx_from_double(double d, int emax) {
     const int hi = __double2hiint(d);
-    const unsigned long long m =
+    unsigned long long m =
         ((unsigned long long)((unsigned)(hi & 0xfffff) | 0x100000u) << 32) | (unsigned)__double2loint(d);
-    const int down = min(emax - ((hi >> 20) & 0x7ff), 63);
-    const long long q = (long long)((m << UP) >> down);
+    const int down = emax - ((hi & 0x7fffffff) >> 20);
+    asm("shr.u64 %0, %1, %2;" : "=l"(m) : "l"(m << UP), "r"(down));
     const long long s = (long long)(hi >> 31);
-    return (q ^ s) - s;
+    return ((long long)m ^ s) - s;
 }
 
-__device__ __forceinline__ void fx_store(void* base, int* ex, size_t h, int s, int ns, const double v[24]) {
-    int mx = 0, mn = 0x7fffffff;
-#pragma unroll
-    for (int k = 0; k < 24; ++k) {
-        const int hi = __double2hiint(v[k]) & 0x7fffffff;
-        mx = max(mx, hi);
-        mn = min(mn, (hi | __double2loint(v[k])) == 0 ? 0x7fffffff : hi);
-    }
-    const int emax = mx >> 20, emin = mn >> 20;
-    longlong2* p = reinterpret_cast<longlong2*>(base);
-    if (mn != 0x7fffffff && (emax == 0x7ff || emax < kFxMinField || emax - emin > kFxSpread)) {
-        for (int k = 0; k < 12; ++k)
-            p[chunk_off(h, k, 12, ns, s)] =
-                make_longlong2(__double_as_longlong(v[2 * k]), __double_as_longlong(v[2 * k + 1]));
-        ex[h * ns + s] = kFxRaw;
-        return;
-    }
-    const int e = mn == 0x7fffffff ? 2046 : emax;  // an all-zero site: every significand shifted out
-#pragma unroll
-    for (int k = 0; k < 12; ++k)
-        p[chunk_off(h, k, 12, ns, s)] = make_longlong2(fx_from_double<6>(v[2 * k], e), fx_from_double<6>(v[2 * k + 1], e));
-    ex[h * ns + s] = mn == 0x7fffffff ? kFxZero : emax - 1081;  // 1023 + 52 + 6
-}
-
-// q 2^e for |q| < 2^63; the exponent is added to the converted double's where no result can leave
-// the normal range
-__device__ __forceinline__ double fx_to_double(long long q, int e) {
-    const double d = __ll2double_rn(q);
-    if (e < -1000 || e > 950) return q == 0 ? 0.0 : ldexp(d, max(e, -4000));
-    return __hiloint2double(__double2hiint(d) + (q == 0 ? 0 : e << 20), __double2loint(d));
-}
-
-__device__ __forceinline__ void fx_load_double(const void* base, const int* ex, size_t h, int s, int ns, double v[24]) {
-    const longlong2* p = reinterpret_cast<const longlong2*>(base);
-    const int e = __ldg(ex + h * ns + s);
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        const longlong2 q = __ldg(p + chunk_off(h, k, 12, ns, s));
-        v[2 * k] = e == kFxRaw ? __longlong_as_double(q.x) : fx_to_double(q.x, e);
-        v[2 * k + 1] = e == kFxRaw ? __longlong_as_double(q.y) : fx_to_double(q.y, e);
-    }
-}
-
-// One real of a half spinor as limbs
+// One real as limbs
 struct FxLimbs {
     int hi, lo;
 };
@@ -92,10 +55,71 @@ __device__ __forceinline__ FxLimbs fx_split(long long q) {
     return l;
 }
 
-__device__ __forceinline__ long long fx_mad(int a, int b, long long c) {
-    long long d;
-    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
-    return d;
+__device__ __forceinline__ long long fx_join(int hi, int lo) { return ((long long)hi << 31) + lo; }
+
+__device__ __forceinline__ void fx_store(void* base, int* ex, size_t h, int s, int ns, const double v[24]) {
+    int mx = 0;
+    unsigned mn = 0xffffffffu;  // smallest high word of a nonzero component, less one
+#pragma unroll
+    for (int k = 0; k < 24; ++k) {
+        const int hi = __double2hiint(v[k]) & 0x7fffffff;
+        mx = max(mx, hi);
+        mn = min(mn, (unsigned)(hi - 1));
+    }
+    const int emax = mx >> 20, emin = (int)((mn + 1) >> 20);
+    int4* p = reinterpret_cast<int4*>(base);
+    bool zero = false;
+    if (emax == 0x7ff || emax < kFxMinField || (mn != 0xffffffffu && emax - emin > kFxSpread)) {
+        zero = true;
+        for (int k = 0; k < 24; ++k) zero = zero && v[k] == 0.0;
+        if (!zero) {
+            for (int k = 0; k < 12; ++k)
+                p[chunk_off(h, k, 12, ns, s)] = make_int4(__double2hiint(v[2 * k]), __double2loint(v[2 * k]),
+                                                          __double2hiint(v[2 * k + 1]), __double2loint(v[2 * k + 1]));
+            ex[h * ns + s] = kFxRaw;
+            return;
+        }
+    }
+    const int e = zero ? 2046 : emax;  // an all-zero site: every significand shifted out
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const FxLimbs re = fx_split(fx_from_double<6>(v[2 * k], e)), im = fx_split(fx_from_double<6>(v[2 * k + 1], e));
+        p[chunk_off(h, k, 12, ns, s)] = make_int4(re.hi, re.lo, im.hi, im.lo);
+    }
+    ex[h * ns + s] = zero ? kFxZero : emax - 1081;  // 1023 + 52 + 6
 }
+
+// q 2^e, the exponent added to the converted double's; |q| < 2^63 and kFxMinExp <= e <= kFxMaxExp for
+// a hop's sums, |q| < 2^59 and any exponent of a stored site: no result leaves the normal range
+constexpr int kFxMinExp = -1000, kFxMaxExp = 950;
+__device__ __forceinline__ double fx_to_double(long long q, int e) {
+    const double d = __ll2double_rn(q);
+    const int hi = __double2hiint(d);
+    return __hiloint2double(hi == 0 ? 0 : hi + (e << 20), __double2loint(d));
+}
+
+__device__ __forceinline__ void fx_load_double(const void* base, const int* ex, size_t h, int s, int ns, double v[24]) {
+    const int4* p = reinterpret_cast<const int4*>(base);
+    const int e = __ldg(ex + h * ns + s);
+    int4 q[12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) q[k] = __ldg(p + chunk_off(h, k, 12, ns, s));
+    if (e == kFxRaw) {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            v[2 * k] = __hiloint2double(q[k].x, q[k].y);
+            v[2 * k + 1] = __hiloint2double(q[k].z, q[k].w);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            v[2 * k] = fx_to_double(fx_join(q[k].x, q[k].y), e);
+            v[2 * k + 1] = fx_to_double(fx_join(q[k].z, q[k].w), e);
+        }
+    }
+}
+
+// 64-bit accumulation of a 32 x 32-bit product (one instruction)
+__device__ __forceinline__ long long fx_mad(int a, int b, long long c) { return (long long)a * b + c; }
 
 }  // namespace odwf

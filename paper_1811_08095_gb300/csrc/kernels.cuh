@@ -91,6 +91,9 @@ struct HopParams {
     unsigned* counters;         // [sys]
     int sys_base;               // system index offset (blockIdx.y + sys_base)
     unsigned long long* prof_count;  // optional: counts running (system, launch) pairs
+    const double* tab5;              // fixed-point hops: fifth-dimension scan tables (Engine::init)
+    const int* link_ex;              // fixed-point hops: the links' exponents
+    const void* links_d;             // fixed-point hops: the FP64 links
     unsigned* bounds_flag;           // debug builds: where out-of-range indices are recorded
     Coef5<R> cf;
 };

@@ -46,8 +46,10 @@ cudaError_t launch_hop_fx(const HopParams<double>& P, Epi e, int nsys, cudaStrea
 // op(in) of an FP64 field into fixed point
 enum class FxOp { ID, B, MINVDAG, B_MINV };
 cudaError_t launch_m5_fx(const FieldRef& in, const FieldRef& out, size_t n_sites, int ns, const double* r_sys,
-                         int sys_base, int nsys, FxOp op, const Coef5<double>& cf, cudaStream_t st,
-                         const SysState* gate_st = nullptr, int need = 0);
+                         int sys_base, int nsys, FxOp op, const Coef5<double>& cf, const double* tab5,
+                         cudaStream_t st, const SysState* gate_st = nullptr, int need = 0);
+// the fixed-point link array of n_links FP64 links: 144 bytes per link, then an int exponent per link
+cudaError_t launch_links_fx(const void* d18, void* fx, size_t n_links, cudaStream_t st);
 // Float-float path (float-float fields and links, float-float arithmetic on the FP32 pipe): the
 // reliable updates of the mixed-precision CG.  Epilogues MINV, SCHUR_MDINV, D_MINVDAG, D_NORMAL,
 // D_NORMAL_RESID.

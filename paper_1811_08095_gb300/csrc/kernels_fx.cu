@@ -22,8 +22,10 @@ cudaError_t launch_hop_fx(const HopParams<double>& P, Epi e, int nsys, cudaStrea
 // out = op(in) of an FP64 field into the fixed-point format
 __global__ void __launch_bounds__(128) m5_fx_kernel(FieldRef in, FieldRef out, size_t n_sites, int ns, int lg_ns,
                                                     const double* r_sys, int sys_base, FxOp op,
-                                                    const __grid_constant__ Coef5<double> cf, const SysState* gate_st,
-                                                    int need) {
+                                                    const __grid_constant__ Coef5<double> cf, const double* tab5,
+                                                    const SysState* gate_st, int need) {
+    extern __shared__ __align__(16) double s_cols[];
+    __shared__ double s_fac;
     const int sys = blockIdx.y + sys_base;
     if (gate_st && gate_st[sys].status != need) return;
     const size_t gi = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -38,18 +40,69 @@ __global__ void __launch_bounds__(128) m5_fx_kernel(FieldRef in, FieldRef out, s
 #pragma unroll
         for (int k = 0; k < 24; ++k) v[k] = 0.0;
     }
-    if (op == FxOp::MINVDAG) minv_apply(v, cf, r, s, ns, true);
-    if (op == FxOp::B_MINV) minv_apply(v, cf, r, s, ns, false);
+    if (op == FxOp::MINVDAG || op == FxOp::B_MINV) {
+        if (threadIdx.x == 0) s_fac = fx_corner(tab5, r, ns);
+        __syncthreads();
+        fx_minv(v, s_cols, tab5, s_fac, s, ns, lg_ns, op == FxOp::MINVDAG);
+    }
     if (op == FxOp::B || op == FxOp::B_MINV) fx_bidiag(v, cf.rho, cf.sigma, r, s, ns, false);
     if (valid) fx_store(out.d(sys), reinterpret_cast<int*>(out.n(sys)), h, s, ns, v);
 }
 
 cudaError_t launch_m5_fx(const FieldRef& in, const FieldRef& out, size_t n_sites, int ns, const double* r_sys,
-                         int sys_base, int nsys, FxOp op, const Coef5<double>& cf, cudaStream_t st,
-                         const SysState* gate_st, int need) {
+                         int sys_base, int nsys, FxOp op, const Coef5<double>& cf, const double* tab5,
+                         cudaStream_t st, const SysState* gate_st, int need) {
+    const size_t n = n_sites * ns;
+    const int bs = fx_threads(n, ns);
+    const size_t smem = op == FxOp::MINVDAG || op == FxOp::B_MINV ? fx_smem(bs, ns, false) : 0;
     note_launch();
-    m5_fx_kernel<<<dim3(blocks_for(n_sites * ns, 128), nsys), 128, 0, st>>>(in, out, n_sites, ns, lg2(ns), r_sys,
-                                                                            sys_base, op, cf, gate_st, need);
+    m5_fx_kernel<<<dim3(blocks_for(n, bs), nsys), bs, smem, st>>>(in, out, n_sites, ns, lg2(ns), r_sys, sys_base, op,
+                                                                  cf, tab5, gate_st, need);
+    return cudaGetLastError();
+}
+
+// FP64 links into fixed point (fx.cuh), one thread per link.  The exponent leaves room for eight
+// directions in a 63-bit sum: with the largest entry below 2^e and every row and column sum of
+// |re| + |im| at most 2.5 2^e (SU(3): sqrt 6), a product component stays below 5 times the
+// neighbour's largest.
+__global__ void __launch_bounds__(128) links_fx_kernel(const double2* __restrict__ d18, int4* __restrict__ out,
+                                                       int* __restrict__ ex, size_t n) {
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    double2 u[9];
+    int mx = 0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        u[k] = d18[i * 9 + k];
+        mx = max(mx, max(__double2hiint(u[k].x) & 0x7fffffff, __double2hiint(u[k].y) & 0x7fffffff));
+    }
+    const int emax = mx >> 20;
+    const bool raw = emax == 0x7ff || (emax < kFxMinField && mx > 0);  // non-finite, or below 2^-958
+    const int e = emax < kFxMinField ? 2046 : emax;                    // a zero link: everything shifted out
+    long long q[18];
+    unsigned row[3] = {0, 0, 0}, col[3] = {0, 0, 0};
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        q[2 * k] = fx_from_double<7>(u[k].x, e);
+        q[2 * k + 1] = fx_from_double<7>(u[k].y, e);
+        const unsigned a = (unsigned)abs((int)(q[2 * k] >> 31)) + (unsigned)abs((int)(q[2 * k + 1] >> 31));
+        row[k / 3] += a;
+        col[k % 3] += a;
+    }
+    const unsigned big = max(max(max(row[0], row[1]), row[2]), max(max(col[0], col[1]), col[2]));
+    const int more = big > 1342177280u ? 2 : 0;  // 2.5 x 2^29
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const FxLimbs re = fx_split(q[2 * k] >> more), im = fx_split(q[2 * k + 1] >> more);
+        out[i * 9 + k] = make_int4(re.hi, re.lo, im.hi, im.lo);
+    }
+    ex[i] = raw ? kFxRaw : emax < kFxMinField ? kFxZero : emax - 1022 + more;
+}
+
+cudaError_t launch_links_fx(const void* d18, void* fx, size_t n_links, cudaStream_t st) {
+    note_launch();
+    links_fx_kernel<<<blocks_for(n_links, 128), 128, 0, st>>>((const double2*)d18, (int4*)fx,
+                                                              (int*)((char*)fx + n_links * 144), n_links);
     return cudaGetLastError();
 }
 

@@ -2,10 +2,11 @@
 // kernels.cuh with its epilogues.  The input is a fixed-point field; a non-dagger hop reads
 // chi = B psi, shifted once per site by the kernel that produced it.
 //
-// What bounds it: the FP64 pipe of the epilogues (conversions and the fifth-dimension operators,
-// 200 to 400 operations per 5D site at 2 per clock and SM) and the integer pipe of the stencil
-// (about 3000 operations at 64 per clock and SM), which overlap across warps.  The FP64 stencil it
-// replaces needed 1334 to 1700 FP64 operations per 5D site.
+// What bounds it: the FP64 pipe of the epilogues (about 130 to 220 operations per 5D site at 2 per
+// clock and SM: 42 to 60% busy) and the latency of the integer stencil (1728 multiply-adds at 32 per
+// clock and SM) with the 12 warps per SM that 168 registers leave.  16^3x32x16, one system, the four
+// hops of S^dag S: 0.57 / 0.69 / 0.61 / 0.49 ms; the FP64 stencil they replace, 1334 to 1700 FP64
+// operations per 5D site, took 2.6 to 3.0 ms each.  Four blocks per SM (128 registers) spill.
 #pragma once
 
 #include "fx.cuh"
@@ -39,21 +40,67 @@ __device__ __forceinline__ void fx_bidiag(double v[24], const double* a, const d
     }
 }
 
-// ---------------------------------------------------------------- the stencil
-// (1 + sg gamma_mu) projection of the colour c in integers: h = up + sg G dn for both spins
-template <int MU, bool PLUS>
-__device__ __forceinline__ void fx_project(const longlong2& u0, const longlong2& u1, const longlong2& d0,
-                                           const longlong2& d1, long long h[4]) {
-    // G d: mu 0 (-i d1, -i d0), 1 (-d1, d0), 2 (-i d0, i d1), 3 (d0, d1)
-    long long g[4];
-    bool n[4];  // whether G d enters with a minus sign
-    if (MU == 0) { g[0] = d1.y; g[1] = d1.x; g[2] = d0.y; g[3] = d0.x; n[0] = false; n[1] = true; n[2] = false; n[3] = true; }
-    else if (MU == 1) { g[0] = d1.x; g[1] = d1.y; g[2] = d0.x; g[3] = d0.y; n[0] = true; n[1] = true; n[2] = false; n[3] = false; }
-    else if (MU == 2) { g[0] = d0.y; g[1] = d0.x; g[2] = d1.y; g[3] = d1.x; n[0] = false; n[1] = true; n[2] = true; n[3] = false; }
-    else { g[0] = d0.x; g[1] = d0.y; g[2] = d1.x; g[3] = d1.y; n[0] = n[1] = n[2] = n[3] = false; }
-    const long long u[4] = {u0.x, u0.y, u1.x, u1.y};
+// ---------------------------------------------------------------- M^-1 along s
+// The cyclic bidiagonal solves of minv_apply as serial recurrences: the block's spinors are turned
+// in shared memory so that a thread walks the Ns values of one real of one site, w = inv_d v + al w,
+// then adds A fac w_last (the corner).  Three FP64 operations per real against six of the log2 Ns
+// shuffle scan, and the division of fac once per block.
+//   tab: inv_d[Ns], then for each of the four recurrences (M^-1 up, M^-1 down, M^-dag up, M^-dag down)
+//   al[Ns] = -c_s / d_s and A[Ns], its running product in the order of the recurrence.
+// buf: (blockDim / Ns) * 24 columns of Ns + 1 doubles.  Every thread of the block must call.
+__device__ __forceinline__ void fx_minv(double v[24], double* buf, const double* tab, double fac, int s, int ns,
+                                        int lg_ns, bool dag) {
+    double* mine = buf + (size_t)(threadIdx.x >> lg_ns) * 24 * (ns + 1) + s;
+    __syncthreads();
 #pragma unroll
-    for (int i = 0; i < 4; ++i) h[i] = (n[i] == PLUS) ? u[i] - g[i] : u[i] + g[i];
+    for (int k = 0; k < 24; ++k) mine[k * (ns + 1)] = v[k];
+    __syncthreads();
+    const int ncol = (blockDim.x >> lg_ns) * 24;
+    // with 1.5 columns per thread, alternate blocks give the second one to the other warps (schedulers)
+    for (int c = threadIdx.x ^ ((blockIdx.x & 1) * (blockDim.x >> 1)); c < ncol; c += blockDim.x) {
+        const int down = (c % 24) >= 12;
+        const double* al = tab + ns * (1 + 2 * ((dag ? 2 : 0) + down));
+        const int step = (down != 0) == dag ? 1 : -1;  // M^-1: up forward, down backward; M^-dag the reverse
+        int i = step > 0 ? 0 : ns - 1;
+        double* p = buf + c * (ns + 1);
+        double w = 0.0;
+#pragma unroll 8
+        for (int n = 0; n < ns; ++n, i += step) {
+            w = fma(__ldg(al + i), w, __ldg(tab + i) * p[i]);
+            p[i] = w;
+        }
+        const double wc = fac * w;
+        for (int n = 0; n < ns; ++n) p[n] = fma(__ldg(al + ns + n), wc, p[n]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 24; ++k) v[k] = mine[k * (ns + 1)];
+}
+
+// fac = -r / (1 + r A_last); A_last, the product of all al, is the same for the four recurrences
+__device__ __forceinline__ double fx_corner(const double* tab, double r, int ns) {
+    return -r / fma(r, __ldg(tab + 3 * ns - 1), 1.0);
+}
+
+// ---------------------------------------------------------------- the stencil
+// (1 + sg gamma_mu) projection of one colour, limb by limb: h = up + sg G dn for both spins,
+// (h0.re, h0.im, h1.re, h1.im); |h| < 2^60
+template <int MU, bool PLUS>
+__device__ __forceinline__ void fx_project(const int4& u0, const int4& u1, const int4& d0, const int4& d1,
+                                           FxLimbs h[4]) {
+    const FxLimbs u[4] = {{u0.x, u0.y}, {u0.z, u0.w}, {u1.x, u1.y}, {u1.z, u1.w}};
+    const FxLimbs d[4] = {{d0.x, d0.y}, {d0.z, d0.w}, {d1.x, d1.y}, {d1.z, d1.w}};
+    // G d: mu 0 (-i d1, -i d0), 1 (-d1, d0), 2 (-i d0, i d1), 3 (d0, d1): source real and whether it
+    // enters with a minus sign
+    constexpr int src[4][4] = {{3, 2, 1, 0}, {2, 3, 0, 1}, {1, 0, 3, 2}, {0, 1, 2, 3}};
+    constexpr bool neg[4][4] = {{false, true, false, true}, {true, true, false, false}, {false, true, true, false},
+                                {false, false, false, false}};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const FxLimbs g = d[src[MU][i]];
+        h[i].hi = (neg[MU][i] == PLUS) ? u[i].hi - g.hi : u[i].hi + g.hi;
+        h[i].lo = (neg[MU][i] == PLUS) ? u[i].lo - g.lo : u[i].lo + g.lo;
+    }
 }
 
 // lower spins of the colour: acc += sg G^dag w, w = (w0, w1) complex
@@ -75,17 +122,14 @@ __device__ __forceinline__ void fx_lower(const long long w[4], long long& a0r, l
 
 // One direction: acc += [w ; sg G^dag w], w = (U h) >> sh, U staged as nine (re1, re0, im1, im0)
 template <int MU, bool PLUS>
-__device__ __forceinline__ void fx_dir(const longlong2* __restrict__ p, int ns, const int4* U, int sh,
+__device__ __forceinline__ void fx_dir(const int4* __restrict__ p, int ns, const int4* U, int sh,
                                        long long acc[24]) {
     FxLimbs h[3][4];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const longlong2 u0 = __ldg(p + c * ns), u1 = __ldg(p + (3 + c) * ns), d0 = __ldg(p + (6 + c) * ns),
-                        d1 = __ldg(p + (9 + c) * ns);
-        long long t[4];
-        fx_project<MU, PLUS>(u0, u1, d0, d1, t);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) h[c][i] = fx_split(t[i]);
+        const int4 u0 = __ldg(p + c * ns), u1 = __ldg(p + (3 + c) * ns), d0 = __ldg(p + (6 + c) * ns),
+                   d1 = __ldg(p + (9 + c) * ns);
+        fx_project<MU, PLUS>(u0, u1, d0, d1, h[c]);
     }
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -130,7 +174,7 @@ static __device__ __noinline__ void fx_hop_slow(const HopParams<double>& P, cons
         project(mu, sg, v, hp);
         const size_t idx = (j & 1) == 0 ? ((size_t)(P.p_out * 4 + mu) * P.g.Vh + h)
                                         : ((size_t)((1 - P.p_out) * 4 + mu) * P.g.Vh + hn);
-        LinkIO<LinkD18, double>::load(P.links, idx, u);
+        LinkIO<LinkD18, double>::load(P.links_d, idx, u);
         su3_mul(u, hp, w, (j & 1) != 0);
         if (raw < 0)
             for (int k = 0; k < 12; ++k) w[k] = -w[k];
@@ -138,42 +182,9 @@ static __device__ __noinline__ void fx_hop_slow(const HopParams<double>& P, cons
     }
 }
 
-// Link d of a site into shared memory: the FP64 link (its adjoint for a backward hop, negated across
-// the antiperiodic boundary) as limbs; returns its exponent (kFxRaw for a non-finite link).
-// The exponent leaves room for eight directions in a 63-bit sum: with the largest entry below 2^eu
-// and every row and column sum of |re| + |im| at most 2.5 2^eu (SU(3): sqrt 6), a product component
-// stays below 5 times the neighbour's largest.
-__device__ __forceinline__ int fx_stage_link(const void* links, size_t idx, bool adj, bool neg, int4* dst) {
-    const double2* p = reinterpret_cast<const double2*>(reinterpret_cast<const char*>(links) + idx * 144);
-    double2 u[9];
-    int mx = 0;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        u[k] = __ldg(p + k);
-        mx = max(mx, max(__double2hiint(u[k].x) & 0x7fffffff, __double2hiint(u[k].y) & 0x7fffffff));
-    }
-    const int emax = mx >> 20;
-    if (emax == 0x7ff) return kFxRaw;
-    const int e = emax < kFxMinField ? 2046 : emax;  // a link below 2^-958: nothing survives the shift
-    long long q[18];
-    unsigned row[3] = {0, 0, 0}, col[3] = {0, 0, 0};
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        q[2 * k] = fx_from_double<7>(u[k].x, e);
-        q[2 * k + 1] = fx_from_double<7>(u[k].y, e);
-        const unsigned a = (unsigned)abs((int)(q[2 * k] >> 31)) + (unsigned)abs((int)(q[2 * k + 1] >> 31));
-        row[k / 3] += a;
-        col[k % 3] += a;
-    }
-    const unsigned big = max(max(max(row[0], row[1]), row[2]), max(max(col[0], col[1]), col[2]));
-    const int more = big > 1342177280u ? 2 : 0;  // 2.5 x 2^29
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        const FxLimbs re = fx_split((neg ? -q[2 * k] : q[2 * k]) >> more);
-        const FxLimbs im = fx_split((neg != adj ? -q[2 * k + 1] : q[2 * k + 1]) >> more);
-        dst[adj ? 3 * (k % 3) + k / 3 : k] = make_int4(re.hi, re.lo, im.hi, im.lo);
-    }
-    return emax < kFxMinField ? kFxZero : emax - 1022 + more;
+// index of the link of direction j at site h (parity p_out) with neighbour hn
+__device__ __forceinline__ size_t fx_link_index(const HopParams<double>& P, int j, int h, int hn) {
+    return (j & 1) ? (size_t)((1 - P.p_out) * 4 + (j >> 1)) * P.g.Vh + hn : (size_t)(P.p_out * 4 + (j >> 1)) * P.g.Vh + h;
 }
 
 template <int F>
@@ -203,39 +214,39 @@ __global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) hop_fx_kernel(const 
     const double r = P.r_sys[sys];
 
     int nb[8];
-    unsigned flip = 0;
     {
         const int4* tp = reinterpret_cast<const int4*>(P.nbr + ((size_t)P.p_out * P.g.Vh + h) * 8);
         const int4 n0 = __ldg(tp), n1 = __ldg(tp + 1);
         const int raw[8] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w};
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            nb[j] = checked_index(raw[j] & 0x7fffffff, P.g.Vh, P.bounds_flag, kBoundsNeighbour);
-            flip |= ((unsigned)raw[j] >> 31) << j;
-        }
+        for (int j = 0; j < 8; ++j) nb[j] = checked_index(raw[j] & 0x7fffffff, P.g.Vh, P.bounds_flag, kBoundsNeighbour);
     }
-    // the site's eight links: lane d of its group stages links d, d + ns, ...
+    // the site's eight links into shared memory, 72 elements over its Ns lanes: the adjoint for a
+    // backward hop, negated (the -1 of -1/2 W) except across the antiperiodic boundary
     int4* my_links = s_links + (threadIdx.x >> P.lg_ns) * kFxSite;
-    int* s_eu = reinterpret_cast<int*>(s_links + (blockDim.x >> P.lg_ns) * kFxSite) + (threadIdx.x >> P.lg_ns) * 8;
-#pragma unroll 1
-    for (int d = s; d < 8; d += ns) {
-        int hn = nb[0];
-#pragma unroll
-        for (int j = 1; j < 8; ++j) hn = d == j ? nb[j] : hn;
+    const int4* lk = reinterpret_cast<const int4*>(P.links);
+    for (int i = s; i < 72; i += ns) {
+        const int d = i / 9, k = i - 9 * d;
+        const int raw = __ldg(P.nbr + ((size_t)P.p_out * P.g.Vh + h) * 8 + d);
         const bool back = d & 1;
-        const size_t idx = back ? ((size_t)((1 - P.p_out) * 4 + (d >> 1)) * P.g.Vh + hn)
-                                : ((size_t)(P.p_out * 4 + (d >> 1)) * P.g.Vh + h);
-        s_eu[d] = fx_stage_link(P.links, idx, back, (flip >> d) & 1, my_links + d * 9);
+        const size_t idx = fx_link_index(P, d, h, checked_index(raw & 0x7fffffff, P.g.Vh, P.bounds_flag, kBoundsNeighbour));
+        int4 u = __ldg(lk + idx * 9 + k);
+        if (raw >= 0) u = make_int4(-u.x, -u.y, -u.z, -u.w);
+        if (back) {
+            u.z = -u.z;
+            u.w = -u.w;
+        }
+        my_links[9 * d + (back ? 3 * (k % 3) + k / 3 : k)] = u;
     }
     __syncwarp();
 
-    const longlong2* in = reinterpret_cast<const longlong2*>(P.in.d(sys)) + chunk_slot(s, ns);
+    const int4* in = reinterpret_cast<const int4*>(P.in.d(sys)) + chunk_slot(s, ns);
     const int* ex = reinterpret_cast<const int*>(P.in.n(sys));
     int e[8], M = kFxZero;
     bool slow = false;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-        const int en = __ldg(ex + (size_t)nb[j] * ns + s), eu = s_eu[j];
+        const int en = __ldg(ex + (size_t)nb[j] * ns + s), eu = __ldg(P.link_ex + fx_link_index(P, j, h, nb[j]));
         slow |= en == kFxRaw || eu == kFxRaw;
         e[j] = en + eu;
         M = max(M, e[j]);
@@ -251,20 +262,29 @@ __global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) hop_fx_kernel(const 
     ODWF_FX_DIR(2, 0); ODWF_FX_DIR(2, 1);
     ODWF_FX_DIR(3, 0); ODWF_FX_DIR(3, 1);
 #undef ODWF_FX_DIR
-    // -1/2 W psi (or -1/2 W^dag psi): acc 2^(M + 2), halved and negated in the exponent and sign
+    // -1/2 W psi (or -1/2 W^dag psi) = acc 2^(M + 2) / 2
     double v[24];
 #pragma unroll
-    for (int k = 0; k < 24; ++k) v[k] = fx_to_double(-acc[k], M + 1);
-    if (slow) {
+    for (int k = 0; k < 24; ++k) v[k] = fx_to_double(acc[k], M + 1);
+    if (slow || ((M < kFxMinExp || M >= kFxMaxExp) && M > kFxZero / 2)) {
         double y[24];
         fx_hop_slow(P, P.in.d(sys), ex, h, s, DAG, y);
 #pragma unroll
         for (int k = 0; k < 24; ++k) v[k] = -0.5 * y[k];
     }
 
+    // the links are read: their shared memory now holds the recurrences of M^-1 (fx_minv)
+    double* buf = reinterpret_cast<double*>(s_links);
+    __shared__ double s_fac;
+    if (HOPOP != OP_ID || POST != 0) {
+        if (threadIdx.x == 0) s_fac = fx_corner(P.tab5, r, ns);
+        __syncthreads();
+    }
+    const double fac = s_fac;
+
     if (DAG) fx_bidiag(v, P.cf.rho, P.cf.sigma, r, s, ns, true);  // B^dag: H^dag psi
-    if (HOPOP == OP_MINV) minv_apply(v, P.cf, r, s, ns, false);
-    if (HOPOP == OP_MINVDAG) minv_apply(v, P.cf, r, s, ns, true);
+    if (HOPOP == OP_MINV) fx_minv(v, buf, P.tab5, fac, s, ns, P.lg_ns, false);
+    if (HOPOP == OP_MINVDAG) fx_minv(v, buf, P.tab5, fac, s, ns, P.lg_ns, true);
     if (ZOP != ZOP_NONE) {
         double z[24];
         if (F & FX_ZFX) fx_load_double(P.z.d(sys), reinterpret_cast<const int*>(P.z.n(sys)), (size_t)h, s, ns, z);
@@ -279,8 +299,8 @@ __global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) hop_fx_kernel(const 
 #pragma unroll
         for (int k = 0; k < 24; ++k) nrm = fma(v[k], v[k], nrm);
     }
-    if (POST == OP_MINV) minv_apply(v, P.cf, r, s, ns, false);
-    if (POST == OP_MINVDAG) minv_apply(v, P.cf, r, s, ns, true);
+    if (POST == OP_MINV) fx_minv(v, buf, P.tab5, fac, s, ns, P.lg_ns, false);
+    if (POST == OP_MINVDAG) fx_minv(v, buf, P.tab5, fac, s, ns, P.lg_ns, true);
     if (F & FX_OUTB) fx_bidiag(v, P.cf.rho, P.cf.sigma, r, s, ns, false);
 
     if (valid) {
@@ -320,14 +340,19 @@ __global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) hop_fx_kernel(const 
 // Threads per block: 128, or 64 while that leaves fewer than two blocks for each of the 152 SMs
 // (a small lattice then spreads over twice the SMs) and for Ns = 2, whose staged links fill shared memory.
 inline int fx_threads(size_t n5, int ns) { return ns == 2 || n5 < (size_t)kFxThreads * 304 ? 64 : kFxThreads; }
+// dynamic shared memory of a block: its staged links or the recurrences' columns, whichever is larger
+inline size_t fx_smem(int bs, int ns, bool links) {
+    const size_t cols = (size_t)(bs / ns) * 24 * (ns + 1) * sizeof(double);
+    const size_t lk = links ? (size_t)(bs / ns) * kFxSite * sizeof(int4) : 0;
+    return cols > lk ? cols : lk;
+}
 
 template <int F>
 cudaError_t hop_fx(const HopParams<double>& P, int nsys, cudaStream_t st) {
     const size_t n = (size_t)P.g.Vh * P.ns;
     const int bs = fx_threads(n, P.ns);
-    const size_t smem = (size_t)(bs / P.ns) * (kFxSite * sizeof(int4) + 8 * sizeof(int));
     note_launch();
-    hop_fx_kernel<F><<<dim3(blocks_for(n, bs), nsys), bs, smem, st>>>(P);
+    hop_fx_kernel<F><<<dim3(blocks_for(n, bs), nsys), bs, fx_smem(bs, P.ns, true), st>>>(P);
     return cudaGetLastError();
 }
 
