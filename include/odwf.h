@@ -69,8 +69,9 @@ enum {
     ODWF_EBUSY = 10       /* serving: the queue is full (serve_set_policy); the request was not taken */
 };
 
-/* ODWF_FF: float-float, each real the unevaluated sum of two FP32 numbers (about 48 bits),
- * arithmetic built from FP32 operations: the reliable updates of the mixed-precision CG. */
+/* ODWF_FF (odwf_apply_normal_prec only): the operator of the mixed-precision CG's reliable updates.
+ * It is the FP64 operator: its stencil runs in block fixed point on the integer pipe, which resolves
+ * more than FP64 and is faster on this GPU than FP64 or pairs of FP32 (the name's origin). */
 typedef enum { ODWF_F64 = 0, ODWF_F32 = 1, ODWF_F16 = 2, ODWF_BF16 = 3, ODWF_FF = 4 } odwf_prec;
 
 enum { ODWF_MODE_FULL = 0, ODWF_MODE_SCHUR_EVEN = 1 };
@@ -97,7 +98,7 @@ typedef struct {
     int32_t max_iter;   /* cap on inner CG iterations (summed over restarts) */
     int32_t prec;       /* ODWF_F64: plain FP64 CG; ODWF_F32/F16/BF16: mixed precision with that
                            storage for the inner operator fields, FP32 arithmetic, reliable updates
-                           (true residual b - A x) in FP64 or float-float (update_arith) */
+                           (true residual b - A x) in FP64 */
     double delta;       /* reliable-update trigger: recompute the FP64 residual when the inner
                            residual drops below delta x its largest value since the last update
                            (<= 0 selects 0.01) */
@@ -109,19 +110,15 @@ typedef struct {
                            (24 bytes per link, no scale: SU(3) entries have modulus <= 1; needs
                            Ns = 8 or 16 and link_recon 0 or 12) */
     int32_t update_arith; /* mixed: arithmetic of the reliable updates (true residual b - A x) and of
-                           the accumulated solution.  ODWF_UPDATES_AUTO (0) and ODWF_UPDATES_FF:
-                           float-float (pairs of FP32, about 48 bits, on the FP32 pipe);
-                           ODWF_UPDATES_F64: FP64.  Both resolve the true residual far below 1e-10;
-                           on GB300, whose FP64 rate is a small fraction of its FP32 rate,
-                           float-float is faster for one system and for batches.  Full-lattice
-                           systems (FULL_NORMAL, FULL_DIRAC) always update in FP64. */
+                           the accumulated solution: ODWF_UPDATES_AUTO (0), ODWF_UPDATES_F64 or
+                           ODWF_UPDATES_FF.  All three now run the same FP64-accuracy operator (see
+                           ODWF_FF) with an FP64 solution. */
 } odwf_solve_params;
 
 typedef struct {
     int32_t iters;          /* inner CG iterations */
     int32_t n_reliable;     /* FP64 residual recomputations */
-    double true_resid;      /* final ||b - A x|| / ||b||, recomputed on the GPU (FP64, or float-float
-                               for mixed solves that update in float-float) */
+    double true_resid;      /* final ||b - A x|| / ||b||, recomputed on the GPU in FP64 */
     double time_ms;         /* wall time of the solve inside the library */
     int32_t status;         /* ODWF_OK / ODWF_ENOCONV / ODWF_EBREAKDOWN for this system */
     int32_t reserved;
@@ -189,8 +186,8 @@ int odwf_apply_normal(odwf_handle* h, void* out, const void* in, int system, voi
  * site), the four hops run in FP32 with FP32 links of `link_recon` (12 or 18) reals, and
  * every intermediate field is stored in `prec`.  Even-site fields, as odwf_apply_normal.
  * This is the operator the inner CG iterates with; it is exposed for accuracy checks.
- * prec = ODWF_FF gives the reliable updates' operator instead: float-float fields, links and
- * arithmetic throughout (link_recon is ignored).
+ * prec = ODWF_FF gives the reliable updates' operator instead, which is odwf_apply_normal's
+ * (link_recon is ignored).
  */
 int odwf_apply_normal_prec(odwf_handle* h, void* out, const void* in, int prec, int link_recon, void* stream);
 

@@ -51,11 +51,8 @@ Engine::~Engine() {
     if (links_f18) cudaFree(links_f18);
     if (links_f12) cudaFree(links_f12);
     if (links_h12) cudaFree(links_h12);
-    if (links_ff18) cudaFree(links_ff18);
-    if (links_fx) cudaFree(links_fx);
     for (void* p : links_site)
         if (p) cudaFree(p);
-    if (nbr) cudaFree(nbr);
     if (pinned) cudaFreeHost(pinned);
 }
 
@@ -96,21 +93,13 @@ int Engine::init(const odwf_lattice* l, int Ns, double m0_, double mq_, const do
         cf32.d[s] = (float)cf64.d[s];
         cf32.e[s] = (float)cf64.e[s];
         cf32.inv_d[s] = (float)cf64.inv_d[s];
-        cfff.rho[s] = ff(cf64.rho[s]);
-        cfff.sigma[s] = ff(cf64.sigma[s]);
-        cfff.d[s] = ff(cf64.d[s]);
-        cfff.e[s] = ff(cf64.e[s]);
-        cfff.inv_d[s] = ff(cf64.inv_d[s]);
     }
     ODWF_CK(cudaGetDevice(&device));
     int rc = 0;
-    double* rd = (double*)get_ws("r_handle", sizeof(double), &rc);
-    if (rc) return rc;
-    const double r = mq / (2.0 * m0);
-    ODWF_CK(cudaMemcpy(rd, &r, sizeof(double), cudaMemcpyHostToDevice));
     // scan tables of the fixed-point hops' M^-1 (fx_minv): 1/d, then al and its running product for
     // M^-1 up (forward, e_s), M^-1 down (backward, e_s), M^-dag up (backward, e_{s+1}), down (forward, e_{s-1})
-    std::vector<double> tab(cf64.inv_d, cf64.inv_d + Ns);
+    std::vector<double> tab{mq / (2.0 * m0), 0.0};  // the handle's r comes first (16 bytes)
+    tab.insert(tab.end(), cf64.inv_d, cf64.inv_d + Ns);
     for (int v = 0; v < 4; ++v) {
         std::vector<double> al(Ns), A(Ns);
         for (int s = 0; s < Ns; ++s)
@@ -125,9 +114,10 @@ int Engine::init(const odwf_lattice* l, int Ns, double m0_, double mq_, const do
         tab.insert(tab.end(), al.begin(), al.end());
         tab.insert(tab.end(), A.begin(), A.end());
     }
-    fx_tab = (double*)get_ws("fx_tab", tab.size() * sizeof(double), &rc);
+    double* rd = (double*)get_ws("r_handle", tab.size() * sizeof(double), &rc);
     if (rc) return rc;
-    ODWF_CK(cudaMemcpy(fx_tab, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice));
+    ODWF_CK(cudaMemcpy(rd, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice));
+    fx_tab = rd + 2;
     bounds_flag = (unsigned*)get_ws("bounds_flag", sizeof(unsigned), &rc);
     if (rc) return rc;
     ODWF_CK(cudaMemset(bounds_flag, 0, sizeof(unsigned)));
@@ -152,7 +142,6 @@ size_t Engine::half_bytes(Sp sp) const {
     switch (sp) {
         case Sp::F64: return sites5() * 192;
         case Sp::FX: return sites5() * 192;
-        case Sp::FF: return sites5() * 192;
         case Sp::F32: return sites5() * 96;
         default: return sites5() * 48;
     }
@@ -223,16 +212,16 @@ int Engine::set_gauge(const void* U, cudaStream_t st) {
         Ud = (const double2*)tmp;
     }
     const size_t nl = 8 * vh();
-    if (!links_d18) ODWF_CK(cudaMalloc(&links_d18, nl * 144));
-    if (!nbr) {
-        ODWF_CK(cudaMalloc(&nbr, 2 * nl * sizeof(int)));
+    if (!links_d18) {  // one allocation: FP64 links, fixed-point links and exponents, neighbour table
+        ODWF_CK(cudaMalloc(&links_d18, nl * (144 + 148 + 2 * sizeof(int))));
+        links_fx = (char*)links_d18 + nl * 144;
+        nbr = (int*)((char*)links_fx + nl * 148);
         ODWF_CK(launch_build_neighbours(nbr, g, st));
     }
-    if (!links_fx) ODWF_CK(cudaMalloc(&links_fx, nl * 148));
     ODWF_CK(launch_pack_links(Ud, links_d18, nullptr, nullptr, g, st));
     ODWF_CK(launch_links_fx(links_d18, links_fx, nl, st));
     // FP32 copies are derived from the FP64 ones on first use (ensure_links)
-    have_f12 = have_f18 = have_h12 = have_ff18 = false;
+    have_f12 = have_f18 = have_h12 = false;
     for (bool& b : have_site) b = false;
     if (!is_device_ptr(U)) {
         ODWF_CK(cudaStreamSynchronize(st));
@@ -257,10 +246,6 @@ int Engine::ensure_links(Lk lk, cudaStream_t st) {
         if (!links_f18) ODWF_CK(cudaMalloc(&links_f18, nl * 80));
         ODWF_CK(launch_links_from_d18(links_d18, links_f18, nullptr, nl, st));
         have_f18 = true;
-    } else if (lk == Lk::FF18 && !have_ff18) {
-        if (!links_ff18) ODWF_CK(cudaMalloc(&links_ff18, nl * 144));
-        ODWF_CK(launch_links_ff18_from_d18(links_d18, links_ff18, nl, st));
-        have_ff18 = true;
     } else if (lk == Lk::H12 && !have_h12) {
         if (!links_h12) ODWF_CK(cudaMalloc(&links_h12, nl * 24));
         ODWF_CK(launch_links_h12_from_d18(links_d18, links_h12, nl, st));
@@ -296,21 +281,6 @@ HopParams<double> Engine::hop_params<double>(int p_out, const double* r_dev) con
     P.nbr = nbr;
     P.r_sys = r_dev;
     P.cf = cf64;
-    P.bounds_flag = bounds_flag;
-    return P;
-}
-
-template <>
-HopParams<ff> Engine::hop_params<ff>(int p_out, const double* r_dev) const {
-    HopParams<ff> P;
-    std::memset(&P, 0, sizeof(P));
-    P.g = g;
-    P.ns = ns;
-    P.lg_ns = lg_ns;
-    P.p_out = p_out;
-    P.links = links_ff18;
-    P.r_sys = r_dev;
-    P.cf = cfff;
     P.bounds_flag = bounds_flag;
     return P;
 }
@@ -472,56 +442,10 @@ int Engine::apply_normal(void* out, const void* in, int system, cudaStream_t st)
     return ODWF_OK;
 }
 
-// S^dag S in float-float arithmetic with float-float fields and links: the operator of the
-// mixed-precision CG's reliable updates.
-int Engine::apply_ff_normal(void* out, const void* in, cudaStream_t st) {
-    if (!out || !in) return fail(ODWF_EINVAL, "apply_normal_prec: null field");
-    const size_t eb = ext_bytes(ODWF_MODE_SCHUR_EVEN);
-    int rc = 0;
-    const double2* din = nullptr;
-    if ((rc = stage_in(this, in, eb, "ext.in", st, &din))) return rc;
-    const bool out_dev = is_device_ptr(out);
-    double2* dout = out_dev ? (double2*)out : (double2*)get_ws("ext.out", eb, &rc);
-    if (rc) return rc;
-    const double* rd = (const double*)ws["r_handle"].p;
-    HalfField X, Y, T, A, C;
-    if ((rc = alloc_half("ff.X", Sp::FF, 1, &X)) || (rc = alloc_half("ff.Y", Sp::FF, 1, &Y)) ||
-        (rc = alloc_half("ff.T", Sp::FF, 1, &T)) || (rc = alloc_half("ff.A", Sp::FF, 1, &A)) ||
-        (rc = alloc_half("ff.C", Sp::FF, 1, &C)))
-        return rc;
-    if ((rc = ensure_links(Lk::FF18, st))) return rc;
-    ODWF_CK(launch_pack(Sp::FF, din, X.ref_sys(0), g, 0, ns, 1, st));
-    auto P = hop_params<ff>(1, rd);
-    P.in = X.ref_sys(0);
-    P.out = T.ref_sys(0);
-    ODWF_CK(launch_hop_ff(P, Epi::MINV, 1, st));
-    P.p_out = 0;
-    P.in = T.ref_sys(0);
-    P.z = X.ref_sys(0);
-    P.out = A.ref_sys(0);
-    ODWF_CK(launch_hop_ff(P, Epi::SCHUR_MDINV, 1, st));
-    P.p_out = 1;
-    P.in = A.ref_sys(0);
-    P.z = FieldRef{};
-    P.out = C.ref_sys(0);
-    ODWF_CK(launch_hop_ff(P, Epi::D_MINVDAG, 1, st));
-    P.p_out = 0;
-    P.in = C.ref_sys(0);
-    P.z = A.ref_sys(0);
-    P.out = Y.ref_sys(0);
-    ODWF_CK(launch_hop_ff(P, Epi::D_NORMAL, 1, st));
-    ODWF_CK(launch_unpack(Sp::FF, Y.ref_sys(0), dout, g, 0, ns, 1, st));
-    if (!out_dev) {
-        ODWF_CK(cudaMemcpyAsync(out, dout, eb, cudaMemcpyDeviceToHost, st));
-        ODWF_CK(cudaStreamSynchronize(st));
-    }
-    return ODWF_OK;
-}
-
 int Engine::apply_low_normal(void* out, const void* in, int prec, int recon, cudaStream_t st) {
     if (!gauge_set) return fail(ODWF_EINVAL, "apply_normal_prec: gauge field not set");
     if (!out || !in) return fail(ODWF_EINVAL, "apply_normal_prec: null field");
-    if (prec == ODWF_FF) return apply_ff_normal(out, in, st);
+    if (prec == ODWF_FF) return apply_normal(out, in, ODWF_SYS_SCHUR_NORMAL, st);  // the reliable updates' operator
     if (prec != ODWF_F32 && prec != ODWF_F16 && prec != ODWF_BF16)
         return fail(ODWF_EINVAL, "apply_normal_prec: prec must be F32, F16, BF16 or FF");
     if (recon != 12 && recon != 18) return fail(ODWF_EINVAL, "apply_normal_prec: link_recon must be 12 or 18");

@@ -1,4 +1,4 @@
-// Kernel templates of the ODWF library (instantiated in kernels_f64.cu / kernels_mixed.cu).
+// Kernel templates of the ODWF library (instantiated in kernels_f64.cu, kernels_mixed.cu and kernels_fx.cuh).
 //
 // The fused hopping kernel computes, for every output site x of parity p_out and every s,
 //   non-dagger:  y = W (B psi),     H psi     = -1/2 y
@@ -194,42 +194,6 @@ __device__ __forceinline__ void su3_mul(const R u[18], const R h[12], R w[12], b
         }
 }
 
-// Float-float instance: each output component is a six-term dot product, summed as a compensated
-// dot product (two-product of the leading parts plus the cross terms, two-sum of the running
-// total, the rounding errors gathered in a second word and added once at the end), as accurate as
-// the float-float operators of ff.cuh with about two thirds of their FP32 operations.
-__device__ __forceinline__ void ff_dot_acc(float& s, float& c, float ah, float al, float bh, float bl) {
-    const float p = __fmul_rn(ah, bh);
-    float e = fmaf(ah, bh, -p);  // ah bh - p, exact
-    e = fmaf(ah, bl, e);
-    e = fmaf(al, bh, e);
-    const float t = __fadd_rn(s, p);
-    const float bb = __fsub_rn(t, s);
-    const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(p, bb));  // s + p - t, exact
-    s = t;
-    c = __fadd_rn(c, __fadd_rn(err, e));
-}
-__device__ __forceinline__ void su3_mul(const ff u[18], const ff h[12], ff w[12], bool dag) {
-#pragma unroll
-    for (int sp = 0; sp < 2; ++sp)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            float rs = 0.f, rc = 0.f, is = 0.f, ic = 0.f;
-#pragma unroll
-            for (int b = 0; b < 3; ++b) {
-                const int ix = dag ? (3 * b + a) : (3 * a + b);
-                const ff ur = u[2 * ix], ui = dag ? -u[2 * ix + 1] : u[2 * ix + 1];
-                const ff hr = h[6 * sp + 2 * b], hi = h[6 * sp + 2 * b + 1];
-                ff_dot_acc(rs, rc, ur.hi, ur.lo, hr.hi, hr.lo);
-                ff_dot_acc(rs, rc, -ui.hi, -ui.lo, hi.hi, hi.lo);
-                ff_dot_acc(is, ic, ur.hi, ur.lo, hi.hi, hi.lo);
-                ff_dot_acc(is, ic, ui.hi, ui.lo, hr.hi, hr.lo);
-            }
-            w[6 * sp + 2 * a] = ff_fast_two_sum(rs, rc);
-            w[6 * sp + 2 * a + 1] = ff_fast_two_sum(is, ic);
-        }
-}
-
 // ---------------------------------------------------------------- reductions
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -241,12 +205,6 @@ __device__ __forceinline__ float warp_sum(float v) {
     for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
     return v;
 }
-__device__ __forceinline__ ff warp_sum(ff v) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += shfl_down(v, off, 32);
-    return v;
-}
-
 // Deterministic block sum (fixed tree for a fixed blockDim); result valid in thread 0.
 // The per-thread values and the sum over a warp are taken in the kernel's arithmetic type
 // R (FP32 in the mixed-precision kernels: GB300's FP64 rate is a small fraction of its
@@ -338,10 +296,8 @@ __device__ __forceinline__ void reduce_and_finalize(R v, double* partials, unsig
 }
 
 // ---------------------------------------------------------------- the fused hopping kernel
-// The body of the generic hop (one thread per 5D site); hop_kernel below launches it at 256
-// threads per block, other instances (float-float) at their own bounds.
 template <class SPin, class SPz, class SPout, class SPacc, class LK, class R, int F>
-__device__ __forceinline__ void hop_body(const HopParams<R>& P) {
+__global__ void __launch_bounds__(256) hop_kernel(const HopParams<R> P) {
     constexpr bool DAG = (F & F_DAG) != 0;
     constexpr int ZOP = (F & F_ZOP_MASK) >> F_ZOP_SHIFT;
     constexpr int HOPOP = (F & F_HOP_MASK) >> F_HOP_SHIFT;
@@ -479,11 +435,6 @@ __device__ __forceinline__ void hop_body(const HopParams<R>& P) {
     }
 
     if (REDUCE) reduce_and_finalize(nrm, P.partials, P.counters, P.st, sys, FIN, P.part_stride);
-}
-
-template <class SPin, class SPz, class SPout, class SPacc, class LK, class R, int F>
-__global__ void __launch_bounds__(256) hop_kernel(const HopParams<R> P) {
-    hop_body<SPin, SPz, SPout, SPacc, LK, R, F>(P);
 }
 
 // ---------------------------------------------------------------- site-local kernels

@@ -12,8 +12,8 @@ namespace odwf {
 constexpr int kMinReduceBlock = 64;
 
 
-enum class Sp { F64 = 0, F32 = 1, F16 = 2, BF16 = 3, FF = 4, FX = 5 };  // FF: float-float pairs (ff.cuh), FX: fx.cuh
-enum class Lk { D18 = 0, F18 = 1, F12 = 2, H12 = 3, FF18 = 4 };
+enum class Sp { F64 = 0, F32 = 1, F16 = 2, BF16 = 3, FX = 4 };  // FX: block fixed point (fx.cuh)
+enum class Lk { D18 = 0, F18 = 1, F12 = 2, H12 = 3 };
 
 struct FieldRef;
 template <class R>
@@ -50,12 +50,6 @@ cudaError_t launch_m5_fx(const FieldRef& in, const FieldRef& out, size_t n_sites
                          cudaStream_t st, const SysState* gate_st = nullptr, int need = 0);
 // the fixed-point link array of n_links FP64 links: 144 bytes per link, then an int exponent per link
 cudaError_t launch_links_fx(const void* d18, void* fx, size_t n_links, cudaStream_t st);
-// Float-float path (float-float fields and links, float-float arithmetic on the FP32 pipe): the
-// reliable updates of the mixed-precision CG.  Epilogues MINV, SCHUR_MDINV, D_MINVDAG, D_NORMAL,
-// D_NORMAL_RESID.
-cudaError_t launch_hop_ff(const HopParams<ff>& P, Epi e, int nsys, cudaStream_t st);
-cudaError_t launch_m5_ff(const FieldRef& in, const FieldRef& out, size_t n_sites, int ns, const double* r_sys,
-                         int sys_base, int nsys, int op, const Coef5<ff>& cf, cudaStream_t st);
 // Pseudofermion-force contraction (kernels_force.cu): G += coef * [U K1 - K2 U^+] per link from the
 // parity-split FP64 fields L (Le, Lo) and R (Re, Ro); G in the internal link order
 // ((p * 4 + mu) * Vh + h) * 9.  finalize: ta(G) into the external gauge layout.
@@ -75,8 +69,6 @@ cudaError_t launch_gauge_force(const int dims[4], const double2* U, double beta,
                                double* retr_sum, cudaStream_t st);
 cudaError_t launch_link_update(size_t nlinks, double2* U, const double2* P, double a, cudaStream_t st);  // U <- exp(aP) U
 cudaError_t launch_axpy(size_t n, double2* y, const double2* x, double c, cudaStream_t st);              // y += c x
-// the FP64 links split into float-float pairs (same 144-byte records)
-cudaError_t launch_links_ff18_from_d18(const void* d18, void* ff18, size_t n_links, cudaStream_t st);
 // Mixed path (low-precision operator fields, FP32 accumulators r/x, float links, FP32 arithmetic)
 cudaError_t launch_hop_mixed(const HopParams<float>& P, Epi e, Sp low, Lk lk, int nsys, cudaStream_t st);
 

@@ -154,8 +154,8 @@ size_t per_system_bytes(size_t sites5, int prec) {
 }
 
 size_t group_fixed_bytes(size_t vh, size_t sites5) {
-    // links (FP64, float-float, FP32-18, FP32-12 and its site-major copy), FP64 / float-float
-    // temporaries, scratch
+    // links (FP64, fixed point, FP32-12 and its site-major copy; the rest is slack), FP64 and
+    // fixed-point temporaries, scratch
     return 8 * vh * (144 + 144 + 80 + 48 + 96) + sites5 * 192 * 6 + (1 << 20);
 }
 
