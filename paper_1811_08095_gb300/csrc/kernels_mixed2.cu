@@ -77,12 +77,10 @@ __global__ void __launch_bounds__(kBS2, 3) hop2_kernel(const HopParams<float> P)
 
     const void* in = P.in.d(sys);
     const float* in_n = P.in.n(sys);
-    float2 AUr[3], AUi[3], ADr[3], ADi[3], ADSr[3], ADSi[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) AUr[c] = AUi[c] = ADr[c] = ADi[c] = ADSr[c] = ADSi[c] = make_float2(0.f, 0.f);
+    HopAcc A;
+    A.clear();
     const float2* L2p = reinterpret_cast<const float2*>(my_links);
     // forward hops use (1 - gamma) for D and (1 + gamma) for D^dag; backward the opposite
-    constexpr float SF = DAG ? 1.f : -1.f;
     // neighbour j + 1 is fetched before neighbour j is processed
     RawSite<SP> rs[2];
     fetch_site<SP>(in, in_n, (unsigned)nb[0], s, NS, rs[0]);
@@ -92,23 +90,16 @@ __global__ void __launch_bounds__(kBS2, 3) hop2_kernel(const HopParams<float> P)
         if (j_ < 7) fetch_site<SP>(in, in_n, (unsigned)nb[j_ + 1 < 8 ? j_ + 1 : 7], s, NS, rs[(j_ + 1) & 1]);        \
         const float sgn_ = (flip & (1u << j_)) ? -1.f : 1.f;                                                     \
         const LinkStaged2 ls_{L2p + j_ * 9};                                                                      \
-        hop_dir_packed<SP, MU_, DIR_ == 1>(rs[j_ & 1], sgn_, DIR_ == 0 ? SF : -SF, ls_, AUr, AUi, ADr, ADi, ADSr,  \
-                                           ADSi);                                                                 \
+        hop_dir_packed<SP, MU_, DIR_ == 1, (DIR_ == 0) == DAG>(rs[j_ & 1], sgn_, ls_, A);                        \
     }
     ODWF_HOP_DIR(0, 0); ODWF_HOP_DIR(0, 1);
     ODWF_HOP_DIR(1, 0); ODWF_HOP_DIR(1, 1);
+    A.swap_lower();
     ODWF_HOP_DIR(2, 0); ODWF_HOP_DIR(2, 1);
     ODWF_HOP_DIR(3, 0); ODWF_HOP_DIR(3, 1);
 #undef ODWF_HOP_DIR
-    // y = W psi (or W^dag psi) in pairs; the lower half gathers AD and the swapped ADS
-    Half6 up, dn;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        up.R[c] = AUr[c];
-        up.I[c] = AUi[c];
-        dn.R[c] = __fadd2_rn(ADr[c], make_float2(ADSr[c].y, ADSr[c].x));
-        dn.I[c] = __fadd2_rn(ADi[c], make_float2(ADSi[c].y, ADSi[c].x));
-    }
+    Half6 up, dn;  // W psi (or W^dag psi) in pairs
+    A.halves(up, dn);
 
     const Coef5<float>& cf = P.cf;
     float nrm = 0.f;  // per-thread partial sums in FP32, FP64 across warps and blocks (block_sum)

@@ -55,24 +55,15 @@ __device__ __forceinline__ RawSite<SP> raw_of(const RawPair& r, int v) {
     return o;
 }
 
-struct Acc {
-    float2 AUr[3], AUi[3], ADr[3], ADi[3], ADSr[3], ADSi[3];
-};
-
 // One hop direction for both values of the lane: the link element (a, b) is read from shared
 // memory once and multiplied into both spinors.
-template <class SP, int MU, bool DAGU>
-__device__ __forceinline__ void hop_dir_pair(const RawPair& raw, float sgn, float sg, const float2* L, Acc& A,
-                                             Acc& B) {
-    constexpr bool SW = (MU == 0 || MU == 1);
+template <class SP, int MU, bool DAGU, bool PLUS>
+__device__ __forceinline__ void hop_dir_pair(const RawPair& raw, float sgn, const float2* L, HopAcc& A,
+                                             HopAcc& B) {
+    constexpr float sg = PLUS ? 1.f : -1.f;
     float2 HrA[3], HiA[3], NhA[3], HrB[3], HiB[3], NhB[3];
-    {
-        float2 Ur[3], Ui[3], Dr[3], Di[3];
-        unpack_site<SP, SW>(raw_of<SP>(raw, 0), Ur, Ui, Dr, Di);
-        project_pairs<MU>(Ur, Ui, Dr, Di, sg, HrA, HiA);
-        unpack_site<SP, SW>(raw_of<SP>(raw, 1), Ur, Ui, Dr, Di);
-        project_pairs<MU>(Ur, Ui, Dr, Di, sg, HrB, HiB);
-    }
+    project_site<SP, MU, PLUS>(raw_of<SP>(raw, 0), HrA, HiA);
+    project_site<SP, MU, PLUS>(raw_of<SP>(raw, 1), HrB, HiB);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         NhA[c] = DAGU ? make_float2(-HrA[c].x, -HrA[c].y) : make_float2(-HiA[c].x, -HiA[c].y);
@@ -89,8 +80,8 @@ __device__ __forceinline__ void hop_dir_pair(const RawPair& raw, float sgn, floa
             su3_row_acc<DAGU>(ur, ui, HrA[b], HiA[b], NhA[b], WrA, WiA);
             su3_row_acc<DAGU>(ur, ui, HrB[b], HiB[b], NhB[b], WrB, WiB);
         }
-        accumulate_row<MU>(mA, sg * mA, WrA, WiA, A.AUr[a], A.AUi[a], A.ADr[a], A.ADi[a], A.ADSr[a], A.ADSi[a]);
-        accumulate_row<MU>(mB, sg * mB, WrB, WiB, B.AUr[a], B.AUi[a], B.ADr[a], B.ADi[a], B.ADSr[a], B.ADSi[a]);
+        accumulate_row<MU>(mA, sg * mA, WrA, WiA, A.AUr[a], A.AUi[a], A.ADr[a], A.ADi[a]);
+        accumulate_row<MU>(mB, sg * mB, WrB, WiB, B.AUr[a], B.AUi[a], B.ADr[a], B.ADi[a]);
     }
 }
 
@@ -208,16 +199,6 @@ __device__ __forceinline__ void minv2(Half6& upA, Half6& dnA, Half6& upB, Half6&
     }
 }
 
-__device__ __forceinline__ void to_pairs(const Acc& a, Half6& up, Half6& dn) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        up.R[c] = a.AUr[c];
-        up.I[c] = a.AUi[c];
-        dn.R[c] = __fadd2_rn(a.ADr[c], make_float2(a.ADSr[c].y, a.ADSr[c].x));
-        dn.I[c] = __fadd2_rn(a.ADi[c], make_float2(a.ADSi[c].y, a.ADSi[c].x));
-    }
-}
-
 // Blocks per SM: K2, which also streams p in and keeps two scans' state, runs faster at four
 // (128 registers, a few spilled: 764 -> 708 us on 32^4 x 16); K1 and K3 at three (168 registers).
 template <int KIND>
@@ -272,30 +253,28 @@ __global__ void __launch_bounds__(kBS3, hop3_min_blocks<KIND>()) hop3_kernel(con
 
     const void* in = P.in.d(sys);
     const float* in_n = P.in.n(sys);
-    Acc A, B;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        A.AUr[c] = A.AUi[c] = A.ADr[c] = A.ADi[c] = A.ADSr[c] = A.ADSi[c] = make_float2(0.f, 0.f);
-        B.AUr[c] = B.AUi[c] = B.ADr[c] = B.ADi[c] = B.ADSr[c] = B.ADSi[c] = make_float2(0.f, 0.f);
-    }
+    HopAcc A, B;
+    A.clear();
+    B.clear();
     const float2* L2p = reinterpret_cast<const float2*>(my_links);
-    constexpr float SF = DAG ? 1.f : -1.f;
     RawPair rp;
 #define ODWF_HOP3_DIR(MU_, DIR_)                                                                   \
     {                                                                                              \
         constexpr int j_ = 2 * MU_ + DIR_;                                                         \
         fetch_pair<NS>(in, in_n, (unsigned)nb[j_], l, rp);                                         \
         const float sgn_ = (flip & (1u << j_)) ? -1.f : 1.f;                                      \
-        hop_dir_pair<SP, MU_, DIR_ == 1>(rp, sgn_, DIR_ == 0 ? SF : -SF, L2p + j_ * 9, A, B);      \
+        hop_dir_pair<SP, MU_, DIR_ == 1, (DIR_ == 0) == DAG>(rp, sgn_, L2p + j_ * 9, A, B);        \
     }
     ODWF_HOP3_DIR(0, 0); ODWF_HOP3_DIR(0, 1);
     ODWF_HOP3_DIR(1, 0); ODWF_HOP3_DIR(1, 1);
+    A.swap_lower();
+    B.swap_lower();
     ODWF_HOP3_DIR(2, 0); ODWF_HOP3_DIR(2, 1);
     ODWF_HOP3_DIR(3, 0); ODWF_HOP3_DIR(3, 1);
 #undef ODWF_HOP3_DIR
     Half6 upA, dnA, upB, dnB;
-    to_pairs(A, upA, dnA);
-    to_pairs(B, upB, dnB);
+    A.halves(upA, dnA);
+    B.halves(upB, dnB);
 
     const Coef5<float>& cf = P.cf;
     float v[24];

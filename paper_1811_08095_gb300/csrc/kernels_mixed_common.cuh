@@ -55,21 +55,11 @@ __device__ __forceinline__ void fetch_site(const void* base, const float* norm, 
 template <class SP, bool SWAP_DN>
 __device__ __forceinline__ void unpack_site(const RawSite<SP>& r, float2 Ur[3], float2 Ui[3], float2 Dr[3],
                                             float2 Di[3]) {
+    static_assert(std::is_same<SP, SpF32>::value, "half storage goes through project_half");
     float2 f[12];  // word w = (spin w/3, colour w%3): (re, im)
-    if (std::is_same<SP, SpF32>::value) {
-        const float* v = reinterpret_cast<const float*>(&r);
+    const float* v = reinterpret_cast<const float*>(&r);
 #pragma unroll
-        for (int w = 0; w < 12; ++w) f[w] = make_float2(v[2 * w], v[2 * w + 1]);
-    } else {
-        using H2 = typename std::conditional<std::is_same<SP, SpF16>::value, __half2, __nv_bfloat162>::type;
-        const uint32_t* wd = reinterpret_cast<const uint32_t*>(&r);
-#pragma unroll
-        for (int w = 0; w < 12; ++w) {
-            H2 hv;
-            *reinterpret_cast<uint32_t*>(&hv) = wd[w];
-            f[w] = Half2Cvt<H2>::to_f2(hv);
-        }
-    }
+    for (int w = 0; w < 12; ++w) f[w] = make_float2(v[2 * w], v[2 * w + 1]);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         Ur[c] = make_float2(f[c].x, f[3 + c].x);
@@ -84,11 +74,52 @@ __device__ __forceinline__ void unpack_site(const RawSite<SP>& r, float2 Ur[3], 
     }
 }
 
+// Half-precision values into FP32 arithmetic without a conversion: sm_100's mixed multiply-add
+// d = a b + c with a, b in FP16 / BF16 and c, d in FP32 runs at the full FP32 rate, a conversion at half.
+// HI selects the upper half of the word.
+template <class SP, bool HI>
+__device__ __forceinline__ float half_fma(uint32_t w, bool minus, float c) {
+    float d;
+    if (std::is_same<SP, SpF16>::value) {
+        const uint16_t one = minus ? 0xbc00 : 0x3c00;
+        if (HI) asm("{.reg .b16 l, h; mov.b32 {l, h}, %1; fma.rn.f32.f16 %0, h, %2, %3;}" : "=f"(d) : "r"(w), "h"(one), "f"(c));
+        else asm("{.reg .b16 l, h; mov.b32 {l, h}, %1; fma.rn.f32.f16 %0, l, %2, %3;}" : "=f"(d) : "r"(w), "h"(one), "f"(c));
+    } else {
+        const uint16_t one = minus ? 0xbf80 : 0x3f80;
+        if (HI) asm("{.reg .b16 l, h; mov.b32 {l, h}, %1; fma.rn.f32.bf16 %0, h, %2, %3;}" : "=f"(d) : "r"(w), "h"(one), "f"(c));
+        else asm("{.reg .b16 l, h; mov.b32 {l, h}, %1; fma.rn.f32.bf16 %0, l, %2, %3;}" : "=f"(d) : "r"(w), "h"(one), "f"(c));
+    }
+    return d;
+}
+
+// unpack_site and project_pairs of one 5D site in half storage: every real of H = v^up + sg G v^dn is
+// one real of v^up plus or minus one of v^dn, two mixed multiply-adds (the second rounds once, as the
+// FP32 form does).
+template <class SP, int MU, bool PLUS>
+__device__ __forceinline__ void project_half(const RawSite<SP>& raw, float2 Hr[3], float2 Hi[3]) {
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(&raw);  // word 3 spin + colour: (re, im)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const uint32_t u0 = w[c], u1 = w[3 + c], d0 = w[6 + c], d1 = w[9 + c];
+        // G d of the two upper spins: mu 0 (-i d1, -i d0), 1 (-d1, d0), 2 (-i d0, i d1), 3 (d0, d1)
+        const uint32_t g0 = (MU == 0 || MU == 1) ? d1 : d0, g1 = (MU == 0 || MU == 1) ? d0 : d1;
+        const float ar = half_fma<SP, false>(u0, false, 0.f), ai = half_fma<SP, true>(u0, false, 0.f);
+        const float br = half_fma<SP, false>(u1, false, 0.f), bi = half_fma<SP, true>(u1, false, 0.f);
+        if (MU == 0 || MU == 2) {  // -+ i d: re +- im(d), im -+ re(d)
+            constexpr bool s1 = MU == 0;  // spin 1 has the sign of spin 0 for mu 0, the other for mu 2
+            Hr[c] = make_float2(half_fma<SP, true>(g0, !PLUS, ar), half_fma<SP, true>(g1, s1 ? !PLUS : PLUS, br));
+            Hi[c] = make_float2(half_fma<SP, false>(g0, PLUS, ai), half_fma<SP, false>(g1, s1 ? PLUS : !PLUS, bi));
+        } else {
+            constexpr bool m0 = MU == 1 ? PLUS : !PLUS;  // spin 0: -d1 (mu 1), d0 (mu 3)
+            Hr[c] = make_float2(half_fma<SP, false>(g0, m0, ar), half_fma<SP, false>(g1, !PLUS, br));
+            Hi[c] = make_float2(half_fma<SP, true>(g0, m0, ai), half_fma<SP, true>(g1, !PLUS, bi));
+        }
+    }
+}
+
 // One hop direction in spin pairs.  H = v^up + sg G v^dn (G of gamma_mu in the chiral basis,
 // gamma_mu = [[0, G], [G^dag, 0]]); W = U H (or U^dag H); then
-//   AU += sc W,  lower spins += sg sc G^dag W,
-// accumulated in AD (order (2, 3)) for mu = 2, 3 and in ADS (order (3, 2)) for mu = 0, 1, so
-// that no pair ever needs its halves exchanged.  The link source returns element (a, b) of U
+//   AU += sc W,  lower spins += sg sc G^dag W (see HopAcc for their order).  The link source returns element (a, b) of U
 // as the broadcast pairs (ur, ur), (ui, ui).
 // Link source for hop_dir_packed: nine float2 (ur, ui) in shared memory, element (a, b) at
 // index 3a + b, returned as the broadcast pairs (ur, ur), (ui, ui) that the spin-pair FMAs need.
@@ -123,6 +154,17 @@ __device__ __forceinline__ void project_pairs(const float2 Ur[3], const float2 U
     }
 }
 
+template <class SP, int MU, bool PLUS>
+__device__ __forceinline__ void project_site(const RawSite<SP>& raw, float2 Hr[3], float2 Hi[3]) {
+    if constexpr (std::is_same<SP, SpF32>::value) {
+        float2 Ur[3], Ui[3], Dr[3], Di[3];
+        unpack_site<SP, (MU == 0 || MU == 1)>(raw, Ur, Ui, Dr, Di);
+        project_pairs<MU>(Ur, Ui, Dr, Di, PLUS ? 1.f : -1.f, Hr, Hi);
+    } else {
+        project_half<SP, MU, PLUS>(raw, Hr, Hi);
+    }
+}
+
 // Row a of W = U H (or U^dag H): W_a = sum_b U_ab H_b, with the link element as broadcast pairs;
 // Nh = -Hi (U) or -Hr (U^dag) supplies the sign of the imaginary cross term.
 template <bool DAGU>
@@ -137,18 +179,19 @@ __device__ __forceinline__ void su3_row_acc(float2 ur, float2 ui, float2 Hr, flo
     }
 }
 
-// Accumulate row a of W, scaled by m (upper spins) and md = sg m (lower spins, sg G^dag W).
+// Accumulate row a of W, scaled by m (upper spins) and md = sg m (lower spins, sg G^dag W).  The
+// lower pair is held in the order (3, 2) while mu = 0, 1 accumulate and in (2, 3) for mu = 2, 3.
 template <int MU>
 __device__ __forceinline__ void accumulate_row(float m, float md, float2 Wr, float2 Wi, float2& AUr, float2& AUi,
-                                               float2& ADr, float2& ADi, float2& ADSr, float2& ADSi) {
+                                               float2& ADr, float2& ADi) {
     AUr = fma2(make_float2(m, m), Wr, AUr);
     AUi = fma2(make_float2(m, m), Wi, AUi);
     if (MU == 0) {          // G^dag = i s1: lower (3, 2) order = i W
-        ADSr = fma2(make_float2(-md, -md), Wi, ADSr);
-        ADSi = fma2(make_float2(md, md), Wr, ADSi);
+        ADr = fma2(make_float2(-md, -md), Wi, ADr);
+        ADi = fma2(make_float2(md, md), Wr, ADi);
     } else if (MU == 1) {   // G^dag = [[0, 1], [-1, 0]]: lower (3, 2) order = W (-1, 1)
-        ADSr = fma2(make_float2(-md, md), Wr, ADSr);
-        ADSi = fma2(make_float2(-md, md), Wi, ADSi);
+        ADr = fma2(make_float2(-md, md), Wr, ADr);
+        ADi = fma2(make_float2(-md, md), Wi, ADi);
     } else if (MU == 2) {   // G^dag = i s3: lower = (i w0, -i w1)
         ADr = fma2(make_float2(-md, md), Wi, ADr);
         ADi = fma2(make_float2(md, -md), Wr, ADi);
@@ -158,16 +201,48 @@ __device__ __forceinline__ void accumulate_row(float m, float md, float2 Wr, flo
     }
 }
 
-template <class SP, int MU, bool DAGU, class LF>
-__device__ __forceinline__ void hop_dir_packed(const RawSite<SP>& raw, float sc_sign, float sg, const LF& lnk,
-                                               float2 AUr[3], float2 AUi[3], float2 ADr[3], float2 ADi[3],
-                                               float2 ADSr[3], float2 ADSi[3]) {
-    constexpr bool SW = (MU == 0 || MU == 1);
-    float2 Ur[3], Ui[3], Dr[3], Di[3];
-    unpack_site<SP, SW>(raw, Ur, Ui, Dr, Di);
+// One chirality half of a 5D site in the hop's own register layout: for colour c,
+// R[c] = (spin_a.re, spin_b.re), I[c] = (spin_a.im, spin_b.im); up = spins (0, 1), down = (2, 3).
+// The fifth-dimension operators act identically on all twelve reals of a chirality, so they run
+// on these pairs directly (packed FMAs, no repacking into memory order).
+struct Half6 {
+    float2 R[3], I[3];
+    __device__ __forceinline__ float2& p(int k) { return k < 3 ? R[k] : I[k - 3]; }
+};
+
+// W psi of one 5D site in spin pairs: upper spins (0, 1), lower spins in the order of the current mu
+struct HopAcc {
+    float2 AUr[3], AUi[3], ADr[3], ADi[3];
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) AUr[c] = AUi[c] = ADr[c] = ADi[c] = make_float2(0.f, 0.f);
+    }
+    __device__ __forceinline__ void halves(Half6& up, Half6& dn) const {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            up.R[c] = AUr[c];
+            up.I[c] = AUi[c];
+            dn.R[c] = ADr[c];
+            dn.I[c] = ADi[c];
+        }
+    }
+    // lower pair from (3, 2) to (2, 3), between mu = 1 and mu = 2: one set of accumulators instead of
+    // one per order (24 registers less with two sites per lane)
+    __device__ __forceinline__ void swap_lower() {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            ADr[c] = make_float2(ADr[c].y, ADr[c].x);
+            ADi[c] = make_float2(ADi[c].y, ADi[c].x);
+        }
+    }
+};
+
+template <class SP, int MU, bool DAGU, bool PLUS, class LF>
+__device__ __forceinline__ void hop_dir_packed(const RawSite<SP>& raw, float sc_sign, const LF& lnk, HopAcc& A) {
+    constexpr float sg = PLUS ? 1.f : -1.f;
     const float sc = raw.sc * sc_sign;
     float2 Hr[3], Hi[3], Nh[3];
-    project_pairs<MU>(Ur, Ui, Dr, Di, sg, Hr, Hi);
+    project_site<SP, MU, PLUS>(raw, Hr, Hi);
 #pragma unroll
     for (int c = 0; c < 3; ++c) Nh[c] = DAGU ? make_float2(-Hr[c].x, -Hr[c].y) : make_float2(-Hi[c].x, -Hi[c].y);
     // all three rows of W first, then the accumulation (this order keeps hop2's registers lowest)
@@ -185,19 +260,10 @@ __device__ __forceinline__ void hop_dir_packed(const RawSite<SP>& raw, float sc_
     }
     const float m = sc, md = sg * sc;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) accumulate_row<MU>(m, md, Wr[a], Wi[a], AUr[a], AUi[a], ADr[a], ADi[a], ADSr[a], ADSi[a]);
+    for (int a = 0; a < 3; ++a) accumulate_row<MU>(m, md, Wr[a], Wi[a], A.AUr[a], A.AUi[a], A.ADr[a], A.ADi[a]);
 }
 
-// ---------------------------------------------------------------- fifth-dimension epilogue on spin pairs
-// One chirality half of a 5D site in the hop's own register layout: for colour c,
-// R[c] = (spin_a.re, spin_b.re), I[c] = (spin_a.im, spin_b.im); up = spins (0, 1), down = (2, 3).
-// The fifth-dimension operators act identically on all twelve reals of a chirality, so they run
-// on these pairs directly (packed FMAs, no repacking into memory order).
-struct Half6 {
-    float2 R[3], I[3];
-    __device__ __forceinline__ float2& p(int k) { return k < 3 ? R[k] : I[k - 3]; }
-};
-
+// ---------------------------------------------------------------- fifth-dimension epilogue
 __device__ __forceinline__ float2 shfl2_idx(float2 v, int src, int w) {
     return make_float2(__shfl_sync(0xffffffffu, v.x, src, w), __shfl_sync(0xffffffffu, v.y, src, w));
 }
