@@ -88,11 +88,12 @@ int BatchCG::init(Engine* e, int capacity, const odwf_solve_params& prm, cudaStr
     // one partial per block of a reducing launch and system: sized for the smallest reducing
     // block (64 threads, one 5D site each), so every kernel's grid fits
     nblk = blocks_for(E->sites5(), kMinReduceBlock);
-    partials = (double*)E->get_ws("cg.partials", sizeof(double) * (size_t)nblk * cap, &rc);
+    partials = (double*)E->get_ws("cg.partials", sizeof(double) * (size_t)(nblk + reduce_groups(nblk)) * cap, &rc);
     if (rc) return rc;
-    counters = (unsigned*)E->get_ws("cg.counters", sizeof(unsigned) * cap, &rc);
+    const size_t cbytes = sizeof(unsigned) * (size_t)(reduce_groups(nblk) + 1) * cap;
+    counters = (unsigned*)E->get_ws("cg.counters", cbytes, &rc);
     if (rc) return rc;
-    ODWF_CK(cudaMemsetAsync(counters, 0, sizeof(unsigned) * cap, s));
+    ODWF_CK(cudaMemsetAsync(counters, 0, cbytes, s));
     // pinned: state mirror [cap], initial-state staging [cap], r staging [cap]
     if (cudaMallocHost(&st_host, 2 * sizeof(SysState) * cap + sizeof(double) * cap) != cudaSuccess) {
         cudaGetLastError();
@@ -466,9 +467,10 @@ bool BatchCG::slot_finished(int i) const {
 }
 
 int BatchCG::any_running() const {
+    int n = 0;
     for (int i = 0; i < cap; ++i)
-        if (active[i] && (slot_running(i) || upd[i])) return 1;
-    return 0;
+        if (active[i] && (slot_running(i) || upd[i])) ++n;
+    return n;
 }
 
 int BatchCG::resume(cudaStream_t s, bool block) {

@@ -59,9 +59,9 @@ struct BatchCG {
     SysState* st = nullptr;        // device [cap]
     SysState* st_host = nullptr;   // pinned mirror
     double* r_dev = nullptr;       // device [cap]
-    double* partials = nullptr;    // device [cap * nblk]
+    double* partials = nullptr;    // device, see reduce_and_finalize
     int nblk = 0;                  // partials per system (every reducing launch's grid fits)
-    unsigned* counters = nullptr;  // device [cap]
+    unsigned* counters = nullptr;  // device, see reduce_and_finalize
     // reliable updates run on their own stream, overlapping the other systems' iterations
     cudaStream_t s_rel = nullptr;
     std::vector<cudaEvent_t> ev_rel;  // per slot: end of its update on s_rel
@@ -113,7 +113,7 @@ struct BatchCG {
     int set_state(int slot, const SysState& init, double r, cudaStream_t s);
     bool slot_running(int i) const;
     bool slot_finished(int i) const;
-    int any_running() const;
+    int any_running() const;  // how many systems still iterate or wait for an update
 
    private:
     template <class R>

@@ -95,7 +95,7 @@ int Engine::solve_full(void* x, const void* b, const odwf_solve_params* prm, odw
     };
     auto norm2 = [&](const HalfField& a, double* out) -> int {
         ODWF_CK(launch_vec(Sp::F64, Sp::F64, a.ref_sys(0), a.ref_sys(0), n5, ns, 3, 0.0, bc.st, 0, 0, bc.partials,
-                           bc.counters, 0, 1, st));
+                           bc.counters, 0, 1, st, bc.nblk));
         ODWF_CK(cudaMemcpyAsync(out, &bc.st[0].sum, sizeof(double), cudaMemcpyDeviceToHost, st));
         ODWF_CK(cudaStreamSynchronize(st));
         return ODWF_OK;

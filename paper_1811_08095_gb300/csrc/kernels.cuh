@@ -13,6 +13,7 @@
 // last block to finish, which also updates the per-system CG scalars.
 #pragma once
 
+#include "kernels.h"
 #include "odwf_internal.h"
 
 namespace odwf {
@@ -86,9 +87,9 @@ struct HopParams {
     int gate;                   // 1: run only systems whose st[sys].status == need_status
     int need_status;
     SysState* st;               // per-system scalars (gate / norm / cg / resid)
-    double* partials;           // [sys][part_stride] (part_stride 0: gridDim.x)
-    int part_stride;            // partials per system, fixed for every launch of one batch
-    unsigned* counters;         // [sys]
+    double* partials;           // reduce_and_finalize's partials and counters
+    int part_stride;            // most blocks of a reducing launch, fixed for every launch of one batch
+    unsigned* counters;
     int sys_base;               // system index offset (blockIdx.y + sys_base)
     unsigned long long* prof_count;  // optional: counts running (system, launch) pairs
     const double* tab5;              // fixed-point hops: fifth-dimension scan tables (Engine::init)
@@ -205,25 +206,6 @@ __device__ __forceinline__ float warp_sum(float v) {
     for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
     return v;
 }
-// Deterministic block sum (fixed tree for a fixed blockDim); result valid in thread 0.
-// The per-thread values and the sum over a warp are taken in the kernel's arithmetic type
-// R (FP32 in the mixed-precision kernels: GB300's FP64 rate is a small fraction of its
-// FP32 rate), the sums across warps, blocks and the grid in FP64.
-template <class R>
-__device__ __forceinline__ double block_sum(R v, double* sm) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    v = warp_sum(v);
-    __syncthreads();
-    if (lane == 0) sm[wid] = (double)v;
-    __syncthreads();
-    double t = 0.0;
-    if (wid == 0) {
-        t = lane < nw ? sm[lane] : 0.0;
-        t = warp_sum(t);
-    }
-    return t;
-}
-
 __device__ __forceinline__ void finalize_scalar(SysState* st, double total, int fin) {
     if (fin == FIN_STORE) {
         st->sum = total;
@@ -241,58 +223,82 @@ __device__ __forceinline__ void finalize_scalar(SysState* st, double total, int 
         if (!isfinite(rr_new)) {
             st->status = kBreakdown;
         } else if (rr_new <= st->stop_in || st->iter >= st->max_iter ||
-                   (st->reliable && sqrt(rr_new) < st->delta * st->r_max)) {
+                   (st->reliable && rr_new < (st->delta * st->r_max) * (st->delta * st->r_max))) {
             // park the system: the host recomputes the true residual in FP64 (and, in mixed
             // precision, folds the inner solution into the FP64 one) before it continues
             st->status = kNeedUpdate;
         } else {
             st->beta = rr_new / st->rr;
             st->rr = rr_new;
-            st->r_max = fmax(st->r_max, sqrt(rr_new));
+            if (rr_new > st->r_max * st->r_max) st->r_max = sqrt(rr_new);
         }
     }
 }
 
-// Block-level reduction of `v` for system `sys`; the last block to arrive sums the
-// partials in index order and finalizes.
-// Per-block sum of v (the kernel's arithmetic type within a warp, FP64 across warps), written to
-// the system's partial of this block; the last block to finish (counted atomically) sums the
-// partials in index order and finalizes the scalar.  One block barrier: after it the other warps
-// leave and warp 0 alone writes the partial and, in the last block, sums all partials.  The sum
-// order is fixed whatever block finishes last, so results are deterministic.  Must be the
-// kernel's last statement (warps other than 0 return here).
-// System sys's partials start at sys * part_stride (part_stride >= every grid's block count, the same
-// for every launch of a batch, so that launches of different block counts for different systems can
-// run concurrently); part_stride 0 means gridDim.x.
+// Sum of n partials in a fixed order by one warp, valid in lane 0: eight independent loads in flight
+// per lane (the partials lie in L2; taken one at a time they cost a round trip each)
+__device__ __forceinline__ double sum_partials(const double* part, int n, int lane) {
+    double t = 0.0;
+    for (int i = lane; i < n; i += kReduceGroup) {
+        double a[kReduceGroup / 32];
+#pragma unroll
+        for (int k = 0; k < kReduceGroup / 32; ++k) a[k] = i + 32 * k < n ? __ldcg(part + i + 32 * k) : 0.0;
+#pragma unroll
+        for (int k = 0; k < kReduceGroup / 32; ++k) t += a[k];
+    }
+    return warp_sum(t);
+}
+
+// Sum over the grid of v (the kernel's arithmetic type within a warp, FP64 above) for system `sys`.
+// Each block writes its partial; the last block of a group of kReduceGroup blocks to finish (counted
+// atomically) sums the group's, and the last group to finish sums the groups' and finalizes the
+// scalar.  Two levels, so that a grid of thousands of blocks does not end in one warp walking all
+// partials.  The sum order is fixed whatever block finishes last: results are deterministic.  One
+// block barrier: after it the other warps leave.  Must be the kernel's last statement (warps other
+// than 0 return here).
+// part_stride: the most blocks any reducing launch of the batch has; a system owns part_stride partials
+// and reduce_groups(part_stride) group partials, and reduce_groups(part_stride) + 1 counters, so that
+// launches of different block counts for different systems can run concurrently.
 template <class R>
 __device__ __forceinline__ void reduce_and_finalize(R v, double* partials, unsigned* counters, SysState* st,
                                                     int sys, int fin, int part_stride) {
-    __shared__ double sm[32];
+    __shared__ R sm[32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
     v = warp_sum(v);
-    if (lane == 0) sm[wid] = (double)v;
+    if (lane == 0) sm[wid] = v;
     __syncthreads();
     if (wid != 0) return;
-    double bs = lane < nw ? sm[lane] : 0.0;
-    bs = warp_sum(bs);
-    const int nb = gridDim.x;
-    double* part = partials + (size_t)sys * (size_t)(part_stride > 0 ? part_stride : nb);
-    unsigned prev = 0;
+    double bs = lane < nw ? (double)sm[lane] : 0.0;
+    for (int off = 16; off > 0; off >>= 1)
+        if (off < nw) bs += __shfl_down_sync(0xffffffffu, bs, off);
+    const int nb = gridDim.x, ng = reduce_groups(nb), g = blockIdx.x / kReduceGroup;
+    const int in_group = min(kReduceGroup, nb - g * kReduceGroup);
+    const int sg = reduce_groups(part_stride);
+    double* part = partials + (size_t)sys * (part_stride + sg);
+    double* gpart = part + part_stride;
+    unsigned* cnt = counters + (size_t)sys * (sg + 1);
+    unsigned last = 0;
     if (lane == 0) {
         part[blockIdx.x] = bs;
         __threadfence();
-        prev = atomicAdd(counters + sys, 1u);
+        last = atomicAdd(cnt + g, 1u) == (unsigned)(in_group - 1);
     }
-    prev = __shfl_sync(0xffffffffu, prev, 0);
-    if (prev != (unsigned)(nb - 1)) return;
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
     __threadfence();
-    double t = 0.0;
-    for (int i = lane; i < nb; i += 32) t += *((volatile double*)(part + i));
-    t = warp_sum(t);
-    if (lane == 0) {
-        finalize_scalar(st + sys, t, fin);
-        counters[sys] = 0u;
+    double t = sum_partials(part + g * kReduceGroup, in_group, lane);
+    if (lane == 0) cnt[g] = 0u;
+    if (ng > 1) {
+        if (lane == 0) {
+            gpart[g] = t;
+            __threadfence();
+            last = atomicAdd(cnt + sg, 1u) == (unsigned)(ng - 1);
+        }
+        if (!__shfl_sync(0xffffffffu, last, 0)) return;
+        __threadfence();
+        t = sum_partials(gpart, ng, lane);
+        if (lane == 0) cnt[sg] = 0u;
     }
+    if (lane == 0) finalize_scalar(st + sys, t, fin);
 }
 
 // ---------------------------------------------------------------- the fused hopping kernel

@@ -10,6 +10,9 @@ namespace odwf {
 // Reducing kernels write one partial per block and system; the buffer is sized for blocks of at
 // least this many threads, each thread one 5D site (or more).
 constexpr int kMinReduceBlock = 64;
+// Partials are summed in groups of this many blocks (reduce_and_finalize)
+constexpr int kReduceGroup = 256;
+__host__ __device__ constexpr int reduce_groups(int blocks) { return (blocks + kReduceGroup - 1) / kReduceGroup; }
 
 
 enum class Sp { F64 = 0, F32 = 1, F16 = 2, BF16 = 3, FX = 4 };  // FX: block fixed point (fx.cuh)
@@ -74,6 +77,11 @@ cudaError_t launch_hop_mixed(const HopParams<float>& P, Epi e, Sp low, Lk lk, in
 
 // Second-generation mixed CG kernels (Ns = 8 or 16): kind 1..4 = K1..K4 of the iteration
 // (see kernels_mixed2.cu); the non-dagger hops read chi = B psi fields.
+// Launches of at most 16384 half-precision 5D sites (all systems) take the one-s-per-lane kernels with
+// every neighbour fetched up front: they are bound by the chain of memory latencies of one block.  One
+// GB300, FP16: 4^4x8 (1024 sites) K1 6.2 -> 4.2 us, K2 10.2 -> 8.3; 8^4x8 (16384) K2 10.4 -> 8.3, K4
+// 11.5 -> 10.3; 8^4x16 (32768) K2 10.6 -> 12.4.
+bool hop_deep(Sp low, size_t n5);
 bool hop2_supported(int ns, Sp low, size_t vh);
 cudaError_t launch_hop2(const HopParams<float>& P, int kind, Sp low, Lk lk, int nsys, cudaStream_t st);
 // The hops K1, K2, K3 with two adjacent s per lane (kernels_mixed3.cu): Ns = 8 or 16, FP16 / BF16.
@@ -103,7 +111,7 @@ cudaError_t launch_unpack(Sp sp, const FieldRef& in, double2* ext, const Geom& g
                           cudaStream_t st);
 
 // Vector kernels (kinds as in kernels.cuh); x and y formats given separately
-// part_stride: partials per system of a reducing launch (kind 3), 0 for the grid's block count
+// part_stride: as HopParams::part_stride, for a reducing launch (kind 3)
 cudaError_t launch_vec(Sp spx, Sp spy, const FieldRef& x, const FieldRef& y, size_t n5, int ns, int kind,
                        double coef, SysState* st, int gate, int need, double* partials,
                        unsigned* counters, int sys_base, int nsys, cudaStream_t stream, int part_stride = 0);

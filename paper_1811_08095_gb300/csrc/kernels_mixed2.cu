@@ -27,9 +27,14 @@ namespace {
 using namespace mx;
 
 constexpr int kBS2 = 256;
+constexpr int kBS2Deep = 64;
 
-template <class SP, class LK, int NS, int KIND>
-__global__ void __launch_bounds__(kBS2, 3) hop2_kernel(const HopParams<float> P) {
+// DEEP: all eight neighbours are fetched before the first is used, in blocks of 64 threads (see
+// hop_deep for when)
+template <class SP, class LK, int NS, int KIND, bool DEEP>
+__global__ void __launch_bounds__(DEEP ? kBS2Deep : kBS2, DEEP ? 4 : 3) hop2_kernel(const HopParams<float> P) {
+    constexpr int BS = DEEP ? kBS2Deep : kBS2;
+    constexpr int AHEAD = DEEP ? 8 : 2;  // neighbours in flight
     constexpr int kLS = 18;            // floats per staged link: 9 x (ur, ui)
     constexpr int kSL = 8 * kLS + 4;   // floats per site (padding spreads banks)
     constexpr bool DAG = (KIND == K3 || KIND == K4);
@@ -60,11 +65,17 @@ __global__ void __launch_bounds__(kBS2, 3) hop2_kernel(const HopParams<float> P)
         }
     }
 
+    const void* in = P.in.d(sys);
+    const float* in_n = P.in.n(sys);
+    RawSite<SP> rs[AHEAD];
+#pragma unroll
+    for (int j = 0; j < AHEAD - 1 + (DEEP ? 1 : 0); ++j) fetch_site<SP>(in, in_n, (unsigned)nb[j], s, NS, rs[j]);
+
     // stage the site's eight links in shared memory as (ur, ui) pairs: lane d < 8 of the group
     // loads direction d from the site-major link array (the eight links of a site are contiguous,
     // so the loads neither wait for the neighbour table nor scatter); the group's Ns lanes then
     // read them (the group lies in one warp)
-    __shared__ __align__(16) float s_links[(kBS2 / NS) * kSL];
+    __shared__ __align__(16) float s_links[(BS / NS) * kSL];
     float* my_links = s_links + (threadIdx.x / NS) * kSL;
     if (lane < 8) {
         float u[18];
@@ -75,22 +86,19 @@ __global__ void __launch_bounds__(kBS2, 3) hop2_kernel(const HopParams<float> P)
     }
     __syncwarp();
 
-    const void* in = P.in.d(sys);
-    const float* in_n = P.in.n(sys);
     HopAcc A;
     A.clear();
     const float2* L2p = reinterpret_cast<const float2*>(my_links);
     // forward hops use (1 - gamma) for D and (1 + gamma) for D^dag; backward the opposite
-    // neighbour j + 1 is fetched before neighbour j is processed
-    RawSite<SP> rs[2];
-    fetch_site<SP>(in, in_n, (unsigned)nb[0], s, NS, rs[0]);
+    // neighbour j + AHEAD - 1 is fetched before neighbour j is processed
 #define ODWF_HOP_DIR(MU_, DIR_)                                                                                   \
     {                                                                                                             \
         constexpr int j_ = 2 * MU_ + DIR_;                                                                        \
-        if (j_ < 7) fetch_site<SP>(in, in_n, (unsigned)nb[j_ + 1 < 8 ? j_ + 1 : 7], s, NS, rs[(j_ + 1) & 1]);        \
+        if (!DEEP && j_ < 7)                                                                                      \
+            fetch_site<SP>(in, in_n, (unsigned)nb[j_ + 1 < 8 ? j_ + 1 : 7], s, NS, rs[(j_ + 1) % AHEAD]);          \
         const float sgn_ = (flip & (1u << j_)) ? -1.f : 1.f;                                                     \
         const LinkStaged2 ls_{L2p + j_ * 9};                                                                      \
-        hop_dir_packed<SP, MU_, DIR_ == 1, (DIR_ == 0) == DAG>(rs[j_ & 1], sgn_, ls_, A);                        \
+        hop_dir_packed<SP, MU_, DIR_ == 1, (DIR_ == 0) == DAG>(rs[j_ % AHEAD], sgn_, ls_, A);                    \
     }
     ODWF_HOP_DIR(0, 0); ODWF_HOP_DIR(0, 1);
     ODWF_HOP_DIR(1, 0); ODWF_HOP_DIR(1, 1);
@@ -211,18 +219,32 @@ __global__ void __launch_bounds__(kBS2) p_update2_kernel(FieldRef rr, FieldRef p
     if (valid) SpinorIO<SP, float>::store(chi.d(sys), chi.n(sys), h, s, NS, v);
 }
 
-template <class SP, class LK, int NS>
-cudaError_t hop2_k(const HopParams<float>& P, int kind, int nsys, cudaStream_t st) {
+template <class SP, class LK, int NS, bool DEEP>
+cudaError_t hop2_kd(const HopParams<float>& P, int kind, int nsys, cudaStream_t st) {
+    constexpr int BS = DEEP ? kBS2Deep : kBS2;
+    // the others run as hop3 kernels
+    constexpr bool all = DEEP || std::is_same<SP, SpF32>::value;
     const size_t n = (size_t)P.g.Vh * NS;
-    dim3 grid(blocks_for(n, kBS2), nsys);
-    note_launch();
-    switch (kind) {
-        case K1: hop2_kernel<SP, LK, NS, K1><<<grid, kBS2, 0, st>>>(P); break;
-        case K2: hop2_kernel<SP, LK, NS, K2><<<grid, kBS2, 0, st>>>(P); break;
-        case K3: hop2_kernel<SP, LK, NS, K3><<<grid, kBS2, 0, st>>>(P); break;
-        default: hop2_kernel<SP, LK, NS, K4><<<grid, kBS2, 0, st>>>(P); break;
+    dim3 grid(blocks_for(n, BS), nsys);
+    if (kind == K4) {
+        note_launch();
+        hop2_kernel<SP, LK, NS, K4, DEEP><<<grid, BS, 0, st>>>(P);
+    } else if constexpr (all) {
+        note_launch();
+        if (kind == K1) hop2_kernel<SP, LK, NS, K1, DEEP><<<grid, BS, 0, st>>>(P);
+        else if (kind == K2) hop2_kernel<SP, LK, NS, K2, DEEP><<<grid, BS, 0, st>>>(P);
+        else hop2_kernel<SP, LK, NS, K3, DEEP><<<grid, BS, 0, st>>>(P);
+    } else {
+        return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
+}
+
+template <class SP, class LK, int NS>
+cudaError_t hop2_k(const HopParams<float>& P, int kind, int nsys, cudaStream_t st) {
+    if constexpr (!std::is_same<SP, SpF32>::value)
+        if (hop_deep(Sp::F16, (size_t)P.g.Vh * NS * nsys)) return hop2_kd<SP, LK, NS, true>(P, kind, nsys, st);
+    return hop2_kd<SP, LK, NS, false>(P, kind, nsys, st);
 }
 
 template <class SP, class LK>
@@ -267,6 +289,8 @@ cudaError_t pupd_ns(int ns, const FieldRef& r, const FieldRef& p, const FieldRef
 }
 
 }  // namespace
+
+bool hop_deep(Sp low, size_t n5) { return low != Sp::F32 && n5 <= 16384; }
 
 bool hop2_supported(int ns, Sp low, size_t vh) {
     // 32-bit chunk indices: a half field must have fewer than 2^32 16-byte chunks

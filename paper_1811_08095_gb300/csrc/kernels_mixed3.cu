@@ -381,7 +381,7 @@ cudaError_t launch_hop3(const HopParams<float>& P, int kind, Sp low, Lk lk, int 
 }
 
 cudaError_t launch_hop_prod(const HopParams<float>& P, int kind, Sp low, Lk lk, int nsys, cudaStream_t st) {
-    return hop3_supported(P.ns, low, kind) ? launch_hop3(P, kind, low, lk, nsys, st)
+    return hop3_supported(P.ns, low, kind) && !hop_deep(low, (size_t)P.g.Vh * P.ns * nsys) ? launch_hop3(P, kind, low, lk, nsys, st)
                                            : launch_hop2(P, kind, low, lk, nsys, st);
 }
 
