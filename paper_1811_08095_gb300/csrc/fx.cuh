@@ -122,4 +122,11 @@ __device__ __forceinline__ void fx_load_double(const void* base, const int* ex, 
 // 64-bit accumulation of a 32 x 32-bit product (one instruction)
 __device__ __forceinline__ long long fx_mad(int a, int b, long long c) { return (long long)a * b + c; }
 
+// -a, opaque to the compiler: it would turn c + (-a) b into a product and a 64-bit subtraction
+__device__ __forceinline__ int fx_neg(int a) {
+    int r;
+    asm("neg.s32 %0, %1;" : "=r"(r) : "r"(a));
+    return r;
+}
+
 }  // namespace odwf

@@ -99,6 +99,13 @@ struct HopParams {
     Coef5<R> cf;
 };
 
+// site s (coordinates c) moved one step along mu (dir > 0: forward), periodic
+__device__ __forceinline__ size_t gauge_shift(const GaugeLex& g, const int c[4], size_t s, int mu, int dir) {
+    const int x = c[mu];
+    if (dir > 0) return x + 1 == g.L[mu] ? s - (size_t)(g.L[mu] - 1) * g.stride[mu] : s + g.stride[mu];
+    return x == 0 ? s + (size_t)(g.L[mu] - 1) * g.stride[mu] : s - g.stride[mu];
+}
+
 // ---------------------------------------------------------------- spin algebra (chiral basis)
 // gamma_mu = [[0, G_mu], [G_mu^dag, 0]]:  G_1 = -i s1, G_2 = -i s2, G_3 = -i s3, G_4 = 1.
 // (1 + sg gamma_mu) chi = [h ; sg G^dag h] with h = chi^up + sg G chi^dn.

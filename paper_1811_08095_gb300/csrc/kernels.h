@@ -68,8 +68,19 @@ cudaError_t launch_sum_partials(const double* partials, int nb, double* out, cud
 // gauge force: F (may be null) = -(beta/3) ta(U Sigma) per link; *retr_sum = sum_links Re tr(U Sigma)
 // (partials: gauge_force_blocks(V) doubles)
 size_t gauge_force_blocks(size_t V);
-cudaError_t launch_gauge_force(const int dims[4], const double2* U, double beta, double2* F, double* partials,
-                               double* retr_sum, cudaStream_t st);
+// work: gauge_force_work(V) bytes for the fixed-point kernel (kernels_gauge_fx.cu), or null to run in FP64
+size_t gauge_force_work(size_t V);
+cudaError_t launch_gauge_force(const int dims[4], const double2* U, void* work, double beta, double2* F,
+                               double* partials, double* retr_sum, cudaStream_t st);
+// lexicographic sites of the external gauge layout
+struct GaugeLex {
+    int L[4];
+    size_t stride[4];
+    size_t V;
+};
+// its split and force kernels; work = 36 V int4 limbs and the flag of links outside the fixed-point range
+cudaError_t launch_gauge_force_fx(const GaugeLex& g, const double2* U, void* work, double beta, double2* F,
+                                  double* partials, cudaStream_t st);
 cudaError_t launch_link_update(size_t nlinks, double2* U, const double2* P, double a, cudaStream_t st);  // U <- exp(aP) U
 cudaError_t launch_axpy(size_t n, double2* y, const double2* x, double c, cudaStream_t st);              // y += c x
 // Mixed path (low-precision operator fields, FP32 accumulators r/x, float links, FP32 arithmetic)

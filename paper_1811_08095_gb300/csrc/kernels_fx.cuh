@@ -139,7 +139,7 @@ __device__ __forceinline__ void fx_dir(const int4* __restrict__ p, int ns, const
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
             const int4 u = U[3 * a + b];
-            const int m1 = -u.z, m0 = -u.w;
+            const int m1 = fx_neg(u.z), m0 = fx_neg(u.w);
 #pragma unroll
             for (int sp = 0; sp < 2; ++sp) {
                 const FxLimbs x = h[b][2 * sp], y = h[b][2 * sp + 1];

@@ -65,21 +65,12 @@ __device__ __forceinline__ Z3 mdm(const Z3& a, const Z3& b) {  // a^+ b
     return c;
 }
 
-struct Lex {
-    int L[4];
-    size_t stride[4];
-    size_t V;
-};
-
-__device__ __forceinline__ size_t shift(const Lex& g, const int c[4], size_t s, int mu, int dir) {
-    const int x = c[mu];
-    if (dir > 0) return x + 1 == g.L[mu] ? s - (size_t)(g.L[mu] - 1) * g.stride[mu] : s + g.stride[mu];
-    return x == 0 ? s + (size_t)(g.L[mu] - 1) * g.stride[mu] : s - g.stride[mu];
-}
-
-// one thread per link (mu, s): Pi (optional) and per-block sums of Re tr(U Sigma)
-__global__ void __launch_bounds__(kBSM) gauge_force_kernel(Lex g, const double2* __restrict__ U, double beta,
-                                                           double2* __restrict__ F, double* __restrict__ part) {
+// one thread per link (mu, s): Pi (optional) and per-block sums of Re tr(U Sigma); for fields the
+// fixed-point kernel (kernels_gauge_fx.cu) does not take
+__global__ void __launch_bounds__(kBSM) gauge_force_kernel(GaugeLex g, const double2* __restrict__ U, double beta,
+                                                           double2* __restrict__ F, double* __restrict__ part,
+                                                           const int* __restrict__ run) {
+    if (run && !*run) return;
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     double retr = 0.0;
     if (i < 4 * g.V) {
@@ -94,14 +85,14 @@ __global__ void __launch_bounds__(kBSM) gauge_force_kernel(Lex g, const double2*
         Z3 S;
 #pragma unroll
         for (int k = 0; k < 9; ++k) S.m[k] = make_double2(0.0, 0.0);
-        const size_t xm = shift(g, c, s, mu, +1);
+        const size_t xm = gauge_shift(g, c, s, mu, +1);
 #pragma unroll 1
         for (int nu = 0; nu < 4; ++nu) {
             if (nu == mu) continue;
-            const size_t xn = shift(g, c, s, nu, +1), xb = shift(g, c, s, nu, -1);
+            const size_t xn = gauge_shift(g, c, s, nu, +1), xb = gauge_shift(g, c, s, nu, -1);
             int cb[4] = {c[0], c[1], c[2], c[3]};
             cb[nu] = c[nu] == 0 ? g.L[nu] - 1 : c[nu] - 1;
-            const size_t xmb = shift(g, cb, xb, mu, +1);  // x + mu - nu
+            const size_t xmb = gauge_shift(g, cb, xb, mu, +1);  // x + mu - nu
             // upper: U_nu(x+mu) U_mu(x+nu)^+ U_nu(x)^+
             const Z3 up = mmd(mmd(ld(U, g.V, nu, xm), ld(U, g.V, mu, xn)), ld(U, g.V, nu, s));
             // lower: U_nu(x+mu-nu)^+ U_mu(x-nu)^+ U_nu(x-nu)
@@ -198,9 +189,11 @@ __global__ void axpy_kernel(size_t n, double2* __restrict__ y, const double2* __
 
 size_t gauge_force_blocks(size_t V) { return (4 * V + kBSM - 1) / kBSM; }
 
-cudaError_t launch_gauge_force(const int dims[4], const double2* U, double beta, double2* F, double* partials,
-                               double* retr_sum, cudaStream_t st) {
-    Lex g;
+size_t gauge_force_work(size_t V) { return 36 * V * sizeof(int4) + sizeof(int4); }
+
+cudaError_t launch_gauge_force(const int dims[4], const double2* U, void* work, double beta, double2* F,
+                               double* partials, double* retr_sum, cudaStream_t st) {
+    GaugeLex g;
     size_t stride = 1;
     for (int d = 0; d < 4; ++d) {
         g.L[d] = dims[d];
@@ -209,8 +202,14 @@ cudaError_t launch_gauge_force(const int dims[4], const double2* U, double beta,
     }
     g.V = stride;
     const size_t nb = gauge_force_blocks(g.V);
+    const int* bad = nullptr;  // with a workspace: the FP64 kernel runs only if the split found a bad link
+    if (work) {
+        const cudaError_t e = launch_gauge_force_fx(g, U, work, beta, F, partials, st);
+        if (e != cudaSuccess) return e;
+        bad = (const int*)((const char*)work + gauge_force_work(g.V) - sizeof(int4));
+    }
     note_launch();
-    gauge_force_kernel<<<(unsigned)nb, kBSM, 0, st>>>(g, U, beta, F, partials);
+    gauge_force_kernel<<<(unsigned)nb, kBSM, 0, st>>>(g, U, beta, F, partials, bad);
     return launch_sum_partials(partials, (int)nb, retr_sum, st);
 }
 

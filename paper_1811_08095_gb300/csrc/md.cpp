@@ -30,9 +30,11 @@ int Engine::gauge_force(const double2* U, double beta, double* action, double2* 
     const size_t nb = gauge_force_blocks(V);
     double* part = (double*)get_ws("md.gpart", (nb + 1) * sizeof(double), &rc);
     if (rc) return rc;
+    // the fixed-point kernel's limbs; a device too full for them runs the FP64 kernel
+    void* work = get_ws("md.glimbs", gauge_force_work(V), &rc);
     {
         ProfScope ps("md.gauge_force", (double)V * 4 * (144 + (F ? 144 : 0)), st);  // U in, F out
-        ODWF_CK(launch_gauge_force(lat.dims, U, beta, F, part, part + nb, st));
+        ODWF_CK(launch_gauge_force(lat.dims, U, work, beta, F, part, part + nb, st));
     }
     if (action) {
         double retr = 0.0;
