@@ -298,7 +298,7 @@ int BatchCG::launch_iterations(int k, int lo, int n, cudaStream_t s) {
     const size_t n5 = E->sites5();
     for (int it = 0; it < k; ++it) {
         if (!mixed) {
-            ODWF_CK(launch_m5_fx(P64.ref(), C64.ref(), E->vh(), E->ns, r_dev, lo, n, FxOp::B, E->cf64, E->fx_tab, s, st, kRunning));
+            ODWF_CK(launch_m5_fx(P64.ref(), C64.ref(), E->g, 0, E->ns, r_dev, lo, n, FxOp::B, E->fx_tab, s, st, kRunning));
             const FieldRef f[5] = {C64.ref(), A64.ref(), C64.ref(), A64.ref(), FieldRef{}};
             const Epi e[4] = {Epi::MINV, Epi::SCHUR_NORM_MDINV, Epi::D_MINVDAG, Epi::D_NORMAL_CG};
             for (int h = 0; h < 4; ++h) {
@@ -500,7 +500,7 @@ int BatchCG::resume(cudaStream_t s, bool block) {
 // shared buffers, B loaded with the slot's right-hand side)
 int BatchCG::fp64_residual(int slot, cudaStream_t s) {
     const FieldRef a = mixed ? A1.ref_shared() : A64.ref(), c = mixed ? C1.ref_shared() : C64.ref();
-    ODWF_CK(launch_m5_fx(X64.ref(), c, E->vh(), E->ns, r_dev, slot, 1, FxOp::B, E->cf64, E->fx_tab, s));
+    ODWF_CK(launch_m5_fx(X64.ref(), c, E->g, 0, E->ns, r_dev, slot, 1, FxOp::B, E->fx_tab, s));
     const FieldRef f[5] = {c, a, c, a, Rref()};
     const Epi e[4] = {Epi::MINV, Epi::SCHUR_MDINV, Epi::D_MINVDAG, Epi::D_NORMAL_RESID};
     for (int h = 0; h < 4; ++h) {

@@ -96,23 +96,29 @@ int Engine::init(const odwf_lattice* l, int Ns, double m0_, double mq_, const do
     }
     ODWF_CK(cudaGetDevice(&device));
     int rc = 0;
-    // scan tables of the fixed-point hops' M^-1 (fx_minv): 1/d, then al and its running product for
-    // M^-1 up (forward, e_s), M^-1 down (backward, e_s), M^-dag up (backward, e_{s+1}), down (forward, e_{s-1})
+    // tables of the fixed-point hops' operators along s (fx_columns), for the upper spins and, with s
+    // reversed, for the lower: 1/d; al and its running product for M^-1 (up forward, down backward, e_s)
+    // and for M^-dag (up backward with e_{s+1}, down forward with e_{s-1}); omega/d; omega; d; e
     std::vector<double> tab{mq / (2.0 * m0), 0.0};  // the handle's r comes first (16 bytes)
-    tab.insert(tab.end(), cf64.inv_d, cf64.inv_d + Ns);
-    for (int v = 0; v < 4; ++v) {
-        std::vector<double> al(Ns), A(Ns);
-        for (int s = 0; s < Ns; ++s)
-            al[s] = -cf64.e[v == 2 ? (s + 1) % Ns : v == 3 ? (s + Ns - 1) % Ns : s] * cf64.inv_d[s];
-        const bool fwd = v == 0 || v == 3;
-        double prod = 1.0;
-        for (int n = 0; n < Ns; ++n) {
-            const int s = fwd ? n : Ns - 1 - n;
-            prod *= al[s];
-            A[s] = prod;
+    for (int down = 0; down < 2; ++down) {
+        std::vector<double> t[9];
+        for (auto& v : t) v.resize(Ns);
+        for (int i = 0; i < Ns; ++i) {
+            const int s = down ? Ns - 1 - i : i;
+            t[0][i] = cf64.inv_d[s];
+            t[1][i] = -cf64.e[s] * cf64.inv_d[s];
+            t[3][i] = -cf64.e[(s + (down ? Ns - 1 : 1)) % Ns] * cf64.inv_d[s];
+            t[5][i] = w[s] * cf64.inv_d[s];
+            t[6][i] = w[s];  // rho = sigma = omega
+            t[7][i] = cf64.d[s];
+            t[8][i] = cf64.e[s];
         }
-        tab.insert(tab.end(), al.begin(), al.end());
-        tab.insert(tab.end(), A.begin(), A.end());
+        double fwd = 1.0, bwd = 1.0;
+        for (int i = 0; i < Ns; ++i) {
+            t[2][i] = fwd *= t[1][i];
+            t[4][Ns - 1 - i] = bwd *= t[3][Ns - 1 - i];
+        }
+        for (auto& v : t) tab.insert(tab.end(), v.begin(), v.end());
     }
     double* rd = (double*)get_ws("r_handle", tab.size() * sizeof(double), &rc);
     if (rc) return rc;
@@ -305,7 +311,7 @@ int Engine::apply_schur64(const HalfField& in, const HalfField& out, bool dag, c
     int rc = 0;
     HalfField T, A;
     if ((rc = alloc_half("op.T", Sp::FX, 1, &T)) || (rc = alloc_half("op.A", Sp::FX, 1, &A))) return rc;
-    ODWF_CK(launch_m5_fx(in.ref_sys(0), A.ref_sys(0), vh(), ns, r_dev, 0, 1, dag ? FxOp::MINVDAG : FxOp::B, cf64, fx_tab, st));
+    ODWF_CK(launch_m5_fx(in.ref_sys(0), A.ref_sys(0), g, 0, ns, r_dev, 0, 1, dag ? FxOp::MINVDAG : FxOp::B, fx_tab, st));
     auto P = hop_params<double>(1, r_dev);
     P.in = A.ref_sys(0);
     P.out = T.ref_sys(0);
@@ -321,13 +327,14 @@ int Engine::apply_schur64(const HalfField& in, const HalfField& out, bool dag, c
 int Engine::apply_full64(const HalfField& in_e, const HalfField& in_o, const HalfField& out_e,
                          const HalfField& out_o, bool dag, const double* r_dev, cudaStream_t st) {
     int rc = 0;
-    HalfField A;
-    if ((rc = alloc_half("op.A", Sp::FX, 1, &A))) return rc;
+    HalfField F[2];  // the hops' inputs on even and odd sites, both read before out (which may be in) is written
+    if ((rc = alloc_half("op.T", Sp::FX, 1, &F[0])) || (rc = alloc_half("op.A", Sp::FX, 1, &F[1]))) return rc;
+    for (int p = 0; p < 2; ++p)
+        ODWF_CK(launch_m5_fx((p == 0 ? in_e : in_o).ref_sys(0), F[p].ref_sys(0), g, p, ns, r_dev, 0, 1,
+                             dag ? FxOp::ID : FxOp::B, fx_tab, st));
     for (int p = 0; p < 2; ++p) {
-        const HalfField& other = p == 0 ? in_o : in_e;
-        ODWF_CK(launch_m5_fx(other.ref_sys(0), A.ref_sys(0), vh(), ns, r_dev, 0, 1, dag ? FxOp::ID : FxOp::B, cf64, fx_tab, st));
         auto P = hop_params<double>(p, r_dev);
-        P.in = A.ref_sys(0);
+        P.in = F[1 - p].ref_sys(0);
         P.z = (p == 0 ? in_e : in_o).ref_sys(0);
         P.out = (p == 0 ? out_e : out_o).ref_sys(0);
         ODWF_CK(launch_hop_fx(P, dag ? Epi::D_FULL : Epi::FULL, 1, st));
@@ -340,7 +347,7 @@ int Engine::apply_normal64(const HalfField& in, const HalfField& out, const doub
     int rc = 0;
     HalfField T, A;
     if ((rc = alloc_half("op.T", Sp::FX, 1, &T)) || (rc = alloc_half("op.A", Sp::FX, 1, &A))) return rc;
-    ODWF_CK(launch_m5_fx(in.ref_sys(0), A.ref_sys(0), vh(), ns, r_dev, 0, 1, FxOp::B, cf64, fx_tab, st));
+    ODWF_CK(launch_m5_fx(in.ref_sys(0), A.ref_sys(0), g, 0, ns, r_dev, 0, 1, FxOp::B, fx_tab, st));
     const HalfField* f[5] = {&A, &T, &A, &T, &out};
     const Epi e[4] = {Epi::MINV, Epi::SCHUR_MDINV, Epi::D_MINVDAG, Epi::D_NORMAL};
     for (int k = 0; k < 4; ++k) {
@@ -382,20 +389,11 @@ int Engine::apply(void* out, const void* in, int mode, bool dag, cudaStream_t st
     double2* dout = out_dev ? (double2*)out : (double2*)get_ws("ext.out", eb, &rc);
     if (rc) return rc;
     const double* rd = (const double*)ws["r_handle"].p;
-    HalfField Xe, Xo, Ye, Yo;
-    if ((rc = alloc_half("io.Xe", Sp::F64, 1, &Xe)) || (rc = alloc_half("io.Ye", Sp::F64, 1, &Ye))) return rc;
-    if (mode == ODWF_MODE_SCHUR_EVEN) {
-        ODWF_CK(launch_pack(Sp::F64, din, Xe.ref_sys(0), g, 0, ns, 1, st));
-        if ((rc = apply_schur64(Xe, Ye, dag, rd, st))) return rc;
-        ODWF_CK(launch_unpack(Sp::F64, Ye.ref_sys(0), dout, g, 0, ns, 1, st));
-    } else {
-        if ((rc = alloc_half("io.Xo", Sp::F64, 1, &Xo)) || (rc = alloc_half("io.Yo", Sp::F64, 1, &Yo))) return rc;
-        ODWF_CK(launch_pack(Sp::F64, din, Xe.ref_sys(0), g, 0, ns, 0, st));
-        ODWF_CK(launch_pack(Sp::F64, din, Xo.ref_sys(0), g, 1, ns, 0, st));
-        if ((rc = apply_full64(Xe, Xo, Ye, Yo, dag, rd, st))) return rc;
-        ODWF_CK(launch_unpack(Sp::F64, Ye.ref_sys(0), dout, g, 0, ns, 0, st));
-        ODWF_CK(launch_unpack(Sp::F64, Yo.ref_sys(0), dout, g, 1, ns, 0, st));
-    }
+    // the operators read and write the caller's fields in place
+    const int layout = mode == ODWF_MODE_SCHUR_EVEN ? 1 : 2;
+    const HalfField X = HalfField::external(din, layout), Y = HalfField::external(dout, layout);
+    rc = layout == 1 ? apply_schur64(X, Y, dag, rd, st) : apply_full64(X, X, Y, Y, dag, rd, st);
+    if (rc) return rc;
     if (!out_dev) {
         ODWF_CK(cudaMemcpyAsync(out, dout, eb, cudaMemcpyDeviceToHost, st));
         ODWF_CK(cudaStreamSynchronize(st));
@@ -417,23 +415,15 @@ int Engine::apply_normal(void* out, const void* in, int system, cudaStream_t st)
     double2* dout = out_dev ? (double2*)out : (double2*)get_ws("ext.out", eb, &rc);
     if (rc) return rc;
     const double* rd = (const double*)ws["r_handle"].p;
-    HalfField Xe, Ye;
-    if ((rc = alloc_half("io.Xe", Sp::F64, 1, &Xe)) || (rc = alloc_half("io.Ye", Sp::F64, 1, &Ye))) return rc;
-    if (system == ODWF_SYS_SCHUR_NORMAL) {
-        ODWF_CK(launch_pack(Sp::F64, din, Xe.ref_sys(0), g, 0, ns, 1, st));
-        if ((rc = apply_normal64(Xe, Ye, rd, st))) return rc;
-        ODWF_CK(launch_unpack(Sp::F64, Ye.ref_sys(0), dout, g, 0, ns, 1, st));
+    const int layout = system == ODWF_SYS_SCHUR_NORMAL ? 1 : 2;
+    const HalfField X = HalfField::external(din, layout), Y = HalfField::external(dout, layout);
+    if (layout == 1) {
+        if ((rc = apply_normal64(X, Y, rd, st))) return rc;
     } else {
-        HalfField Xo, Yo, Ze, Zo;
-        if ((rc = alloc_half("io.Xo", Sp::F64, 1, &Xo)) || (rc = alloc_half("io.Yo", Sp::F64, 1, &Yo)) ||
-            (rc = alloc_half("io.Ze", Sp::F64, 1, &Ze)) || (rc = alloc_half("io.Zo", Sp::F64, 1, &Zo)))
-            return rc;
-        ODWF_CK(launch_pack(Sp::F64, din, Xe.ref_sys(0), g, 0, ns, 0, st));
-        ODWF_CK(launch_pack(Sp::F64, din, Xo.ref_sys(0), g, 1, ns, 0, st));
-        if ((rc = apply_full64(Xe, Xo, Ze, Zo, false, rd, st))) return rc;
-        if ((rc = apply_full64(Ze, Zo, Ye, Yo, true, rd, st))) return rc;
-        ODWF_CK(launch_unpack(Sp::F64, Ye.ref_sys(0), dout, g, 0, ns, 0, st));
-        ODWF_CK(launch_unpack(Sp::F64, Yo.ref_sys(0), dout, g, 1, ns, 0, st));
+        HalfField Ze, Zo;
+        if ((rc = alloc_half("io.Ze", Sp::F64, 1, &Ze)) || (rc = alloc_half("io.Zo", Sp::F64, 1, &Zo))) return rc;
+        if ((rc = apply_full64(X, X, Ze, Zo, false, rd, st))) return rc;
+        if ((rc = apply_full64(Ze, Zo, Y, Y, true, rd, st))) return rc;
     }
     if (!out_dev) {
         ODWF_CK(cudaMemcpyAsync(out, dout, eb, cudaMemcpyDeviceToHost, st));

@@ -42,10 +42,18 @@ struct HalfField {
     float* norm = nullptr;
     size_t stride = 0;       // bytes per system
     size_t norm_stride = 0;  // floats per system
-    FieldRef ref() const { return FieldRef{data, norm, stride, norm_stride}; }
+    int ext = 0;             // see FieldRef::ext
+    // a caller's complex128 field (device) read or written in place: even-site (1) or full (2) layout
+    static HalfField external(const void* p, int layout) {
+        HalfField f;
+        f.data = const_cast<void*>(p);
+        f.ext = layout;
+        return f;
+    }
+    FieldRef ref() const { return FieldRef{data, norm, stride, norm_stride, ext}; }
     FieldRef ref_shared() const { return FieldRef{data, norm, 0, 0}; }  // same buffer for every system
     FieldRef ref_sys(int i) const {  // system i as a single-system field
-        return FieldRef{(char*)data + i * stride, norm ? norm + i * norm_stride : nullptr, 0, 0};
+        return FieldRef{(char*)data + i * stride, norm ? norm + i * norm_stride : nullptr, 0, 0, ext};
     }
 };
 
@@ -105,7 +113,7 @@ struct Engine {
     template <class R>
     HopParams<R> hop_params(int p_out, const double* r_dev) const;
 
-    // FP64 operators on internal half fields (single system, r from r_dev[0])
+    // FP64 operators on half fields, internal or the caller's (single system, r from r_dev[0])
     int apply_schur64(const HalfField& in, const HalfField& out, bool dag, const double* r_dev, cudaStream_t st);
     int apply_full64(const HalfField& in_e, const HalfField& in_o, const HalfField& out_e, const HalfField& out_o,
                      bool dag, const double* r_dev, cudaStream_t st);

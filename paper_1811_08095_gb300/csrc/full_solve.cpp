@@ -101,8 +101,8 @@ int Engine::solve_full(void* x, const void* b, const odwf_solve_params* prm, odw
         return ODWF_OK;
     };
 
-    auto to_fx = [&](const HalfField& a, FxOp op) {  // F = op(a)
-        return launch_m5_fx(a.ref_sys(0), F.ref_sys(0), vh(), ns, rd, 0, 1, op, cf64, fx_tab, st);
+    auto to_fx = [&](const HalfField& a, FxOp op) {  // F = op(a), an internal field
+        return launch_m5_fx(a.ref_sys(0), F.ref_sys(0), g, 0, ns, rd, 0, 1, op, fx_tab, st);
     };
     auto hop = [&](int p_out, Epi e, const HalfField& z, const HalfField& out) {  // out from F and z
         auto P = hop_params<double>(p_out, rd);

@@ -57,38 +57,6 @@ __device__ __forceinline__ FxLimbs fx_split(long long q) {
 
 __device__ __forceinline__ long long fx_join(int hi, int lo) { return ((long long)hi << 31) + lo; }
 
-__device__ __forceinline__ void fx_store(void* base, int* ex, size_t h, int s, int ns, const double v[24]) {
-    int mx = 0;
-    unsigned mn = 0xffffffffu;  // smallest high word of a nonzero component, less one
-#pragma unroll
-    for (int k = 0; k < 24; ++k) {
-        const int hi = __double2hiint(v[k]) & 0x7fffffff;
-        mx = max(mx, hi);
-        mn = min(mn, (unsigned)(hi - 1));
-    }
-    const int emax = mx >> 20, emin = (int)((mn + 1) >> 20);
-    int4* p = reinterpret_cast<int4*>(base);
-    bool zero = false;
-    if (emax == 0x7ff || emax < kFxMinField || (mn != 0xffffffffu && emax - emin > kFxSpread)) {
-        zero = true;
-        for (int k = 0; k < 24; ++k) zero = zero && v[k] == 0.0;
-        if (!zero) {
-            for (int k = 0; k < 12; ++k)
-                p[chunk_off(h, k, 12, ns, s)] = make_int4(__double2hiint(v[2 * k]), __double2loint(v[2 * k]),
-                                                          __double2hiint(v[2 * k + 1]), __double2loint(v[2 * k + 1]));
-            ex[h * ns + s] = kFxRaw;
-            return;
-        }
-    }
-    const int e = zero ? 2046 : emax;  // an all-zero site: every significand shifted out
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        const FxLimbs re = fx_split(fx_from_double<6>(v[2 * k], e)), im = fx_split(fx_from_double<6>(v[2 * k + 1], e));
-        p[chunk_off(h, k, 12, ns, s)] = make_int4(re.hi, re.lo, im.hi, im.lo);
-    }
-    ex[h * ns + s] = zero ? kFxZero : emax - 1081;  // 1023 + 52 + 6
-}
-
 // q 2^e, the exponent added to the converted double's; |q| < 2^63 and kFxMinExp <= e <= kFxMaxExp for
 // a hop's sums, |q| < 2^59 and any exponent of a stored site: no result leaves the normal range
 constexpr int kFxMinExp = -1000, kFxMaxExp = 950;

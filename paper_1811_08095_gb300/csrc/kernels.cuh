@@ -67,6 +67,7 @@ struct FieldRef {
     float* norm;          // scales of FP16/BF16 fields (nullptr otherwise)
     size_t sys_stride;    // bytes between systems
     size_t norm_stride;   // floats between systems
+    int ext = 0;          // FP64 fields of the fixed-point kernels: 0 internal, 1 / 2 the caller's even-site / full field
     __device__ __forceinline__ void* d(int sys) const { return (char*)data + sys * sys_stride; }
     __device__ __forceinline__ float* n(int sys) const { return norm ? norm + sys * norm_stride : nullptr; }
 };

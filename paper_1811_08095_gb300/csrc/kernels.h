@@ -8,8 +8,8 @@
 namespace odwf {
 
 // Reducing kernels write one partial per block and system; the buffer is sized for blocks of at
-// least this many threads, each thread one 5D site (or more).
-constexpr int kMinReduceBlock = 64;
+// least this many 5D sites.
+constexpr int kMinReduceBlock = 32;
 // Partials are summed in groups of this many blocks (reduce_and_finalize)
 constexpr int kReduceGroup = 256;
 __host__ __device__ constexpr int reduce_groups(int blocks) { return (blocks + kReduceGroup - 1) / kReduceGroup; }
@@ -42,15 +42,16 @@ enum class Epi {
 };
 
 // FP64-accuracy path (kernels_fx.cuh): hops in block fixed point with FP64 links and epilogues.  P.in is
-// a fixed-point field (Sp::FX; chi = B psi for the non-dagger epilogues), P.nbr the neighbour table.
-// MINV writes B M^-1 H p, the next hop's input; MINV, SCHUR_NORM_MDINV, SCHUR_MDINV and D_MINVDAG write
+// a fixed-point field (Sp::FX; (1 + L) psi for the non-dagger epilogues, B = omega (1 + L)), P.nbr the
+// neighbour table.  MINV writes (1 + L) M^-1 H p, the next hop's input; MINV, SCHUR_NORM_MDINV, SCHUR_MDINV and D_MINVDAG write
 // fixed point, the others FP64; z is FP64 except for D_NORMAL, D_NORMAL_CG and D_NORMAL_RESID.
 cudaError_t launch_hop_fx(const HopParams<double>& P, Epi e, int nsys, cudaStream_t st);
-// op(in) of an FP64 field into fixed point
+// z, out and launch_m5_fx's in may be a caller's field (FieldRef::ext).
+// op(in) of an FP64 field on the sites of parity p into fixed point: 1, 1 + L, M^-dag, (1 + L) M^-1
 enum class FxOp { ID, B, MINVDAG, B_MINV };
-cudaError_t launch_m5_fx(const FieldRef& in, const FieldRef& out, size_t n_sites, int ns, const double* r_sys,
-                         int sys_base, int nsys, FxOp op, const Coef5<double>& cf, const double* tab5,
-                         cudaStream_t st, const SysState* gate_st = nullptr, int need = 0);
+cudaError_t launch_m5_fx(const FieldRef& in, const FieldRef& out, const Geom& g, int p, int ns, const double* r_sys,
+                         int sys_base, int nsys, FxOp op, const double* tab5, cudaStream_t st,
+                         const SysState* gate_st = nullptr, int need = 0);
 // the fixed-point link array of n_links FP64 links: 144 bytes per link, then an int exponent per link
 cudaError_t launch_links_fx(const void* d18, void* fx, size_t n_links, cudaStream_t st);
 // Pseudofermion-force contraction (kernels_force.cu): G += coef * [U K1 - K2 U^+] per link from the

@@ -19,45 +19,44 @@ cudaError_t launch_hop_fx(const HopParams<double>& P, Epi e, int nsys, cudaStrea
     }
 }
 
-// out = op(in) of an FP64 field into the fixed-point format
-__global__ void __launch_bounds__(128) m5_fx_kernel(FieldRef in, FieldRef out, size_t n_sites, int ns, int lg_ns,
-                                                    const double* r_sys, int sys_base, FxOp op,
-                                                    const __grid_constant__ Coef5<double> cf, const double* tab5,
-                                                    const SysState* gate_st, int need) {
+// out = op(in) of an FP64 field into the fixed-point format, two threads per 5D site as the hops
+__global__ void __launch_bounds__(kFxThreads) m5_fx_kernel(FieldRef in, FieldRef out, Geom g, int p, int ns, int lg_ns,
+                                                           const double* r_sys, int sys_base, FxOp op,
+                                                           const double* tab5, const SysState* gate_st, int need) {
     extern __shared__ __align__(16) double s_cols[];
     __shared__ double s_fac;
     const int sys = blockIdx.y + sys_base;
     if (gate_st && gate_st[sys].status != need) return;
     const size_t gi = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int s = (int)(gi & (size_t)(ns - 1));
-    const size_t h = gi >> lg_ns;
-    const bool valid = h < n_sites;
+    const FxLane t(threadIdx.x, ns, lg_ns);
+    const int a = t.a, s = t.s;
+    const size_t hh = gi >> (lg_ns + 1);
+    const bool valid = hh < (size_t)g.Vh;
+    const int h = valid ? (int)hh : 0;
+    const int site = threadIdx.x >> (lg_ns + 1), sites = blockDim.x >> (lg_ns + 1);
     const double r = r_sys[sys];
-    double v[24];
-    if (valid) {
-        SpinorIO<SpF64, double>::load(in.d(sys), nullptr, h, s, ns, v);
-    } else {
-#pragma unroll
-        for (int k = 0; k < 24; ++k) v[k] = 0.0;
-    }
-    if (op == FxOp::MINVDAG || op == FxOp::B_MINV) {
-        if (threadIdx.x == 0) s_fac = fx_corner(tab5, r, ns);
+    double v[12];
+    FxF64(in, sys, g, p, h, s, a, ns).load(v);
+    if (op != FxOp::ID) {
+        double* mine = s_cols + site * 24 * (ns + 1);
+        if (op != FxOp::B && threadIdx.x == 0) s_fac = fx_corner(tab5, r, ns);
         __syncthreads();
-        fx_minv(v, s_cols, tab5, s_fac, s, ns, lg_ns, op == FxOp::MINVDAG);
+        const double fac = s_fac;
+        if (op == FxOp::B) fx_turn<C_ONEL>(v, s_cols, mine, s_cols, tab5, r, fac, a, s, sites, ns);
+        else if (op == FxOp::MINVDAG) fx_turn<C_MINVDAG>(v, s_cols, mine, s_cols, tab5, r, fac, a, s, sites, ns);
+        else fx_turn<C_MINV | C_OUTL>(v, s_cols, mine, s_cols, tab5, r, fac, a, s, sites, ns);
     }
-    if (op == FxOp::B || op == FxOp::B_MINV) fx_bidiag(v, cf.rho, cf.sigma, r, s, ns, false);
-    if (valid) fx_store(out.d(sys), reinterpret_cast<int*>(out.n(sys)), h, s, ns, v);
+    fx_store(out.d(sys), reinterpret_cast<int*>(out.n(sys)), (size_t)h, t, ns, valid, v);
 }
 
-cudaError_t launch_m5_fx(const FieldRef& in, const FieldRef& out, size_t n_sites, int ns, const double* r_sys,
-                         int sys_base, int nsys, FxOp op, const Coef5<double>& cf, const double* tab5,
-                         cudaStream_t st, const SysState* gate_st, int need) {
-    const size_t n = n_sites * ns;
-    const int bs = fx_threads(n, ns);
-    const size_t smem = op == FxOp::MINVDAG || op == FxOp::B_MINV ? fx_smem(bs, ns, false) : 0;
+cudaError_t launch_m5_fx(const FieldRef& in, const FieldRef& out, const Geom& g, int p, int ns, const double* r_sys,
+                         int sys_base, int nsys, FxOp op, const double* tab5, cudaStream_t st,
+                         const SysState* gate_st, int need) {
+    const size_t n = (size_t)g.Vh * ns;
+    const int bs = fx_threads(n);
     note_launch();
-    m5_fx_kernel<<<dim3(blocks_for(n, bs), nsys), bs, smem, st>>>(in, out, n_sites, ns, lg2(ns), r_sys, sys_base, op,
-                                                                  cf, tab5, gate_st, need);
+    m5_fx_kernel<<<dim3(blocks_for(2 * n, bs), nsys), bs, op == FxOp::ID ? 0 : fx_smem(bs, ns, 1, false), st>>>(
+        in, out, g, p, ns, lg2(ns), r_sys, sys_base, op, tab5, gate_st, need);
     return cudaGetLastError();
 }
 

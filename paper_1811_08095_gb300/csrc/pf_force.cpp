@@ -42,14 +42,14 @@ int term_fields(Engine* E, const HalfField& A, const HalfField& psi, const doubl
     if ((rc = E->alloc_half("op.A", Sp::FX, 1, &F))) return rc;
     ODWF_CK(launch_m5_f64(A.ref_sys(0), Le.ref_sys(0), vh, ns, r, 0, 1, 3, E->cf64, st));  // L1 = M^-+ A
     ODWF_CK(launch_m5_f64(psi.ref_sys(0), Re.ref_sys(0), vh, ns, r, 0, 1, 4, E->cf64, st));  // B psi
-    ODWF_CK(launch_m5_fx(Re.ref_sys(0), F.ref_sys(0), vh, ns, r, 0, 1, FxOp::ID, E->cf64, E->fx_tab, st));
+    ODWF_CK(launch_m5_fx(psi.ref_sys(0), F.ref_sys(0), E->g, 0, ns, r, 0, 1, FxOp::B, E->fx_tab, st));
     auto P = E->hop_params<double>(1, r);
     P.in = F.ref_sys(0);
     P.out = Ro.ref_sys(0);
     ODWF_CK(launch_hop_fx(P, Epi::PLAIN, 1, st));                                            // H_oe psi
     ODWF_CK(launch_m5_f64(Ro.ref_sys(0), T.ref_sys(0), vh, ns, r, 0, 1, 2, E->cf64, st));  // R1 = M^-1 H_oe psi
     ODWF_CK(launch_m5_f64(T.ref_sys(0), Ro.ref_sys(0), vh, ns, r, 0, 1, 4, E->cf64, st));  // B R1
-    ODWF_CK(launch_m5_fx(Le.ref_sys(0), F.ref_sys(0), vh, ns, r, 0, 1, FxOp::ID, E->cf64, E->fx_tab, st));
+    ODWF_CK(launch_m5_fx(Le.ref_sys(0), F.ref_sys(0), E->g, 0, ns, r, 0, 1, FxOp::ID, E->fx_tab, st));
     P.out = T.ref_sys(0);
     ODWF_CK(launch_hop_fx(P, Epi::D_PLAIN, 1, st));                                          // H_eo^+ L1
     ODWF_CK(launch_m5_f64(T.ref_sys(0), Lo.ref_sys(0), vh, ns, r, 0, 1, 3, E->cf64, st));  // L2

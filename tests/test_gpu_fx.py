@@ -107,3 +107,32 @@ def test_non_finite_values_reach_the_same_sites(torch, bad):
     Ub[1, 2, 1, 3, 0, 1, 1] = bad
     got = _apply(torch, dims, ns, 0.05, w, Ub, syn.gaussian_spinor_even(ns, dims, 9), False)
     assert not np.isfinite(got).all() and np.isfinite(got).any()
+
+
+@pytest.mark.parametrize("ns", [4, 32])
+def test_full_fields_and_in_place(torch, ns):
+    """Operators read and write the caller's fields directly: full fields of both parities on a ragged
+    lattice, and out = in."""
+    dims = (4, 6, 2, 6)
+    U, w = make_case(dims, ns, 0.05, eps=0.6, seed=7)
+    rng = np.random.default_rng(11)
+    shape = (ns, dims[3], dims[2], dims[1], dims[0], 4, 3)
+    psi = rng.standard_normal(shape) + 1j * rng.standard_normal(shape)
+    even = syn.gaussian_spinor_even(ns, dims, 12)
+    with odwf.Handle(dims, ns, M0, 0.05, w) as h:
+        h.set_gauge(to_dev(torch, U))
+        for op in ("apply", "apply_dagger", "apply_normal"):
+            for f in (psi, even):
+                arg = ((odwf.ODWF_SYS_FULL_NORMAL if f is psi else odwf.ODWF_SYS_SCHUR_NORMAL) if op == "apply_normal"
+                       else (odwf.ODWF_MODE_FULL if f is psi else odwf.ODWF_MODE_SCHUR_EVEN))
+                x = to_dev(torch, f)
+                out = torch.empty_like(x)
+                getattr(h, op)(out, x, arg)
+                host = np.empty_like(f)
+                getattr(h, op)(host, f, arg)  # host pointers
+                getattr(h, op)(x, x, arg)
+                assert np.array_equal(from_dev(out), host) and np.array_equal(from_dev(out), from_dev(x))
+                if f is even:
+                    ref = (oracle.normal_op(U, f, M0, 0.05, w) if op == "apply_normal"
+                           else oracle.schur(U, f, M0, 0.05, w, True, dagger=op == "apply_dagger"))
+                    assert_close_componentwise(host, ref, 1e-12)
