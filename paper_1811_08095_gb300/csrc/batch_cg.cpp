@@ -417,6 +417,7 @@ int BatchCG::launch_v2_hops(int lo, int n, cudaStream_t s) {
             P.cg_x = Xin.ref();
             P.cg_p = Pl.ref();
         }
+        P.nb_prev = k == 2 ? hop_blocks(E->ns, low, 2, E->vh(), n) : 0;  // K3 also forms alpha from K2's partials
         auto pb_ = prof_begin(pcls[k], s);
         P.prof_count = pb_.dev_count;
         const cudaError_t e_ = launch_hop_prod(P, k + 1, low, lk, n, s);
@@ -424,6 +425,7 @@ int BatchCG::launch_v2_hops(int lo, int n, cudaStream_t s) {
         P.prof_count = nullptr;
         ODWF_CK(e_);
     }
+    ODWF_CK(launch_beta(partials, hop_blocks(E->ns, low, 4, E->vh(), n), nblk, st, kRunning, lo, n, s));
     return ODWF_OK;
 }
 

@@ -91,6 +91,7 @@ struct HopParams {
     double* partials;           // reduce_and_finalize's partials and counters
     int part_stride;            // most blocks of a reducing launch, fixed for every launch of one batch
     unsigned* counters;
+    int nb_prev;                // production K3: block 0 forms alpha from this many partials of K2 (0: no such block)
     int sys_base;               // system index offset (blockIdx.y + sys_base)
     unsigned long long* prof_count;  // optional: counts running (system, launch) pairs
     const double* tab5;              // fixed-point hops: fifth-dimension scan tables (Engine::init)
@@ -257,6 +258,47 @@ __device__ __forceinline__ double sum_partials(const double* part, int n, int la
     return warp_sum(t);
 }
 
+// Sum of v over the block (the kernel's arithmetic type within a warp, FP64 above), valid in lane 0 of
+// warp 0; the other warps get 0.  One block barrier.
+template <class R>
+__device__ __forceinline__ double block_sum(R v) {
+    __shared__ R sm[32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    v = warp_sum(v);
+    if (lane == 0) sm[wid] = v;
+    __syncthreads();
+    if (wid != 0) return 0.0;
+    double bs = lane < nw ? (double)sm[lane] : 0.0;
+    for (int off = 16; off > 0; off >>= 1)
+        if (off < nw) bs += __shfl_down_sync(0xffffffffu, bs, off);
+    return bs;
+}
+
+// The production mixed hops leave their reduction to a later launch: each block writes its partial and
+// is done, without the fence and the atomic that finding the last block takes (about 6 us at the end of
+// every reducing launch).  alpha, which only K4 needs, is formed by one extra block of K3; beta by
+// beta_kernel before the p update.
+template <class R>
+__device__ __forceinline__ void write_partial(R v, double* partials, int sys, int part_stride) {
+    const double bs = block_sum(v);
+    if (threadIdx.x == 0) partials[(size_t)sys * (part_stride + reduce_groups(part_stride)) + blockIdx.x] = bs;
+}
+
+// One block sums a system's nb partials in a fixed order and finalizes the scalar
+__device__ __forceinline__ void finalize_partials(const double* partials, int nb, SysState* st, int sys, int fin,
+                                                  int part_stride) {
+    const double* part = partials + (size_t)sys * (part_stride + reduce_groups(part_stride));
+    double t = 0.0;
+    for (int i = threadIdx.x; i < nb; i += 8 * blockDim.x) {
+        double a[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) a[k] = i + k * (int)blockDim.x < nb ? __ldcg(part + i + k * blockDim.x) : 0.0;
+        t += ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
+    }
+    t = block_sum(t);
+    if (threadIdx.x == 0) finalize_scalar(st + sys, t, fin);
+}
+
 // Sum over the grid of v (the kernel's arithmetic type within a warp, FP64 above) for system `sys`.
 // Each block writes its partial; the last block of a group of kReduceGroup blocks to finish (counted
 // atomically) sums the group's, and the last group to finish sums the groups' and finalizes the
@@ -270,15 +312,9 @@ __device__ __forceinline__ double sum_partials(const double* part, int n, int la
 template <class R>
 __device__ __forceinline__ void reduce_and_finalize(R v, double* partials, unsigned* counters, SysState* st,
                                                     int sys, int fin, int part_stride) {
-    __shared__ R sm[32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    v = warp_sum(v);
-    if (lane == 0) sm[wid] = v;
-    __syncthreads();
-    if (wid != 0) return;
-    double bs = lane < nw ? (double)sm[lane] : 0.0;
-    for (int off = 16; off > 0; off >>= 1)
-        if (off < nw) bs += __shfl_down_sync(0xffffffffu, bs, off);
+    const int lane = threadIdx.x & 31;
+    const double bs = block_sum(v);
+    if (threadIdx.x >= 32) return;
     const int nb = gridDim.x, ng = reduce_groups(nb), g = blockIdx.x / kReduceGroup;
     const int in_group = min(kReduceGroup, nb - g * kReduceGroup);
     const int sg = reduce_groups(part_stride);

@@ -99,6 +99,12 @@ cudaError_t launch_hop2(const HopParams<float>& P, int kind, Sp low, Lk lk, int 
 // The hops K1, K2, K3 with two adjacent s per lane (kernels_mixed3.cu): Ns = 8 or 16, FP16 / BF16.
 bool hop3_supported(int ns, Sp low, int kind);
 cudaError_t launch_hop3(const HopParams<float>& P, int kind, Sp low, Lk lk, int nsys, cudaStream_t st);
+int hop3_blocks(size_t n5);  // blocks of its launch on n5 5D sites
+// blocks (per system) that the production hop of this kind launches: the partials its reduction writes
+int hop_blocks(int ns, Sp low, int kind, size_t vh, int nsys);
+// beta, |r|^2 and the status of every system whose status is `need` from the nb partials of K4
+cudaError_t launch_beta(const double* partials, int nb, int part_stride, SysState* st, int need, int sys_base, int nsys,
+                        cudaStream_t stream);
 // the production hop for this configuration and kind (hop3 where supported, else hop2)
 cudaError_t launch_hop_prod(const HopParams<float>& P, int kind, Sp low, Lk lk, int nsys, cudaStream_t st);
 // p = r (mode 0) or p = r + beta p (mode 1), and chi = B p

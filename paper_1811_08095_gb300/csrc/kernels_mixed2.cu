@@ -42,7 +42,12 @@ __global__ void __launch_bounds__(DEEP ? kBS2Deep : kBS2, DEEP ? 4 : 3) hop2_ker
     if (P.gate && P.st[sys].status != P.need_status) return;
     if (P.prof_count && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(P.prof_count, 1ull);
 
-    const size_t gi = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int bx = blockIdx.x;
+    if (KIND == K3 && P.nb_prev > 0 && bx-- == 0) {
+        finalize_partials(P.partials, P.nb_prev, P.st, sys, FIN_ALPHA, P.part_stride);
+        return;
+    }
+    const size_t gi = (size_t)bx * blockDim.x + threadIdx.x;
     const int lane = (int)(gi & (NS - 1));  // lane of the site's group; it holds s = s_of_lane(lane)
     const int s = s_of_lane(lane, NS);
     const size_t hh = gi / NS;
@@ -181,8 +186,7 @@ __global__ void __launch_bounds__(DEEP ? kBS2Deep : kBS2, DEEP ? 4 : 3) hop2_ker
             f32_store_cs<NS>(P.cg_x.d(sys), (size_t)h, s, xv);
         }
     }
-    if (KIND == K2) reduce_and_finalize(nrm, P.partials, P.counters, P.st, sys, FIN_ALPHA, P.part_stride);
-    if (KIND == K4) reduce_and_finalize(nrm, P.partials, P.counters, P.st, sys, FIN_BETA, P.part_stride);
+    if (KIND == K2 || KIND == K4) write_partial(nrm, P.partials, sys, P.part_stride);
 }
 
 // p = r + beta p (mode 1) or p = r (mode 0);  chi = B p.  One thread per (site, s), lane groups of NS.
@@ -225,7 +229,7 @@ cudaError_t hop2_kd(const HopParams<float>& P, int kind, int nsys, cudaStream_t 
     // the others run as hop3 kernels
     constexpr bool all = DEEP || std::is_same<SP, SpF32>::value;
     const size_t n = (size_t)P.g.Vh * NS;
-    dim3 grid(blocks_for(n, BS), nsys);
+    dim3 grid(blocks_for(n, BS) + (kind == K3 && P.nb_prev > 0 ? 1 : 0), nsys);
     if (kind == K4) {
         note_launch();
         hop2_kernel<SP, LK, NS, K4, DEEP><<<grid, BS, 0, st>>>(P);
@@ -289,6 +293,27 @@ cudaError_t pupd_ns(int ns, const FieldRef& r, const FieldRef& p, const FieldRef
 }
 
 }  // namespace
+
+// alpha or beta of each running system from the nb partials of its last reducing hop
+__global__ void __launch_bounds__(512) scalar_kernel(const double* partials, int nb, int part_stride, SysState* st,
+                                                     int need, int sys_base, int fin) {
+    const int sys = blockIdx.x + sys_base;
+    if (st[sys].status != need) return;
+    finalize_partials(partials, nb, st, sys, fin, part_stride);
+}
+
+cudaError_t launch_beta(const double* partials, int nb, int part_stride, SysState* st, int need, int sys_base, int nsys,
+                        cudaStream_t stream) {
+    note_launch();
+    scalar_kernel<<<nsys, 512, 0, stream>>>(partials, nb, part_stride, st, need, sys_base, FIN_BETA);
+    return cudaGetLastError();
+}
+
+int hop_blocks(int ns, Sp low, int kind, size_t vh, int nsys) {
+    const size_t n = vh * ns;
+    if (hop_deep(low, n * nsys)) return blocks_for(n, kBS2Deep);
+    return hop3_supported(ns, low, kind) ? hop3_blocks(n) : blocks_for(n, kBS2);
+}
 
 bool hop_deep(Sp low, size_t n5) { return low != Sp::F32 && n5 <= 16384; }
 

@@ -215,7 +215,12 @@ __global__ void __launch_bounds__(kBS3, hop3_min_blocks<KIND>()) hop3_kernel(con
     if (P.gate && P.st[sys].status != P.need_status) return;
     if (P.prof_count && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(P.prof_count, 1ull);
 
-    const size_t gi = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int bx = blockIdx.x;
+    if (KIND == K3 && P.nb_prev > 0 && bx-- == 0) {
+        finalize_partials(P.partials, P.nb_prev, P.st, sys, FIN_ALPHA, P.part_stride);
+        return;
+    }
+    const size_t gi = (size_t)bx * blockDim.x + threadIdx.x;
     const int l = (int)(gi & (LPS - 1));
     const int s0 = 2 * l, s1 = s0 + 1;
     const size_t hh = gi / LPS;
@@ -320,7 +325,7 @@ __global__ void __launch_bounds__(kBS3, hop3_min_blocks<KIND>()) hop3_kernel(con
             pairs_to_mem(upB, dnB, v);
             SpinorIO<SP, float>::store(P.out.d(sys), P.out.n(sys), (size_t)h, s1, NS, v);
         }
-        reduce_and_finalize(nrm, P.partials, P.counters, P.st, sys, FIN_ALPHA, P.part_stride);
+        write_partial(nrm, P.partials, sys, P.part_stride);
     } else if (KIND == K3) {
         bidiag2<NS>(upA, dnA, upB, dnB, cf.rho[s0], cf.sigma[s0], cf.rho[s1], cf.sigma[s1], r, l, true);
         minv2<NS>(upA, dnA, upB, dnB, cf, r, l, true, -0.5f);
@@ -335,8 +340,7 @@ __global__ void __launch_bounds__(kBS3, hop3_min_blocks<KIND>()) hop3_kernel(con
 
 template <class SP, class LK, int NS>
 cudaError_t hop3_k(const HopParams<float>& P, int kind, int nsys, cudaStream_t st) {
-    const size_t n = (size_t)P.g.Vh * (NS / 2);
-    dim3 grid(blocks_for(n, kBS3), nsys);
+    dim3 grid(hop3_blocks((size_t)P.g.Vh * NS) + (kind == K3 && P.nb_prev > 0 ? 1 : 0), nsys);
     note_launch();
     switch (kind) {
         case K1: hop3_kernel<SP, LK, NS, K1><<<grid, kBS3, 0, st>>>(P); break;
@@ -367,6 +371,8 @@ cudaError_t hop3_lk(const HopParams<float>& P, int kind, Lk lk, int nsys, cudaSt
 }
 
 }  // namespace
+
+int hop3_blocks(size_t n5) { return blocks_for(n5 / 2, kBS3); }
 
 bool hop3_supported(int ns, Sp low, int kind) {
     return (ns == 8 || ns == 16) && (low == Sp::F16 || low == Sp::BF16) && kind != K4;

@@ -133,11 +133,12 @@ namespace {
 
 constexpr int kMaxSlots = 16;
 // Requests join, are cancelled and are handed back between two chunks of iterations, so a chunk is kept
-// near 0.6 ms of GPU time: about 2^21 updates of a 5D site (0.29 ns each at FP16), 1 to 8 iterations.
-// (With 8 iterations whatever the lattice, a request waited up to 20 ms to join a 32^4x16 batch.)
+// near half a millisecond of GPU time: about 1.5 M updates of a 5D site (0.3 ns each at FP16), 2 to 8
+// iterations.  (With 8 iterations whatever the lattice, a request waited up to 20 ms to join a 32^4x16
+// batch.)
 int chunk_iterations(size_t sites5, int running) {
-    const size_t k = ((size_t)1 << 21) / std::max<size_t>(1, sites5 * (size_t)std::max(1, running));
-    return (int)std::min<size_t>(8, std::max<size_t>(1, k));
+    const size_t k = ((size_t)3 << 19) / std::max<size_t>(1, sites5 * (size_t)std::max(1, running));
+    return (int)std::min<size_t>(8, std::max<size_t>(2, k));
 }
 
 // Host-side failure injection for tests: with ODWF_SERVE_INJECT_ERROR=n in the environment the
