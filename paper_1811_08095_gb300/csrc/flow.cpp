@@ -224,7 +224,8 @@ int odwf_flow_set_gauge(odwf_flow* f, const void* U, void* stream) {
         if (rc) return rc;
     }
     double2* stage = dev ? nullptr : f->stage;
-    for (int mu = 0; mu < 4 && !rc; ++mu) {
+    const int nmu = dev ? 4 : 1;  // directions per launch: host data is staged one direction at a time
+    for (int mu = 0; mu < 4 && !rc; mu += nmu) {
         const double2* src = (const double2*)U + (size_t)mu * 9 * V;
         if (!dev) {
             cudaError_t e = cudaMemcpyAsync(stage, src, slab, cudaMemcpyHostToDevice, st);
@@ -232,7 +233,7 @@ int odwf_flow_set_gauge(odwf_flow* f, const void* U, void* stream) {
             src = stage;
         }
         if (!rc) {
-            cudaError_t e = odwf::flow::launch_split(src, f->hi[f->cur], f->lo[f->cur], V, mu, st);
+            cudaError_t e = odwf::flow::launch_split(src, f->hi[f->cur], f->lo[f->cur], V, mu, nmu, st);
             odwf::note_launch();
             if (e != cudaSuccess) rc = cuda_fail(e, "flow split kernel");
         }
@@ -263,9 +264,10 @@ int odwf_flow_get_gauge(odwf_flow* f, void* U, void* stream) {
         if (rc) return rc;
     }
     double2* stage = dev ? nullptr : f->stage;
-    for (int mu = 0; mu < 4 && !rc; ++mu) {
+    const int nmu = dev ? 4 : 1;
+    for (int mu = 0; mu < 4 && !rc; mu += nmu) {
         double2* dst = dev ? (double2*)U + (size_t)mu * 9 * V : stage;
-        cudaError_t e = odwf::flow::launch_join(f->hi[f->cur], f->lo[f->cur], dst, V, mu, st);
+        cudaError_t e = odwf::flow::launch_join(f->hi[f->cur], f->lo[f->cur], dst, V, mu, nmu, st);
         odwf::note_launch();
         if (e != cudaSuccess) rc = cuda_fail(e, "flow join kernel");
         if (!rc && !dev) {

@@ -33,8 +33,8 @@ cudaError_t launch_clover(const FlowGeom& g, const float4* hi, const float4* A, 
                           float* e_site, float* q_site, cudaStream_t st);
 cudaError_t launch_reduce(const FlowGeom& g, const double* part_retr, const float* part_min, const double* part_e,
                           const double* part_q, double t, FlowObsDev* out, cudaStream_t st);
-cudaError_t launch_split(const double2* U, float4* hi, float4* lo, size_t V, int mu, cudaStream_t st);
-cudaError_t launch_join(const float4* hi, const float4* lo, double2* U, size_t V, int mu, cudaStream_t st);
+cudaError_t launch_split(const double2* U, float4* hi, float4* lo, size_t V, int mu0, int nmu, cudaStream_t st);
+cudaError_t launch_join(const float4* hi, const float4* lo, double2* U, size_t V, int mu0, int nmu, cudaStream_t st);
 
 }  // namespace flow
 }  // namespace odwf

@@ -35,6 +35,7 @@
 #include <cstdint>
 
 #include "flow.h"
+#include "fx.cuh"
 
 namespace odwf {
 namespace flow {
@@ -640,45 +641,135 @@ __global__ void __launch_bounds__(kRed) reduce_kernel(int nb_plaq, int nb_clover
     }
 }
 
+// u = h + l, h = u rounded to FP32 and l = u - h rounded, in integers: the FP64 pipe runs the two
+// conversions and the subtraction at 2 per clock and SM, which bound split_kernel.  Zeros and values
+// outside [2^-60, 2^60) (non-finite ones among them) take the FP64 operations.
+__device__ __forceinline__ void split_double(double u, float& h, float& l) {
+    const int hw = __double2hiint(u), e = (hw >> 20) & 0x7ff;
+    const unsigned lw = (unsigned)__double2loint(u);
+    if ((unsigned)(e - (1023 - 60)) >= 120u) {
+        h = (float)u;
+        l = (float)(u - (double)h);
+        return;
+    }
+    const unsigned m_hi = (unsigned)(hw & 0xfffff) | 0x100000u;  // significand: m_hi 2^32 + lw, 53 bits
+    unsigned top = (m_hi << 3) | (lw >> 29);                      // its upper 24 bits
+    int rem = (int)(lw & 0x1fffffffu);
+    if (rem > 0x10000000 || (rem == 0x10000000 && (top & 1u))) {  // round to nearest, ties to even
+        top += 1;
+        rem -= 0x20000000;
+    }
+    const unsigned sign = (unsigned)hw & 0x80000000u;
+    h = __uint_as_float(sign | (((unsigned)(e - 1023 + 126) << 23) + top));  // top's leading bit adds the exponent's one
+    const float r = (float)rem * __uint_as_float((unsigned)(e - 1075 + 127) << 23);
+    l = sign ? -r : r;
+}
+
 // external complex128 U[mu][site][a][b] <-> float-float pairs of the first two rows [mu][j][site]
-// (float4 j holds entries 2j and 2j+1); the third row is rebuilt from the first two in FP64
-__global__ void split_kernel(const double2* __restrict__ U, float4* __restrict__ hi, float4* __restrict__ lo, size_t V,
-                             int mu) {
+// (float4 j holds entries 2j and 2j+1); the third row is rebuilt from the first two.  blockIdx.y: mu - mu0.
+__global__ void __launch_bounds__(256) split_kernel(const double2* __restrict__ U, float4* __restrict__ hi,
+                                                    float4* __restrict__ lo, size_t V, int mu0) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 3 * V) return;
     const size_t s = i / 3;
     const int j = (int)(i - s * 3);
-    const double2 u0 = U[s * 9 + 2 * j], u1 = U[s * 9 + 2 * j + 1];
-    const float4 h = make_float4((float)u0.x, (float)u0.y, (float)u1.x, (float)u1.y);
-    const size_t o = ((size_t)mu * 3 + j) * V + s;
+    const double2* p = U + ((size_t)blockIdx.y * V + s) * 9 + 2 * j;
+    const double2 u0 = p[0], u1 = p[1];
+    float4 h, l;
+    split_double(u0.x, h.x, l.x);
+    split_double(u0.y, h.y, l.y);
+    split_double(u1.x, h.z, l.z);
+    split_double(u1.y, h.w, l.w);
+    const size_t o = ((size_t)(mu0 + blockIdx.y) * 3 + j) * V + s;
     hi[o] = h;
-    lo[o] = make_float4((float)(u0.x - (double)h.x), (float)(u0.y - (double)h.y), (float)(u1.x - (double)h.z),
-                        (float)(u1.y - (double)h.w));
+    lo[o] = l;
 }
 
-__global__ void join_kernel(const float4* __restrict__ hi, const float4* __restrict__ lo, double2* __restrict__ U, size_t V,
-                            int mu) {
-    const size_t s = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= V) return;
-    double2 m[9];
+// 60 fraction bits of x, |x| < 2
+__device__ __forceinline__ long long fixed60(float x) {
+    const unsigned b = __float_as_uint(x);
+    const int e = (int)((b >> 23) & 0xff) - 90;  // left shift of the 24-bit significand
+    const long long m = e > -90 ? (long long)((b & 0x7fffffu) | 0x800000u) : 0;
+    const long long q = e >= 0 ? m << e : m >> min(-e, 63);
+    return (int)b < 0 ? -q : q;
+}
+
+// The sums h + l and the third row conj(row0 x row1) in fixed point (60 fraction bits; 72 FP64
+// operations per link bound the FP64 form at 91 us per direction of 24^3x48), converted once per
+// entry.  A link with an entry of 1.5 or more, or a non-finite one, takes the FP64 form.  The block's
+// links go out through shared memory, so that stores are contiguous.
+constexpr int kJoin = 128;
+__global__ void __launch_bounds__(kJoin) join_kernel(const float4* __restrict__ hi, const float4* __restrict__ lo,
+                                                     double2* __restrict__ U, size_t V, int mu0) {
+    __shared__ double2 sm[kJoin * 9];
+    const size_t s0 = (size_t)blockIdx.x * kJoin, s = s0 + threadIdx.x;
+    if (s < V) {
+        float h[12], l[12], big = 0.f;
+        bool nan = false;
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        const size_t o = ((size_t)mu * 3 + j) * V + s;
-        const float4 h = hi[o], l = lo[o];
-        m[2 * j] = make_double2((double)h.x + (double)l.x, (double)h.y + (double)l.y);
-        m[2 * j + 1] = make_double2((double)h.z + (double)l.z, (double)h.w + (double)l.w);
+        for (int j = 0; j < 3; ++j) {
+            const size_t o = ((size_t)(mu0 + blockIdx.y) * 3 + j) * V + s;
+            const float4 a = hi[o], b = lo[o];
+            h[4 * j] = a.x; h[4 * j + 1] = a.y; h[4 * j + 2] = a.z; h[4 * j + 3] = a.w;
+            l[4 * j] = b.x; l[4 * j + 1] = b.y; l[4 * j + 2] = b.z; l[4 * j + 3] = b.w;
+        }
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            big = fmaxf(big, fmaxf(fabsf(h[k]), fabsf(l[k])));
+            nan = nan || h[k] != h[k] || l[k] != l[k];
+        }
+        double2 m[9];
+        if (big < 1.5f && !nan) {
+            long long q[12];
+            FxLimbs x[12];
+#pragma unroll
+            for (int k = 0; k < 12; ++k) {
+                q[k] = fixed60(h[k]) + fixed60(l[k]);
+                x[k] = fx_split(q[k]);
+            }
+#pragma unroll
+            for (int k = 0; k < 6; ++k) m[k] = make_double2(fx_to_double(q[2 * k], -60), fx_to_double(q[2 * k + 1], -60));
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                // conj(a1 b2 - a2 b1), a = row 0, b = row 1: leading and cross sums of the 31-bit limbs
+                const int a1 = 2 * ((k + 1) % 3), a2 = 2 * ((k + 2) % 3), b1 = 6 + a1, b2 = 6 + a2;
+                long long A[2] = {0, 0}, B[2] = {1ll << 28, 1ll << 28};
+                auto mac = [&](int c, const FxLimbs& u, const FxLimbs& v, bool minus) {
+                    const int n1 = minus ? fx_neg(u.hi) : u.hi, n0 = minus ? fx_neg(u.lo) : u.lo;
+                    A[c] = fx_mad(n1, v.hi, A[c]);
+                    B[c] = fx_mad(n1, v.lo, fx_mad(n0, v.hi, B[c]));
+                };
+                mac(0, x[a1], x[b2], false);
+                mac(0, x[a1 + 1], x[b2 + 1], true);
+                mac(0, x[a2], x[b1], true);
+                mac(0, x[a2 + 1], x[b1 + 1], false);
+                mac(1, x[a1], x[b2 + 1], true);
+                mac(1, x[a1 + 1], x[b2], true);
+                mac(1, x[a2], x[b1 + 1], false);
+                mac(1, x[a2 + 1], x[b1], false);
+                m[6 + k] = make_double2(fx_to_double((A[0] << 2) + (B[0] >> 29), -60),
+                                        fx_to_double((A[1] << 2) + (B[1] >> 29), -60));
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 6; ++k)
+                m[k] = make_double2((double)h[2 * k] + (double)l[2 * k], (double)h[2 * k + 1] + (double)l[2 * k + 1]);
+            const double2 *a = m, *b = m + 3;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const int k1 = (k + 1) % 3, k2 = (k + 2) % 3;
+                const double re = (a[k1].x * b[k2].x - a[k1].y * b[k2].y) - (a[k2].x * b[k1].x - a[k2].y * b[k1].y);
+                const double im = (a[k1].x * b[k2].y + a[k1].y * b[k2].x) - (a[k2].x * b[k1].y + a[k2].y * b[k1].x);
+                m[6 + k] = make_double2(re, -im);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 9; ++k) sm[threadIdx.x * 9 + k] = m[k];
     }
-    // row 2 = conj(row0 x row1)
-    const double2 *a = m, *b = m + 3;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const int k1 = (k + 1) % 3, k2 = (k + 2) % 3;
-        const double re = (a[k1].x * b[k2].x - a[k1].y * b[k2].y) - (a[k2].x * b[k1].x - a[k2].y * b[k1].y);
-        const double im = (a[k1].x * b[k2].y + a[k1].y * b[k2].x) - (a[k2].x * b[k1].y + a[k2].y * b[k1].x);
-        m[6 + k] = make_double2(re, -im);
-    }
-#pragma unroll
-    for (int k = 0; k < 9; ++k) U[s * 9 + k] = m[k];
+    __syncthreads();
+    const int n = 9 * (int)(V - s0 < (size_t)kJoin ? V - s0 : (size_t)kJoin);
+    double2* out = U + ((size_t)blockIdx.y * V + s0) * 9;
+    for (int i = threadIdx.x; i < n; i += kJoin) out[i] = sm[i];
 }
 
 }  // namespace
@@ -722,15 +813,13 @@ cudaError_t launch_reduce(const FlowGeom& g, const double* part_retr, const floa
     return cudaGetLastError();
 }
 
-cudaError_t launch_split(const double2* U, float4* hi, float4* lo, size_t V, int mu, cudaStream_t st) {
-    const size_t n = 3 * V;
-    split_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(U, hi, lo, V, mu);
+cudaError_t launch_split(const double2* U, float4* hi, float4* lo, size_t V, int mu0, int nmu, cudaStream_t st) {
+    split_kernel<<<dim3((unsigned)((3 * V + 255) / 256), nmu), 256, 0, st>>>(U, hi, lo, V, mu0);
     return cudaGetLastError();
 }
 
-cudaError_t launch_join(const float4* hi, const float4* lo, double2* U, size_t V, int mu, cudaStream_t st) {
-    const size_t n = V;
-    join_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(hi, lo, U, V, mu);
+cudaError_t launch_join(const float4* hi, const float4* lo, double2* U, size_t V, int mu0, int nmu, cudaStream_t st) {
+    join_kernel<<<dim3((unsigned)((V + kJoin - 1) / kJoin), nmu), kJoin, 0, st>>>(hi, lo, U, V, mu0);
     return cudaGetLastError();
 }
 
