@@ -13,20 +13,30 @@ Lk link_format(const odwf_solve_params& prm) {
     return prm.link_recon == 18 ? Lk::F18 : Lk::F12;
 }
 
-void BatchCG::drop_graphs() {
+void CgHost::drop_graphs() {
     for (auto& kv : graphs)
         if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
     graphs.clear();
 }
 
-BatchCG::~BatchCG() {
+CgHost::~CgHost() {
     drop_graphs();
-    if (s_rel) cudaStreamSynchronize(s_rel);
-    for (cudaEvent_t e : ev_rel)
+    for (cudaEvent_t e : ev_rel) cudaEventDestroy(e);
+    for (cudaStream_t q : {s_rel, s_solve})
+        if (q) {
+            cudaStreamSynchronize(q);
+            cudaStreamDestroy(q);
+        }
+    for (cudaEvent_t e : {ev_sync, ev_solve})
         if (e) cudaEventDestroy(e);
-    if (s_rel) cudaStreamDestroy(s_rel);
-    if (ev_sync) cudaEventDestroy(ev_sync);
-    if (st_host) cudaFreeHost(st_host);
+    if (pinned) cudaFreeHost(pinned);
+}
+
+BatchCG::~BatchCG() {
+    if (!H) return;
+    if (!idle) cudaDeviceSynchronize();  // an error left copies to the pinned memory in flight
+    else if (s_rel) cudaStreamSynchronize(s_rel);
+    H->busy = false;
 }
 
 template <>
@@ -94,12 +104,27 @@ int BatchCG::init(Engine* e, int capacity, const odwf_solve_params& prm, cudaStr
     counters = (unsigned*)E->get_ws("cg.counters", cbytes, &rc);
     if (rc) return rc;
     ODWF_CK(cudaMemsetAsync(counters, 0, cbytes, s));
-    // pinned: state mirror [cap], initial-state staging [cap], r staging [cap]
-    if (cudaMallocHost(&st_host, 2 * sizeof(SysState) * cap + sizeof(double) * cap) != cudaSuccess) {
-        cudaGetLastError();
-        st_host = nullptr;
-        return fail(ODWF_ENOMEM, "pinned host allocation failed");
+    if (!E->cg_host.busy) {
+        H = &E->cg_host;
+    } else {
+        own = std::make_unique<CgHost>();
+        H = own.get();
     }
+    H->busy = true;
+    // pinned: state mirror [cap], initial-state staging [cap], r staging [cap]
+    const size_t pb = 2 * sizeof(SysState) * cap + sizeof(double) * cap;
+    if (H->pinned_bytes < pb) {
+        if (H->pinned) cudaFreeHost(H->pinned);
+        H->pinned = nullptr;
+        H->pinned_bytes = 0;
+        if (cudaMallocHost(&H->pinned, pb) != cudaSuccess) {
+            cudaGetLastError();
+            H->pinned = nullptr;
+            return fail(ODWF_ENOMEM, "pinned host allocation failed");
+        }
+        H->pinned_bytes = pb;
+    }
+    st_host = (SysState*)H->pinned;
     std::memset(st_host, 0, sizeof(SysState) * cap);
     for (int i = 0; i < cap; ++i) st_host[i].status = kIdle;
     ODWF_CK(cudaMemcpyAsync(st, st_host, sizeof(SysState) * cap, cudaMemcpyHostToDevice, s));
@@ -109,11 +134,31 @@ int BatchCG::init(Engine* e, int capacity, const odwf_solve_params& prm, cudaStr
     int prio = 0, least = 0, greatest = 0;
     ODWF_CK(cudaStreamGetPriority(s, &prio));
     ODWF_CK(cudaDeviceGetStreamPriorityRange(&least, &greatest));
-    ODWF_CK(cudaStreamCreateWithPriority(&s_rel, cudaStreamNonBlocking, std::min(least, prio + update_prio_drop)));
-    ODWF_CK(cudaEventCreateWithFlags(&ev_sync, cudaEventDisableTiming));
+    const int rel_prio = std::min(least, prio + update_prio_drop);
+    if (H->s_rel && H->s_rel_prio != rel_prio) {
+        ODWF_CK(cudaStreamDestroy(H->s_rel));
+        H->s_rel = nullptr;
+    }
+    if (!H->s_rel) ODWF_CK(cudaStreamCreateWithPriority(&H->s_rel, cudaStreamNonBlocking, rel_prio));
+    H->s_rel_prio = rel_prio;
+    s_rel = H->s_rel;
+    if (!H->ev_sync) ODWF_CK(cudaEventCreateWithFlags(&H->ev_sync, cudaEventDisableTiming));
+    ev_sync = H->ev_sync;
+    while ((int)H->ev_rel.size() < cap) {
+        cudaEvent_t e = nullptr;
+        ODWF_CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+        H->ev_rel.push_back(e);
+    }
+    ev_rel.assign(H->ev_rel.begin(), H->ev_rel.begin() + cap);
+    // what the iteration's kernels are launched with, besides the slot range and the iteration count
+    const void* bufs[] = {X64.data, R64.data, P64.data, A64.data, C64.data, Rin.data, Xin.data, Pl.data, Tl.data,
+                          Al.data, Cl.data, Chil.data, A64.norm, C64.norm, Pl.norm, Tl.norm, Al.norm, Cl.norm,
+                          Chil.norm, st, r_dev, partials, counters, E->links_fx, E->nbr,
+                          mixed ? E->links_of(lk) : nullptr, v2 ? E->links_site[(int)lk] : nullptr};
+    const int fmt[] = {(int)low, (int)lk, mixed, v2, cap, nblk};
+    graph_key.assign((const char*)bufs, sizeof(bufs));
+    graph_key.append((const char*)fmt, sizeof(fmt));
     bsrc.assign(cap, nullptr);
-    ev_rel.assign(cap, nullptr);
-    for (int i = 0; i < cap; ++i) ODWF_CK(cudaEventCreateWithFlags(&ev_rel[i], cudaEventDisableTiming));
     active.assign(cap, 0);
     mq.assign(cap, 0.0);
     slot_tol.assign(cap, tol);
@@ -154,6 +199,7 @@ int BatchCG::init(Engine* e, int capacity, const odwf_solve_params& prm, cudaStr
 int BatchCG::admit(int slot, const double2* b_ext, double mq_slot, cudaStream_t s, double tol_slot,
                    int max_iter_slot) {
     NvtxRange nv_("odwf.cg.admit");
+    idle = false;
     if (slot < 0 || slot >= cap) return fail(ODWF_EINVAL, "admit: bad slot");
     mq[slot] = mq_slot;
     const size_t eb = E->sites5() * 12 * sizeof(double2);
@@ -209,6 +255,7 @@ int BatchCG::cancel(int slot, cudaStream_t s) {
 }
 
 int BatchCG::admit_internal(int slot, cudaStream_t s, double tol_slot, int max_iter_slot) {
+    idle = false;
     const double tl = tol_slot > 0 ? tol_slot : tol;
     slot_tol[slot] = tl;
     const size_t n5 = E->sites5();
@@ -252,6 +299,7 @@ int BatchCG::admit_internal(int slot, cudaStream_t s, double tol_slot, int max_i
 
 int BatchCG::run_iterations(int k, cudaStream_t s) {
     NvtxRange nv_("odwf.cg.iterations");
+    idle = false;
     int lo = cap, hi = -1;
     for (int i = 0; i < cap; ++i)
         if (active[i] && slot_running(i)) {
@@ -268,16 +316,17 @@ int BatchCG::run_iterations(int k, cudaStream_t s) {
     }();
     if (!graphs_on || prof_enabled() || s == nullptr || s == cudaStreamLegacy || s == cudaStreamPerThread)
         return launch_iterations(k, lo, n, s);
-    const unsigned long long key = ((unsigned long long)lo << 40) | ((unsigned long long)n << 20) | (unsigned)k;
-    auto it = graphs.find(key);
-    if (it == graphs.end()) {
-        if (graphs.size() >= 32) drop_graphs();
+    const int range[3] = {lo, n, k};
+    const std::string key = graph_key + std::string((const char*)range, sizeof(range));
+    auto it = H->graphs.find(key);
+    if (it == H->graphs.end()) {
+        if (H->graphs.size() >= 32) H->drop_graphs();
         const long long c0 = launch_count();
         ODWF_CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
         const int rc = launch_iterations(k, lo, n, s);
         cudaGraph_t g = nullptr;
         const cudaError_t ce = cudaStreamEndCapture(s, &g);
-        GraphEntry e;
+        CgHost::Graph e;
         e.kernels = launch_count() - c0;
         note_launches(-e.kernels);  // captured, not launched
         if (rc || ce != cudaSuccess) {
@@ -287,7 +336,7 @@ int BatchCG::run_iterations(int k, cudaStream_t s) {
         const cudaError_t ie = cudaGraphInstantiate(&e.exec, g, 0);
         cudaGraphDestroy(g);
         if (ie != cudaSuccess) return cuda_fail(ie, "cudaGraphInstantiate(CG iterations)");
-        it = graphs.emplace(key, e).first;
+        it = H->graphs.emplace(key, e).first;
     }
     ODWF_CK(cudaGraphLaunch(it->second.exec, s));
     note_launches(it->second.kernels);
@@ -587,6 +636,7 @@ int BatchCG::finalize(int slot, double2* x_ext, cudaStream_t s, double* true_res
     if (x_ext) ODWF_CK(launch_unpack(Sp::F64, X64.ref_sys(slot), x_ext, E->g, 0, E->ns, 1, s));
     ODWF_CK(cudaMemcpyAsync(st_host + slot, st + slot, sizeof(SysState), cudaMemcpyDeviceToHost, s));
     ODWF_CK(cudaStreamSynchronize(s));
+    idle = true;
     const SysState& S = st_host[slot];
     if (true_resid) *true_resid = S.bb > 0 ? std::sqrt(S.sum / S.bb) : 0.0;
     return ODWF_OK;

@@ -26,6 +26,7 @@
 
 #include <chrono>
 #include <map>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -75,11 +76,11 @@ struct BatchCG {
     std::vector<double> slot_tol;
     // A chunk of k iterations over slots lo..lo+n-1 is captured once into a CUDA graph and
     // replayed (launch-bound small lattices; not while the kernel profiler is enabled).
-    struct GraphEntry {
-        cudaGraphExec_t exec = nullptr;
-        long long kernels = 0;
-    };
-    std::map<unsigned long long, GraphEntry> graphs;
+    // Kept in CgHost under `graph_key`, the buffers and formats of this batch.
+    std::string graph_key;
+    CgHost* H = nullptr;
+    std::unique_ptr<CgHost> own;   // when the engine's is in use
+    bool idle = true;              // nothing of this batch is in flight on the iteration stream
     int pcls[5] = {-1, -1, -1, -1, -1};  // profiler classes: K1..K4, p update
     std::string kname[5];                 // (second-generation kernels) class names and
     double kbytes_sys[5] = {0}, kbytes_launch[5] = {0};  // algorithmic bytes per system / launch
@@ -120,7 +121,6 @@ struct BatchCG {
     HopParams<R> params(int p_out) const;
     int fp64_residual(int slot, cudaStream_t s);
     int launch_iterations(int k, int lo, int n, cudaStream_t s);
-    void drop_graphs();
     FieldRef Rref() const { return mixed ? R64.ref_shared() : R64.ref(); }
     FieldRef Bref() const { return mixed ? B64.ref_shared() : B64.ref(); }
     int load_b(int slot, cudaStream_t s);               // mixed: pack the slot's b into the shared B64

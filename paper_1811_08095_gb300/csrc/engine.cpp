@@ -531,37 +531,24 @@ int check_params(const odwf_solve_params* prm) {
 }
 
 namespace {
-// An internal stream of the highest priority that starts after the work queued on the
-// caller's stream and that the caller's stream waits for at the end.
-struct SolveStream {
-    cudaStream_t s = nullptr;
-    cudaEvent_t ev = nullptr;
-    int open(cudaStream_t user) {
+// The engine's internal stream of the highest priority: starts after the work queued on the caller's
+// stream, which waits for it at the end.
+int open_solve_stream(CgHost& H, cudaStream_t user) {
+    if (!H.s_solve) {
         int least = 0, greatest = 0;
         ODWF_CK(cudaDeviceGetStreamPriorityRange(&least, &greatest));
-        ODWF_CK(cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, greatest));
-        ODWF_CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-        ODWF_CK(cudaEventRecord(ev, user));
-        ODWF_CK(cudaStreamWaitEvent(s, ev, 0));
-        return ODWF_OK;
+        ODWF_CK(cudaStreamCreateWithPriority(&H.s_solve, cudaStreamNonBlocking, greatest));
+        ODWF_CK(cudaEventCreateWithFlags(&H.ev_solve, cudaEventDisableTiming));
     }
-    int close(cudaStream_t user) {
-        int rc = ODWF_OK;
-        if (s && ev) {
-            if (cudaEventRecord(ev, s) != cudaSuccess || cudaStreamWaitEvent(user, ev, 0) != cudaSuccess)
-                rc = fail(ODWF_ECUDA, "solve: joining the caller's stream failed");
-        }
-        if (ev) cudaEventDestroy(ev);
-        if (s) cudaStreamDestroy(s);  // released once its queued work has completed
-        s = nullptr;
-        ev = nullptr;
-        return rc;
-    }
-    ~SolveStream() {
-        if (ev) cudaEventDestroy(ev);
-        if (s) cudaStreamDestroy(s);
-    }
-};
+    ODWF_CK(cudaEventRecord(H.ev_solve, user));
+    ODWF_CK(cudaStreamWaitEvent(H.s_solve, H.ev_solve, 0));
+    return ODWF_OK;
+}
+int close_solve_stream(CgHost& H, cudaStream_t user) {
+    if (cudaEventRecord(H.ev_solve, H.s_solve) != cudaSuccess || cudaStreamWaitEvent(user, H.ev_solve, 0) != cudaSuccess)
+        return fail(ODWF_ECUDA, "solve: joining the caller's stream failed");
+    return ODWF_OK;
+}
 }  // namespace
 
 int Engine::solve(int nsys, void* const* x, const void* const* b, const double* mq_arr,
@@ -579,10 +566,9 @@ int Engine::solve(int nsys, void* const* x, const void* const* b, const double* 
     const auto t0 = std::chrono::steady_clock::now();
     // The solve runs on an internal stream of the highest priority (its reliable updates one
     // level below), joined to the caller's stream at both ends.
-    SolveStream ss;
-    if ((rc = ss.open(st))) return rc;
-    rc = solve_on(nsys, x, b, mq_arr, prm, stats, ss.s);
-    const int rc2 = ss.close(st);
+    if ((rc = open_solve_stream(cg_host, st))) return rc;
+    rc = solve_on(nsys, x, b, mq_arr, prm, stats, cg_host.s_solve);
+    const int rc2 = close_solve_stream(cg_host, st);
     if (stats)
         for (int i = 0; i < nsys; ++i)
             stats[i].time_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();

@@ -35,6 +35,27 @@ struct DevBuf {
     size_t bytes = 0;
 };
 
+// What a batched solve needs on the host side, kept with the engine from one solve to the next (making
+// and freeing it cost a solve of a small lattice most of a millisecond): pinned memory, streams, events,
+// and the iteration graphs, found again by everything their kernels point to.  One batch uses it at a
+// time; another one alive on the same engine makes its own.
+struct CgHost {
+    struct Graph {
+        cudaGraphExec_t exec = nullptr;
+        long long kernels = 0;
+    };
+    bool busy = false;
+    void* pinned = nullptr;
+    size_t pinned_bytes = 0;
+    cudaStream_t s_rel = nullptr, s_solve = nullptr;
+    int s_rel_prio = 0;
+    cudaEvent_t ev_sync = nullptr, ev_solve = nullptr;
+    std::vector<cudaEvent_t> ev_rel;
+    std::map<std::string, Graph> graphs;  // at most 32
+    void drop_graphs();
+    ~CgHost();
+};
+
 // A half field for `nsys` systems (system slabs `stride` bytes apart) in format `sp`.
 struct HalfField {
     Sp sp = Sp::F64;
@@ -85,6 +106,8 @@ struct Engine {
     const void* links_of(Lk lk) const {
         return lk == Lk::F12 ? links_f12 : lk == Lk::F18 ? links_f18 : lk == Lk::H12 ? links_h12 : links_d18;
     }
+
+    CgHost cg_host;
 
     // named workspaces (grow-only)
     std::map<std::string, DevBuf> ws;
