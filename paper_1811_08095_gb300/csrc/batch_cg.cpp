@@ -380,8 +380,12 @@ int BatchCG::launch_iterations(int k, int lo, int n, cudaStream_t s) {
                 ODWF_CK(e_);
             }
         } else if (v2) {
-            int rc = launch_v2_hops(lo, n, s);
-            if (!rc) rc = launch_v2_pupdate(1, lo, n, 1, kRunning, s);
+            // With few partials the p update forms beta and the next K1 puts it into the state, which saves
+            // a launch; the last iteration of the chunk finalizes before the host looks.
+            const int nb = hop_blocks(E->ns, low, 4, E->vh(), n);
+            const bool in_update = nb * n <= kBetaInUpdate, last = it + 1 == k;
+            int rc = launch_v2_hops(lo, n, s, in_update && it > 0, !in_update || last);
+            if (!rc) rc = launch_v2_pupdate(1, lo, n, 1, kRunning, s, in_update && !last ? nb : 0);
             if (rc) return rc;
         } else {
             auto P = params<float>(1);
@@ -448,7 +452,7 @@ int BatchCG::launch_v2_kernel(int kind, int lo, int n, cudaStream_t s) {
     return ODWF_OK;
 }
 
-int BatchCG::launch_v2_hops(int lo, int n, cudaStream_t s) {
+int BatchCG::launch_v2_hops(int lo, int n, cudaStream_t s, bool prev_beta, bool last_beta) {
     auto P = params<float>(1);
     P.gate = 1;
     P.need_status = kRunning;
@@ -466,7 +470,9 @@ int BatchCG::launch_v2_hops(int lo, int n, cudaStream_t s) {
             P.cg_x = Xin.ref();
             P.cg_p = Pl.ref();
         }
-        P.nb_prev = k == 2 ? hop_blocks(E->ns, low, 2, E->vh(), n) : 0;  // K3 also forms alpha from K2's partials
+        // K3 also forms alpha from K2's partials, K1 beta from the last K4's
+        P.nb_prev = k == 2 ? hop_blocks(E->ns, low, 2, E->vh(), n)
+                  : k == 0 && prev_beta ? hop_blocks(E->ns, low, 4, E->vh(), n) : 0;
         auto pb_ = prof_begin(pcls[k], s);
         P.prof_count = pb_.dev_count;
         const cudaError_t e_ = launch_hop_prod(P, k + 1, low, lk, n, s);
@@ -474,15 +480,15 @@ int BatchCG::launch_v2_hops(int lo, int n, cudaStream_t s) {
         P.prof_count = nullptr;
         ODWF_CK(e_);
     }
-    ODWF_CK(launch_beta(partials, hop_blocks(E->ns, low, 4, E->vh(), n), nblk, st, kRunning, lo, n, s));
+    if (last_beta) ODWF_CK(launch_beta(partials, hop_blocks(E->ns, low, 4, E->vh(), n), nblk, st, kRunning, lo, n, s));
     return ODWF_OK;
 }
 
 // p = r + beta p (mode 1) or p = r (mode 0), chi_p = B p, for the slots whose status is `need`.
-int BatchCG::launch_v2_pupdate(int mode, int lo, int n, int gate, int need, cudaStream_t s) {
+int BatchCG::launch_v2_pupdate(int mode, int lo, int n, int gate, int need, cudaStream_t s, int nb) {
     auto pb_ = prof_begin(pcls[4], s);
     const cudaError_t e_ = launch_p_update2(low, E->ns, Rin.ref(), Pl.ref(), Chil.ref(), E->vh(), mode, E->cf32, r_dev,
-                                            st, gate, need, lo, n, pb_.dev_count, s);
+                                            st, gate, need, lo, n, pb_.dev_count, s, partials, nb, nblk);
     prof_end(pb_, s);
     ODWF_CK(e_);
     return ODWF_OK;

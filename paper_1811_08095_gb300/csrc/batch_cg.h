@@ -107,8 +107,10 @@ struct BatchCG {
     int service(cudaStream_t s);                   // reliable updates for parked slots
     int finalize(int slot, double2* x_ext, cudaStream_t s, double* true_resid);
     // second-generation mixed iteration pieces (v2 only): K1..K4 hops, and the p update
-    int launch_v2_hops(int lo, int n, cudaStream_t s);
-    int launch_v2_pupdate(int mode, int lo, int n, int gate, int need, cudaStream_t s);
+    // prev_beta: K1 finalizes the previous iteration's beta; last_beta: finalize this one's after K4
+    int launch_v2_hops(int lo, int n, cudaStream_t s, bool prev_beta = false, bool last_beta = true);
+    // nb > 0: the update forms beta from the nb partials of K4
+    int launch_v2_pupdate(int mode, int lo, int n, int gate, int need, cudaStream_t s, int nb = 0);
     int launch_v2_kernel(int kind, int lo, int n, cudaStream_t s);  // kind 1..4: K1..K4 alone, 5: P
     // write a slot's scalars (and r = m_q / (2 m0)) directly; synchronizes s
     int set_state(int slot, const SysState& init, double r, cudaStream_t s);

@@ -91,7 +91,8 @@ struct HopParams {
     double* partials;           // reduce_and_finalize's partials and counters
     int part_stride;            // most blocks of a reducing launch, fixed for every launch of one batch
     unsigned* counters;
-    int nb_prev;                // production K3: block 0 forms alpha from this many partials of K2 (0: no such block)
+    int nb_prev;                // production K1, K3: block 0 finalizes beta, alpha from this many partials of K4, K2
+                                // (0: no such block)
     int sys_base;               // system index offset (blockIdx.y + sys_base)
     unsigned long long* prof_count;  // optional: counts running (system, launch) pairs
     const double* tab5;              // fixed-point hops: fifth-dimension scan tables (Engine::init)
@@ -215,6 +216,13 @@ __device__ __forceinline__ float warp_sum(float v) {
     for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
     return v;
 }
+// whether |r|^2 = rr_new after this iteration's update parks the system: the host then recomputes the
+// true residual (and, in mixed precision, folds the inner solution into the FP64 one)
+__device__ __forceinline__ bool parks(const SysState& st, double rr_new) {
+    return !isfinite(rr_new) || rr_new <= st.stop_in || st.iter + 1 >= st.max_iter ||
+           (st.reliable && rr_new < (st.delta * st.r_max) * (st.delta * st.r_max));
+}
+
 __device__ __forceinline__ void finalize_scalar(SysState* st, double total, int fin) {
     if (fin == FIN_STORE) {
         st->sum = total;
@@ -227,15 +235,11 @@ __device__ __forceinline__ void finalize_scalar(SysState* st, double total, int 
         }
     } else {  // FIN_BETA
         const double rr_new = total;
+        const bool park = parks(*st, rr_new);
         st->rr_new = rr_new;
         st->iter += 1;
-        if (!isfinite(rr_new)) {
-            st->status = kBreakdown;
-        } else if (rr_new <= st->stop_in || st->iter >= st->max_iter ||
-                   (st->reliable && rr_new < (st->delta * st->r_max) * (st->delta * st->r_max))) {
-            // park the system: the host recomputes the true residual in FP64 (and, in mixed
-            // precision, folds the inner solution into the FP64 one) before it continues
-            st->status = kNeedUpdate;
+        if (park) {
+            st->status = isfinite(rr_new) ? kNeedUpdate : kBreakdown;
         } else {
             st->beta = rr_new / st->rr;
             st->rr = rr_new;
@@ -277,25 +281,30 @@ __device__ __forceinline__ double block_sum(R v) {
 // The production mixed hops leave their reduction to a later launch: each block writes its partial and
 // is done, without the fence and the atomic that finding the last block takes (about 6 us at the end of
 // every reducing launch).  alpha, which only K4 needs, is formed by one extra block of K3; beta by
-// beta_kernel before the p update.
+// a one-block kernel before the p update or, with few partials, by every block of the p update.
 template <class R>
 __device__ __forceinline__ void write_partial(R v, double* partials, int sys, int part_stride) {
     const double bs = block_sum(v);
     if (threadIdx.x == 0) partials[(size_t)sys * (part_stride + reduce_groups(part_stride)) + blockIdx.x] = bs;
 }
 
-// One block sums a system's nb partials in a fixed order and finalizes the scalar
-__device__ __forceinline__ void finalize_partials(const double* partials, int nb, SysState* st, int sys, int fin,
-                                                  int part_stride) {
+// Sum of a system's nb partials by one block, valid in thread 0.  Up to kBetaInUpdate partials 64 threads
+// sum, so that the p update and the kernels that finalize the state, whose blocks differ, get the same bits.
+__device__ __forceinline__ double sum_block_partials(const double* partials, int nb, int sys, int part_stride) {
     const double* part = partials + (size_t)sys * (part_stride + reduce_groups(part_stride));
+    const int w = nb <= kBetaInUpdate ? 64 : (int)blockDim.x;
     double t = 0.0;
-    for (int i = threadIdx.x; i < nb; i += 8 * blockDim.x) {
+    for (int i = (int)threadIdx.x < w ? (int)threadIdx.x : nb; i < nb; i += 8 * w) {
         double a[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) a[k] = i + k * (int)blockDim.x < nb ? __ldcg(part + i + k * blockDim.x) : 0.0;
+        for (int k = 0; k < 8; ++k) a[k] = i + k * w < nb ? __ldcg(part + i + k * w) : 0.0;
         t += ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
     }
-    t = block_sum(t);
+    return block_sum(t);
+}
+__device__ __forceinline__ void finalize_partials(const double* partials, int nb, SysState* st, int sys, int fin,
+                                                  int part_stride) {
+    const double t = sum_block_partials(partials, nb, sys, part_stride);
     if (threadIdx.x == 0) finalize_scalar(st + sys, t, fin);
 }
 

@@ -111,7 +111,12 @@ cudaError_t launch_hop_prod(const HopParams<float>& P, int kind, Sp low, Lk lk, 
 cudaError_t launch_p_update2(Sp low, int ns, const FieldRef& r, const FieldRef& p, const FieldRef& chi,
                              size_t n_sites, int mode, const Coef5<float>& cf, const double* r_sys, SysState* st,
                              int gate, int need, int sys_base, int nsys, unsigned long long* prof,
-                             cudaStream_t stream);
+                             cudaStream_t stream, const double* partials = nullptr, int nb = 0, int part_stride = 0);
+// K4 partials of all systems of a launch up to which the p update forms beta itself (launch_p_update2 with
+// nb > 0).  It saves a launch but every block waits for the sum and the division: per iteration 23.4 -> 22.2
+// us on 4^4x8 (16 partials), 38.2 -> 37.2 on 8^3x16x16 (256), but 61.2 -> 63.9 for eight systems on 8^4x8
+// (512) and 118 -> 124 on 12^3x24x16 (1296).
+constexpr int kBetaInUpdate = 256;
 
 // Site-local M, M^dag, M^-1, M^-dag (op 0..3); op 4 = B (the chiral shift rho + sigma L)
 // gate_st (optional): only systems whose status equals `need` are processed

@@ -43,8 +43,8 @@ __global__ void __launch_bounds__(DEEP ? kBS2Deep : kBS2, DEEP ? 4 : 3) hop2_ker
     if (P.prof_count && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(P.prof_count, 1ull);
 
     int bx = blockIdx.x;
-    if (KIND == K3 && P.nb_prev > 0 && bx-- == 0) {
-        finalize_partials(P.partials, P.nb_prev, P.st, sys, FIN_ALPHA, P.part_stride);
+    if ((KIND == K1 || KIND == K3) && P.nb_prev > 0 && bx-- == 0) {
+        finalize_partials(P.partials, P.nb_prev, P.st, sys, KIND == K1 ? FIN_BETA : FIN_ALPHA, P.part_stride);
         return;
     }
     const size_t gi = (size_t)bx * blockDim.x + threadIdx.x;
@@ -190,11 +190,15 @@ __global__ void __launch_bounds__(DEEP ? kBS2Deep : kBS2, DEEP ? 4 : 3) hop2_ker
 }
 
 // p = r + beta p (mode 1) or p = r (mode 0);  chi = B p.  One thread per (site, s), lane groups of NS.
+// nb > 0 (at most kBetaInUpdate): every block forms beta itself from the nb partials of K4 and the state
+// of the iteration's start, which stays as it is (the next K1 finalizes it), and leaves p alone where that
+// will park the system.
 template <class SP, int NS>
 __global__ void __launch_bounds__(kBS2) p_update2_kernel(FieldRef rr, FieldRef pp, FieldRef chi, size_t n_sites,
                                                           int mode, Coef5<float> cf, const double* r_sys,
                                                           SysState* st, int gate, int need, int sys_base,
-                                                          unsigned long long* prof_count) {
+                                                          unsigned long long* prof_count, const double* partials,
+                                                          int nb, int part_stride) {
     const int sys = blockIdx.y + sys_base;
     if (gate && st[sys].status != need) return;
     if (prof_count && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(prof_count, 1ull);
@@ -202,13 +206,24 @@ __global__ void __launch_bounds__(kBS2) p_update2_kernel(FieldRef rr, FieldRef p
     const int s = (int)(gi & (NS - 1));
     const size_t h = gi / NS;
     const bool valid = h < n_sites;
-    float v[24];
+    float v[24], pv[24];
     if (valid) {
         SpinorIO<SpF32, float>::load(rr.d(sys), nullptr, h, s, NS, v);
+        if (mode == 1) SpinorIO<SP, float>::load(pp.d(sys), pp.n(sys), h, s, NS, pv);
+    }
+    float beta = 0.f;
+    if (nb > 0) {
+        __shared__ float s_beta;
+        const double rr_new = sum_block_partials(partials, nb, sys, part_stride);
+        if (threadIdx.x == 0) s_beta = parks(st[sys], rr_new) ? -1.f : (float)(rr_new / st[sys].rr);
+        __syncthreads();
+        beta = s_beta;
+        if (beta < 0.f) return;  // uniform over the block; a beta that goes on is not negative
+    } else if (mode == 1) {
+        beta = (float)st[sys].beta;
+    }
+    if (valid) {
         if (mode == 1) {
-            const float beta = (float)st[sys].beta;
-            float pv[24];
-            SpinorIO<SP, float>::load(pp.d(sys), pp.n(sys), h, s, NS, pv);
 #pragma unroll
             for (int k = 0; k < 24; ++k) v[k] = fmaf(beta, pv[k], v[k]);
         }
@@ -229,7 +244,7 @@ cudaError_t hop2_kd(const HopParams<float>& P, int kind, int nsys, cudaStream_t 
     // the others run as hop3 kernels
     constexpr bool all = DEEP || std::is_same<SP, SpF32>::value;
     const size_t n = (size_t)P.g.Vh * NS;
-    dim3 grid(blocks_for(n, BS) + (kind == K3 && P.nb_prev > 0 ? 1 : 0), nsys);
+    dim3 grid(blocks_for(n, BS) + ((kind == K1 || kind == K3) && P.nb_prev > 0 ? 1 : 0), nsys);
     if (kind == K4) {
         note_launch();
         hop2_kernel<SP, LK, NS, K4, DEEP><<<grid, BS, 0, st>>>(P);
@@ -273,21 +288,23 @@ cudaError_t hop2_lk(const HopParams<float>& P, int kind, Lk lk, int nsys, cudaSt
 template <class SP, int NS>
 cudaError_t pupd_k(const FieldRef& r, const FieldRef& p, const FieldRef& chi, size_t n_sites, int mode,
                    const Coef5<float>& cf, const double* r_sys, SysState* st, int gate, int need, int sys_base,
-                   int nsys, unsigned long long* prof, cudaStream_t stream) {
+                   int nsys, unsigned long long* prof, cudaStream_t stream,
+                    const double* partials, int nb, int part_stride) {
     dim3 grid(blocks_for(n_sites * NS, kBS2), nsys);
     note_launch();
     p_update2_kernel<SP, NS><<<grid, kBS2, 0, stream>>>(r, p, chi, n_sites, mode, cf, r_sys, st, gate, need,
-                                                         sys_base, prof);
+                                                         sys_base, prof, partials, nb, part_stride);
     return cudaGetLastError();
 }
 
 template <class SP>
 cudaError_t pupd_ns(int ns, const FieldRef& r, const FieldRef& p, const FieldRef& chi, size_t n_sites, int mode,
                     const Coef5<float>& cf, const double* r_sys, SysState* st, int gate, int need, int sys_base,
-                    int nsys, unsigned long long* prof, cudaStream_t stream) {
+                    int nsys, unsigned long long* prof, cudaStream_t stream,
+                    const double* partials, int nb, int part_stride) {
     switch (ns) {
-        case 8: return pupd_k<SP, 8>(r, p, chi, n_sites, mode, cf, r_sys, st, gate, need, sys_base, nsys, prof, stream);
-        case 16: return pupd_k<SP, 16>(r, p, chi, n_sites, mode, cf, r_sys, st, gate, need, sys_base, nsys, prof, stream);
+        case 8: return pupd_k<SP, 8>(r, p, chi, n_sites, mode, cf, r_sys, st, gate, need, sys_base, nsys, prof, stream, partials, nb, part_stride);
+        case 16: return pupd_k<SP, 16>(r, p, chi, n_sites, mode, cf, r_sys, st, gate, need, sys_base, nsys, prof, stream, partials, nb, part_stride);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -335,11 +352,11 @@ cudaError_t launch_hop2(const HopParams<float>& P, int kind, Sp low, Lk lk, int 
 cudaError_t launch_p_update2(Sp low, int ns, const FieldRef& r, const FieldRef& p, const FieldRef& chi,
                              size_t n_sites, int mode, const Coef5<float>& cf, const double* r_sys, SysState* st,
                              int gate, int need, int sys_base, int nsys, unsigned long long* prof,
-                             cudaStream_t stream) {
+                             cudaStream_t stream, const double* partials, int nb, int part_stride) {
     switch (low) {
-        case Sp::F16: return pupd_ns<SpF16>(ns, r, p, chi, n_sites, mode, cf, r_sys, st, gate, need, sys_base, nsys, prof, stream);
-        case Sp::BF16: return pupd_ns<SpBF16>(ns, r, p, chi, n_sites, mode, cf, r_sys, st, gate, need, sys_base, nsys, prof, stream);
-        case Sp::F32: return pupd_ns<SpF32>(ns, r, p, chi, n_sites, mode, cf, r_sys, st, gate, need, sys_base, nsys, prof, stream);
+        case Sp::F16: return pupd_ns<SpF16>(ns, r, p, chi, n_sites, mode, cf, r_sys, st, gate, need, sys_base, nsys, prof, stream, partials, nb, part_stride);
+        case Sp::BF16: return pupd_ns<SpBF16>(ns, r, p, chi, n_sites, mode, cf, r_sys, st, gate, need, sys_base, nsys, prof, stream, partials, nb, part_stride);
+        case Sp::F32: return pupd_ns<SpF32>(ns, r, p, chi, n_sites, mode, cf, r_sys, st, gate, need, sys_base, nsys, prof, stream, partials, nb, part_stride);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -216,8 +216,8 @@ __global__ void __launch_bounds__(kBS3, hop3_min_blocks<KIND>()) hop3_kernel(con
     if (P.prof_count && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(P.prof_count, 1ull);
 
     int bx = blockIdx.x;
-    if (KIND == K3 && P.nb_prev > 0 && bx-- == 0) {
-        finalize_partials(P.partials, P.nb_prev, P.st, sys, FIN_ALPHA, P.part_stride);
+    if ((KIND == K1 || KIND == K3) && P.nb_prev > 0 && bx-- == 0) {
+        finalize_partials(P.partials, P.nb_prev, P.st, sys, KIND == K1 ? FIN_BETA : FIN_ALPHA, P.part_stride);
         return;
     }
     const size_t gi = (size_t)bx * blockDim.x + threadIdx.x;
@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(kBS3, hop3_min_blocks<KIND>()) hop3_kernel(con
 
 template <class SP, class LK, int NS>
 cudaError_t hop3_k(const HopParams<float>& P, int kind, int nsys, cudaStream_t st) {
-    dim3 grid(hop3_blocks((size_t)P.g.Vh * NS) + (kind == K3 && P.nb_prev > 0 ? 1 : 0), nsys);
+    dim3 grid(hop3_blocks((size_t)P.g.Vh * NS) + ((kind == K1 || kind == K3) && P.nb_prev > 0 ? 1 : 0), nsys);
     note_launch();
     switch (kind) {
         case K1: hop3_kernel<SP, LK, NS, K1><<<grid, kBS3, 0, st>>>(P); break;
