@@ -11,61 +11,60 @@
 // by the site-local and hopping operators (see pf_force.cpp); the contraction kernel takes L and
 // R as parity-split FP64 half fields and accumulates coef * G per link.
 //
-// One thread per link; the loop over s reads, per s, the four spinors L(x), R(x+mu), R(x),
-// L(x+mu) once, projects the L's with (1 -+ gamma_mu) and accumulates the two 3x3 outer products.
-// The algorithmic bytes per link are 4 * Ns * 192 (the four spinors) + 144 (the link) + 2 * 144
-// (G in and out): the kernel is bound by the FP64 pipe on this part (about 2 Ns * 180 FMAs).
+// (1 -+ gamma_mu) has rank two: with h the upper half of (1 + sg gamma) L and G its off-diagonal block,
+// the lower half is sg G^+ h, so that sum_spin R conj((1 + sg gamma) L) is the outer product of the
+// projected R with the projected L: 2 x (24 + 72) FP64 operations per s and link instead of 2 x (36 + 144).
+// Bound by the FP64 pipe.  A warp has one mu, so that the projections do not diverge, and eight
+// sites; four lanes share a link's s, read 64 contiguous bytes of each component and add their parts
+// at the end, which also gives four times the warps (8^3 x 16 with Ns = 16: 678 -> 285 us).  The algorithmic bytes per link are
+// 4 * Ns * 192 (the four spinors) + 144 (the link) + 2 * 144 (G in and out).
 #include "kernels.cuh"
 #include "kernels.h"
 
 namespace odwf {
 
 namespace {
-constexpr int kBSF = 128;
+constexpr int kBSF = 128;       // four warps, one per direction
+constexpr int kForceSites = 8;  // sites per block, four lanes each
 
 struct C3 {
     double2 m[9];
 };
 
 __device__ __forceinline__ double2 zmul(double2 a, double2 b) { return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
-__device__ __forceinline__ double2 zmulc(double2 a, double2 b) {  // a conj(b)
-    return make_double2(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
-}
 __device__ __forceinline__ double2 zadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 
-// K_{ba} += sum_spin r[spin][b] conj(w[spin][a])
-__device__ __forceinline__ void outer_acc(const double r[24], const double w[24], C3& K) {
+// K_{ba} += sum_spin r[spin][b] conj(w[spin][a]) over the half spinors r and w
+__device__ __forceinline__ void outer_acc(const double r[12], const double w[12], C3& K) {
 #pragma unroll
     for (int b = 0; b < 3; ++b)
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             double2 acc = K.m[3 * b + a];
 #pragma unroll
-            for (int sp = 0; sp < 4; ++sp) {
-                const double2 rv = make_double2(r[(sp * 3 + b) * 2], r[(sp * 3 + b) * 2 + 1]);
-                const double2 wv = make_double2(w[(sp * 3 + a) * 2], w[(sp * 3 + a) * 2 + 1]);
-                acc = zadd(acc, zmulc(rv, wv));
+            for (int sp = 0; sp < 2; ++sp) {
+                const double rr = r[6 * sp + 2 * b], ri = r[6 * sp + 2 * b + 1];
+                const double wr = w[6 * sp + 2 * a], wi = w[6 * sp + 2 * a + 1];
+                acc.x = fma(rr, wr, acc.x);
+                acc.x = fma(ri, wi, acc.x);
+                acc.y = fma(ri, wr, acc.y);
+                acc.y = fma(-rr, wi, acc.y);
             }
             K.m[3 * b + a] = acc;
         }
 }
 
-// w = (1 + sg gamma_mu) v
-__device__ __forceinline__ void proj_full(int mu, double sg, const double v[24], double w[24]) {
-    double h[12];
-    project(mu, sg, v, h);
-#pragma unroll
-    for (int k = 0; k < 24; ++k) w[k] = 0.0;
-    accumulate(mu, sg, h, w);
+__device__ __forceinline__ double2 shfl_xor2(double2 v, int m) {
+    return make_double2(__shfl_xor_sync(0xffffffffu, v.x, m), __shfl_xor_sync(0xffffffffu, v.y, m));
 }
 
 __global__ void __launch_bounds__(kBSF) force_contract_kernel(Geom g, int ns, const void* __restrict__ links, FieldRef Le,
                                                               FieldRef Lo, FieldRef Re, FieldRef Ro, double coef,
                                                               double2* __restrict__ G, int accumulate_into) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;  // ((p * Vh + h) * 4 + mu)
-    if (i >= (size_t)8 * g.Vh) return;
-    const int mu = (int)(i & 3);
-    const size_t ph = i >> 2;
+    const int mu = threadIdx.x >> 5, sl = threadIdx.x & 3;
+    const size_t site = (size_t)blockIdx.x * kForceSites + ((threadIdx.x & 31) >> 2);
+    const bool valid = site < (size_t)2 * g.Vh;
+    const size_t ph = valid ? site : 0;
     const int p = (int)(ph / g.Vh), h = (int)(ph % g.Vh);
     int c[4];
     site_coords(g, p, h, c);
@@ -79,38 +78,67 @@ __global__ void __launch_bounds__(kBSF) force_contract_kernel(Geom g, int ns, co
     C3 K1, K2;
 #pragma unroll
     for (int k = 0; k < 9; ++k) K1.m[k] = K2.m[k] = make_double2(0.0, 0.0);
-    double v[24], w[24];
+    double v[24], hl[12], hr[12];
 #pragma unroll 1
-    for (int s = 0; s < ns; ++s) {
+    for (int s = sl; s < ns; s += 4) {
         SpinorIO<SpF64, double>::load(Lx.d(0), nullptr, (size_t)h, s, ns, v);
-        proj_full(mu, -1.0, v, w);  // (1 - gamma_mu) L(x)
+        project(mu, -1.0, v, hl);  // (1 - gamma_mu) L(x)
         SpinorIO<SpF64, double>::load(Rn.d(0), nullptr, (size_t)hn, s, ns, v);
-        outer_acc(v, w, K1);
+        project(mu, -1.0, v, hr);
+        outer_acc(hr, hl, K1);
         SpinorIO<SpF64, double>::load(Ln.d(0), nullptr, (size_t)hn, s, ns, v);
-        proj_full(mu, 1.0, v, w);  // (1 + gamma_mu) L(x + mu)
+        project(mu, 1.0, v, hl);  // (1 + gamma_mu) L(x + mu)
         SpinorIO<SpF64, double>::load(Rx.d(0), nullptr, (size_t)h, s, ns, v);
-        outer_acc(v, w, K2);
+        project(mu, 1.0, v, hr);
+        outer_acc(hr, hl, K2);
+    }
+    // the link's sums over its lanes: K1 in the even ones, K2 in the odd ones
+    const bool odd = sl & 1;
+    C3 K;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const double2 send = odd ? K1.m[k] : K2.m[k], keep = odd ? K2.m[k] : K1.m[k];
+        const double2 t = zadd(keep, shfl_xor2(send, 1));
+        K.m[k] = zadd(t, shfl_xor2(t, 2));
     }
     double u[18];
     LinkIO<LinkD18, double>::load(links, (size_t)(p * 4 + mu) * g.Vh + h, u);
     double sgn = coef;
     if (mu == 3 && g.tbc && c[3] == g.L[3] - 1) sgn = -sgn;
     double2* Gl = G + ((size_t)(p * 4 + mu) * g.Vh + h) * 9;
+    // G = U K1 - K2 U^+.  The odd lanes form (K2 U^+)^T = conj(U) K2^T, so that both take the same path.
+    if (odd) {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) u[2 * k + 1] = -u[2 * k + 1];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < a; ++b) {
+                const double2 t = K.m[3 * a + b];
+                K.m[3 * a + b] = K.m[3 * b + a];
+                K.m[3 * b + a] = t;
+            }
+    }
+    C3 Q;
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
             double2 acc = make_double2(0.0, 0.0);
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const double2 uak = make_double2(u[2 * (3 * a + k)], u[2 * (3 * a + k) + 1]);
-                const double2 ubk = make_double2(u[2 * (3 * b + k)], u[2 * (3 * b + k) + 1]);
-                acc = zadd(acc, zmul(uak, K1.m[3 * k + b]));    // (U K1)_{ab}
-                const double2 t = zmulc(K2.m[3 * a + k], ubk);  // K2_{ak} conj(U_{bk}) = (K2 U^+)_{ab}
-                acc = make_double2(acc.x - t.x, acc.y - t.y);
+            for (int k = 0; k < 3; ++k)
+                acc = zadd(acc, zmul(make_double2(u[2 * (3 * a + k)], u[2 * (3 * a + k) + 1]), K.m[3 * k + b]));
+            Q.m[3 * a + b] = acc;
+        }
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const double2 t = shfl_xor2(Q.m[3 * b + a], 1);  // the odd lane's product is transposed
+            if (valid && sl == 0) {
+                const double2 acc = make_double2(sgn * (Q.m[3 * a + b].x - t.x), sgn * (Q.m[3 * a + b].y - t.y));
+                Gl[3 * a + b] = accumulate_into ? zadd(Gl[3 * a + b], acc) : acc;
             }
-            acc = make_double2(sgn * acc.x, sgn * acc.y);
-            Gl[3 * a + b] = accumulate_into ? zadd(Gl[3 * a + b], acc) : acc;
         }
 }
 
@@ -181,9 +209,9 @@ constexpr int kSumsqBlocks = 608;  // 4 blocks per SM of a 152-SM part
 cudaError_t launch_force_contract(const Geom& g, int ns, const void* links_d18, const FieldRef& Le, const FieldRef& Lo,
                                   const FieldRef& Re, const FieldRef& Ro, double coef, double2* G, bool accumulate_into,
                                   cudaStream_t st) {
-    const size_t n = (size_t)8 * g.Vh;
+    const size_t n = (size_t)2 * g.Vh;
     note_launch();
-    force_contract_kernel<<<(unsigned)((n + kBSF - 1) / kBSF), kBSF, 0, st>>>(g, ns, links_d18, Le, Lo, Re, Ro, coef, G,
+    force_contract_kernel<<<(unsigned)((n + kForceSites - 1) / kForceSites), kBSF, 0, st>>>(g, ns, links_d18, Le, Lo, Re, Ro, coef, G,
                                                                              accumulate_into ? 1 : 0);
     return cudaGetLastError();
 }
