@@ -4,7 +4,7 @@
 One step solves the 16^3 x 32 x Ns=16 workload's three systems (m_q = 0.002, 0.04, 0.5,
 one Gaussian right-hand side each) to a true residual of 1e-10 with the batched mixed-
 precision CG (FP16 storage with per-site scales, FP32 links of 12 reals, FP32 arithmetic,
-float-float reliable updates), as one odwf_cg_solve_batched call.  Prints one JSON line.
+reliable updates at FP64 accuracy), as one odwf_cg_solve_batched call.  Prints one JSON line.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference] [--prec f16|bf16|f32]
 
@@ -179,12 +179,12 @@ def ncu_traffic_file(path, kernel_class):
     return None
 
 
-# Kernel classes whose source changed after the committed ncu captures: the block partial of their
-# final reduction moved to a fixed per-system stride (one 8-byte store per block, nothing else).
+# Kernel classes whose source changed after the committed ncu captures: their final reduction became one
+# 8-byte store per block, and later launches sum.
 # Their captured DRAM bytes are reported as prior-capture values, `traffic` itself is null.
 TRAFFIC_CHANGED_SINCE_CAPTURE = ("K2_schur_norm_mdinv", "K4_normal_cg")
-TRAFFIC_NOTE = ("captured before the final reduction's block partial moved to a fixed per-system stride "
-                "(the only change to this kernel since; one 8-byte store per block)")
+TRAFFIC_NOTE = ("captured before this kernel left the sum of its block partials to later launches "
+                "(one 8-byte store per block; its fields are read and written as before)")
 
 
 def traffic_fields(kernel_class, tr):
@@ -210,8 +210,8 @@ def ncu_traffic(kernel_class):
 
 
 def update_arith_name(updates):
-    """The reliable-update arithmetic of a mixed solve (AUTO is float-float)."""
-    return "FP64" if updates == "f64" else "float-float"
+    """The reliable-update arithmetic of a mixed solve: every setting runs the same operator."""
+    return "FP64-accurate fixed point"
 
 
 def aggregate(t_local_s: float, solves_local: int, dist=None, device=None):
@@ -1037,7 +1037,7 @@ def run_batched_c3(args, world, rank, local):
 
 def run_paper_scale_c5(args, world, rank, local):
     """64^4 x Ns=16, m_q = 0.002, links exp(0.2 i H) seed 5 stored as FP32 12-real, BF16 inner
-    solve with float-float reliable updates, one Gaussian right-hand side (seed 5), one solve per
+    solve with reliable updates at FP64 accuracy, one Gaussian right-hand side (seed 5), one solve per
     step.  Reports the solve time, iterations, true residual and the device memory used."""
     import torch
 

@@ -1,7 +1,7 @@
 // Block fixed point for the FP64-accuracy hops.
 //
-// GB300 issues about 2 FP64 operations per clock and SM but 64 integer multiply-adds
-// 32 x 32 + 64 -> 64 bits, so the SU(3) products of the hopping term, which are nearly all of its
+// GB300 issues about 2 FP64 operations per clock and SM but about 28 integer
+// multiply-adds 32 x 32 + 64 -> 64 bits, so the SU(3) products of the hopping term, which are nearly all of its
 // arithmetic, run in integers: a spinor of one 5D site is 24 signed integers with one exponent,
 //     value = q 2^e,  |q| < 2^59,
 // a link 18 integers with one exponent (|u| < 2^60 2^eu), both split into 31-bit limbs

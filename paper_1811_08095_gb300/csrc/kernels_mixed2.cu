@@ -26,6 +26,7 @@ namespace {
 
 using namespace mx;
 
+// K4 on 32^4 x 16, one system: 933 us with a last block that summed the 32768 partials, 820 without (5.8 TB/s)
 constexpr int kBS2 = 256;
 constexpr int kBS2Deep = 64;
 

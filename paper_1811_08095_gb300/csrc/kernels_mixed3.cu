@@ -4,7 +4,8 @@
 // site's Ns/2-lane group holding the 5D sites s = 2l and 2l + 1.  K4, which also streams the FP32
 // CG vectors r and x in and out, stays with one s per lane: at the higher occupancy of that kernel
 // its streams are hidden better (measured on 32^4 x 16, one system: K1 509 -> 422 us, K3 524 ->
-// 425 us, K2 784 -> 708 us here; K4 922 us there against 982 us here).
+// 425 us, K2 784 -> 708 us here; K4 922 us there against 982 us here).  Since then FP16 operands go into the
+// FP32 FMAs unconverted (K1 387, K3 391 us) and K2 leaves the sum of its partials to K3 (527 us).
 //
 // Why two s per lane: on GB300 the one-s-per-lane hops are bound by the L1/shared-memory data
 // path, not by HBM.  With two s per lane
