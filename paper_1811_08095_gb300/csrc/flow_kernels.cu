@@ -709,7 +709,8 @@ __device__ __forceinline__ long long fixed60(float x) {
 
 // The sums h + l and the third row conj(row0 x row1) in fixed point (60 fraction bits; 72 FP64
 // operations per link bound the FP64 form at 91 us per direction of 24^3x48), converted once per
-// entry.  A link with an entry of 1.5 or more, or a non-finite one, takes the FP64 form.  The block's
+// entry.  A link with an entry of 1.25 or more, or a non-finite one, takes the FP64 form: a component of
+// the third row is at most 4 m^2 for entries up to m, and 60 fraction bits hold less than 8.  The block's
 // links go out through shared memory, so that stores are contiguous.
 constexpr int kJoin = 128;
 __global__ void __launch_bounds__(kJoin) join_kernel(const float4* __restrict__ hi, const float4* __restrict__ lo,
@@ -732,7 +733,7 @@ __global__ void __launch_bounds__(kJoin) join_kernel(const float4* __restrict__ 
             nan = nan || h[k] != h[k] || l[k] != l[k];
         }
         double2 m[9];
-        if (big < 1.5f && !nan) {
+        if (big < 1.25f && !nan) {
             long long q[12];
             FxLimbs x[12];
 #pragma unroll
