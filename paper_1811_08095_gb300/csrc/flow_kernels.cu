@@ -698,20 +698,29 @@ __global__ void __launch_bounds__(kSplit) split_kernel(const double2* __restrict
     }
 }
 
-// 60 fraction bits of x, |x| < 2
-__device__ __forceinline__ long long fixed60(float x) {
-    const unsigned b = __float_as_uint(x);
-    const int e = (int)((b >> 23) & 0xff) - 90;  // left shift of the 24-bit significand
-    const long long m = e > -90 ? (long long)((b & 0x7fffffu) | 0x800000u) : 0;
-    const long long q = e >= 0 ? m << e : m >> min(-e, 63);
-    return (int)b < 0 ? -q : q;
+// h + l in integers, exactly the FP64 sum: q 2^e with h's significand at bit 38 of q and what of l lies below
+// bit 0 kept as a sticky bit, so that the one rounding is the conversion of q.  |l| <= |h| in exponent, both
+// finite.
+__device__ __forceinline__ long long pair_sum(float h, float l, int& e) {
+    const unsigned bh = __float_as_uint(h), bl = __float_as_uint(l);
+    const int fh = (int)((bh >> 23) & 0xff), fl = (int)((bl >> 23) & 0xff);
+    const long long mh = (long long)((bh & 0x7fffffu) | (fh ? 0x800000u : 0u)) << 38;
+    const unsigned long long m = (unsigned long long)((bl & 0x7fffffu) | (fl ? 0x800000u : 0u)) << 38;
+    const int down = min(max(fh, 1) - max(fl, 1), 63);
+    const unsigned long long d = m >> down;
+    const long long ml = (long long)(d | (unsigned long long)((d << down) != m));
+    e = max(fh, 1) - 188;  // 127 + 23 + 38
+    return ((int)bh < 0 ? -mh : mh) + ((int)bl < 0 ? -ml : ml);
 }
 
-// The sums h + l and the third row conj(row0 x row1) in fixed point (60 fraction bits; 72 FP64
+// The sums h + l in integers; the third row conj(row0 x row1) in fixed point (60 fraction bits; 72 FP64
 // operations per link bound the FP64 form at 91 us per direction of 24^3x48), converted once per
-// entry.  A link with an entry of 1.25 or more, or a non-finite one, takes the FP64 form: a component of
-// the third row is at most 4 m^2 for entries up to m, and 60 fraction bits hold less than 8.  The block's
-// links go out through shared memory, so that stores are contiguous.
+// entry.  An entry of the third row is two products of two complex numbers, of size D; the fixed-point form
+// errs by about 2^-59.5 of 1 and FP64 by about 2^-53.5 D, so entries with D below 2^-6 are formed in FP64, all of
+// them for a link with an entry of 1.25 or more (a component is at most 4 m^2 for entries up to m, and 60
+// fraction bits hold less than 8) or a non-finite one.  24^3x48, all directions: 127 us for rough links, 183
+// us for links within 1e-3 of 1, which all have small entries (369 us in FP64).  The block's links go out
+// through shared memory, so that stores are contiguous.
 constexpr int kJoin = 128;
 __global__ void __launch_bounds__(kJoin) join_kernel(const float4* __restrict__ hi, const float4* __restrict__ lo,
                                                      double2* __restrict__ U, size_t V, int mu0) {
@@ -719,7 +728,7 @@ __global__ void __launch_bounds__(kJoin) join_kernel(const float4* __restrict__ 
     const size_t s0 = (size_t)blockIdx.x * kJoin, s = s0 + threadIdx.x;
     if (s < V) {
         float h[12], l[12], big = 0.f;
-        bool nan = false;
+        bool odd = false;  // a non-finite value, or a pair out of order
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
             const size_t o = ((size_t)(mu0 + blockIdx.y) * 3 + j) * V + s;
@@ -729,29 +738,42 @@ __global__ void __launch_bounds__(kJoin) join_kernel(const float4* __restrict__ 
         }
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
-            big = fmaxf(big, fmaxf(fabsf(h[k]), fabsf(l[k])));
-            nan = nan || h[k] != h[k] || l[k] != l[k];
+            big = fmaxf(big, fabsf(h[k]));
+            odd = odd || !(fabsf(l[k]) <= fabsf(h[k])) || !(fabsf(h[k]) < INFINITY);
         }
         double2 m[9];
-        if (big < 1.25f && !nan) {
-            long long q[12];
-            FxLimbs x[12];
+        FxLimbs x[12];
+        if (!odd) {
+            double d[12];
 #pragma unroll
             for (int k = 0; k < 12; ++k) {
-                q[k] = fixed60(h[k]) + fixed60(l[k]);
-                x[k] = fx_split(q[k]);
+                int e;
+                const long long q = pair_sum(h[k], l[k], e);
+                d[k] = fx_to_double(q, e);
+                x[k] = fx_split(q >> min(max(-60 - e, 0), 63));  // 60 fraction bits; used below 1.25
             }
 #pragma unroll
-            for (int k = 0; k < 6; ++k) m[k] = make_double2(fx_to_double(q[2 * k], -60), fx_to_double(q[2 * k + 1], -60));
+            for (int k = 0; k < 6; ++k) m[k] = make_double2(d[2 * k], d[2 * k + 1]);
+        } else {
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                // conj(a1 b2 - a2 b1), a = row 0, b = row 1: leading and cross sums of the 31-bit limbs
-                const int a1 = 2 * ((k + 1) % 3), a2 = 2 * ((k + 2) % 3), b1 = 6 + a1, b2 = 6 + a2;
+            for (int k = 0; k < 6; ++k)
+                m[k] = make_double2((double)h[2 * k] + (double)l[2 * k], (double)h[2 * k + 1] + (double)l[2 * k + 1]);
+        }
+        float c[6];  // sizes of the entries of the two rows
+#pragma unroll
+        for (int k = 0; k < 6; ++k) c[k] = fmaxf(fabsf(h[2 * k]), fabsf(h[2 * k + 1]));
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            // conj(a1 b2 - a2 b1), a = row 0, b = row 1
+            const int k1 = (k + 1) % 3, k2 = (k + 2) % 3;
+            if (!odd && big < 1.25f && c[k1] * c[3 + k2] + c[k2] * c[3 + k1] >= 0x1p-6f) {
+                // leading and cross sums of the 31-bit limbs
+                const int a1 = 2 * k1, a2 = 2 * k2, b1 = 6 + a1, b2 = 6 + a2;
                 long long A[2] = {0, 0}, B[2] = {1ll << 28, 1ll << 28};
-                auto mac = [&](int c, const FxLimbs& u, const FxLimbs& v, bool minus) {
+                auto mac = [&](int i, const FxLimbs& u, const FxLimbs& v, bool minus) {
                     const int n1 = minus ? fx_neg(u.hi) : u.hi, n0 = minus ? fx_neg(u.lo) : u.lo;
-                    A[c] = fx_mad(n1, v.hi, A[c]);
-                    B[c] = fx_mad(n1, v.lo, fx_mad(n0, v.hi, B[c]));
+                    A[i] = fx_mad(n1, v.hi, A[i]);
+                    B[i] = fx_mad(n1, v.lo, fx_mad(n0, v.hi, B[i]));
                 };
                 mac(0, x[a1], x[b2], false);
                 mac(0, x[a1 + 1], x[b2 + 1], true);
@@ -763,15 +785,8 @@ __global__ void __launch_bounds__(kJoin) join_kernel(const float4* __restrict__ 
                 mac(1, x[a2 + 1], x[b1], false);
                 m[6 + k] = make_double2(fx_to_double((A[0] << 2) + (B[0] >> 29), -60),
                                         fx_to_double((A[1] << 2) + (B[1] >> 29), -60));
-            }
-        } else {
-#pragma unroll
-            for (int k = 0; k < 6; ++k)
-                m[k] = make_double2((double)h[2 * k] + (double)l[2 * k], (double)h[2 * k + 1] + (double)l[2 * k + 1]);
-            const double2 *a = m, *b = m + 3;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const int k1 = (k + 1) % 3, k2 = (k + 2) % 3;
+            } else {
+                const double2 *a = m, *b = m + 3;
                 const double re = (a[k1].x * b[k2].x - a[k1].y * b[k2].y) - (a[k2].x * b[k1].x - a[k2].y * b[k1].y);
                 const double im = (a[k1].x * b[k2].y + a[k1].y * b[k2].x) - (a[k2].x * b[k1].y + a[k2].y * b[k1].x);
                 m[6 + k] = make_double2(re, -im);
