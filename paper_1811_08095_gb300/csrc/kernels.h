@@ -79,7 +79,12 @@ struct GaugeLex {
     size_t stride[4];
     size_t V;
 };
-// its split and force kernels; work = 36 V int4 limbs and the flag of links outside the fixed-point range
+// what the split of the links found: one outside the fixed-point range, how many with one large entry per row
+struct GaugeFlags {
+    int bad, nweak, pad[2];
+};
+__host__ __device__ inline bool gauge_all_fp64(const GaugeFlags& f, size_t links) { return f.bad || (size_t)f.nweak * 64 > links; }
+// its split and force kernels; work = 36 V int4 limbs, the flags and a mark (one byte) per link
 cudaError_t launch_gauge_force_fx(const GaugeLex& g, const double2* U, void* work, double beta, double2* F,
                                   double* partials, cudaStream_t st);
 cudaError_t launch_link_update(size_t nlinks, double2* U, const double2* P, double a, cudaStream_t st);  // U <- exp(aP) U

@@ -7,7 +7,17 @@
 // and U Sigma to 2^-56, against 2^-53 of each FP64 operation.  Fields whose rows or columns are not of
 // unit length to 2^-16 (the entry points take any matrices) raise a flag in the pass that splits the
 // links, and the FP64 kernel of kernels_md.cu runs instead; both are launched and one of them returns at
-// once.  16^3x32, action and force: 2.04 ms in FP64, 0.49 ms here (split 25 us, force 0.44 ms); bound by
+// once.
+//
+// Where the links have one large entry per row (near the unit field, or an abelian one) the force comes from
+// the small entries, whose products FP64 keeps to 2^-53 of themselves and limbs to 2^-58 of 1.  With links
+// exp(i eps H) both err by 1.4e-16 of the force (rms, FP64 at every eps) at eps = 0.035, where the off-diagonal
+// entries are about 2^-6; the limbs by 1.0e-16 at 0.25, 2.1e-16 at 0.02 and 3.7e-15 at 0.001.  The pass that splits the links marks those
+// whose other six entries are below 2^-6; the FP64 kernel takes the marked ones and this one the others, each
+// adding to its block's sum.  From one marked link in 64 the whole field goes to the FP64 kernel, since a warp that
+// holds one takes as long there as a full one: 0.50 ms at eps = 0.25, 0.58 at 0.1, 1.29 at 0.05, 2.07 from 0.03 down.
+//
+// 16^3x32, action and force: 2.04 ms in FP64, 0.50 ms here (split 25 us, force 0.44 ms); bound by
 // the latency of the integer chains with the 8 warps per SM that 244 registers leave (three blocks per
 // SM spill 300 bytes: 0.50 ms, four 0.56 ms).
 //
@@ -22,6 +32,7 @@ namespace odwf {
 namespace {
 
 constexpr int kBSG = 128;
+constexpr int kWeakEntry = 0x3f900000;  // high word of 2^-6
 
 // element k of link (mu, s) as (re1, re0, im1, im0) at limbs[(k * 4 + mu) * V + s]
 struct FxM {
@@ -111,40 +122,48 @@ __device__ __forceinline__ void fx_staple(const int4* __restrict__ U, size_t V, 
     }
 }
 
-// Links (external layout, n = 4 V of them) into limbs; *bad |= 1 for a link outside the fixed-point range
+// Links (external layout, n = 4 V of them) into limbs and their marks; flags->bad for a link outside the
+// fixed-point range
 __global__ void __launch_bounds__(kBSG) split_links_kernel(const double2* __restrict__ U, size_t n, int4* __restrict__ out,
-                                                           int* __restrict__ bad) {
+                                                           GaugeFlags* __restrict__ flags, unsigned char* __restrict__ weak) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
     float row[3] = {0.f, 0.f, 0.f}, col[3] = {0.f, 0.f, 0.f};
     bool big = false;
+    int large = 0;  // entries of 2^-6 and more: three in a matrix with one such entry per row
+    if (i < n) {
 #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        const double2 u = U[i * 9 + k];
-        const int m = max(__double2hiint(u.x) & 0x7fffffff, __double2hiint(u.y) & 0x7fffffff);
-        big = big || m >= 0x3ff80000;  // 1.5, and non-finite values
-        const long long re = fx_from_double<8>(u.x, 1023), im = fx_from_double<8>(u.y, 1023);  // |u| < 2 to 60 bits
-        const FxLimbs r = fx_split(re), q = fx_split(im);
-        out[(size_t)k * n + i] = make_int4(r.hi, r.lo, q.hi, q.lo);
-        const float a = (float)r.hi * 0x1p-29f, b = (float)q.hi * 0x1p-29f;
-        const float t = fmaf(a, a, b * b);
-        row[k / 3] += t;
-        col[k % 3] += t;
+        for (int k = 0; k < 9; ++k) {
+            const double2 u = U[i * 9 + k];
+            const int m = max(__double2hiint(u.x) & 0x7fffffff, __double2hiint(u.y) & 0x7fffffff);
+            big = big || m >= 0x3ff80000;  // 1.5, and non-finite values
+            large += m >= kWeakEntry;
+            const long long re = fx_from_double<8>(u.x, 1023), im = fx_from_double<8>(u.y, 1023);  // |u| < 2 to 60 bits
+            const FxLimbs r = fx_split(re), q = fx_split(im);
+            out[(size_t)k * n + i] = make_int4(r.hi, r.lo, q.hi, q.lo);
+            const float a = (float)r.hi * 0x1p-29f, b = (float)q.hi * 0x1p-29f;
+            const float t = fmaf(a, a, b * b);
+            row[k / 3] += t;
+            col[k % 3] += t;
+        }
+        float worst = 0.f;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) worst = fmaxf(worst, fmaxf(fabsf(row[k] - 1.f), fabsf(col[k] - 1.f)));
+        if (big || !(worst < 0x1p-15f)) atomicOr(&flags->bad, 1);
+        weak[i] = large <= 3;
     }
-    float worst = 0.f;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) worst = fmaxf(worst, fmaxf(fabsf(row[k] - 1.f), fabsf(col[k] - 1.f)));
-    if (big || !(worst < 0x1p-15f)) atomicOr(bad, 1);
+    const int nweak = __syncthreads_count(i < n && large <= 3);
+    if (threadIdx.x == 0 && nweak) atomicAdd(&flags->nweak, nweak);
 }
 
-// One thread per link (mu, s), as gauge_force_kernel: Pi (optional) and per-block sums of Re tr(U Sigma)
+// One thread per unmarked link (mu, s), as gauge_force_kernel: Pi (optional) and per-block sums of Re tr(U Sigma)
 __global__ void __launch_bounds__(kBSG, 2) gauge_force_fx_kernel(GaugeLex g, const int4* __restrict__ U,
-                                                                 const int* __restrict__ bad, double beta,
+                                                                 const GaugeFlags* __restrict__ flags,
+                                                                 const unsigned char* __restrict__ weak, double beta,
                                                                  double2* __restrict__ F, double* __restrict__ part) {
-    if (*bad) return;
+    if (gauge_all_fp64(*flags, 4 * g.V)) return;
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     double retr = 0.0;
-    if (i < 4 * g.V) {
+    if (i < 4 * g.V && !weak[i]) {
         const int mu = (int)(i / g.V);
         const size_t s = i - (size_t)mu * g.V;
         int c[4];
@@ -217,14 +236,15 @@ __global__ void __launch_bounds__(kBSG, 2) gauge_force_fx_kernel(GaugeLex g, con
 cudaError_t launch_gauge_force_fx(const GaugeLex& g, const double2* U, void* work, double beta, double2* F,
                                   double* partials, cudaStream_t st) {
     int4* limbs = (int4*)work;
-    int* bad = (int*)(limbs + 36 * g.V);
-    cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int), st);
+    GaugeFlags* flags = (GaugeFlags*)(limbs + 36 * g.V);
+    unsigned char* weak = (unsigned char*)(flags + 1);
+    cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(GaugeFlags), st);
     if (e != cudaSuccess) return e;
     const unsigned nb = (unsigned)((4 * g.V + kBSG - 1) / kBSG);
     note_launch();
-    split_links_kernel<<<nb, kBSG, 0, st>>>(U, 4 * g.V, limbs, bad);
+    split_links_kernel<<<nb, kBSG, 0, st>>>(U, 4 * g.V, limbs, flags, weak);
     note_launch();
-    gauge_force_fx_kernel<<<nb, kBSG, 0, st>>>(g, limbs, bad, beta, F, partials);
+    gauge_force_fx_kernel<<<nb, kBSG, 0, st>>>(g, limbs, flags, weak, beta, F, partials);
     return cudaGetLastError();
 }
 
