@@ -69,9 +69,20 @@ cudaError_t launch_sum_partials(const double* partials, int nb, double* out, cud
 // gauge force: F (may be null) = -(beta/3) ta(U Sigma) per link; *retr_sum = sum_links Re tr(U Sigma)
 // (partials: gauge_force_blocks(V) doubles)
 size_t gauge_force_blocks(size_t V);
-// work: gauge_force_work(V) bytes for the fixed-point kernel (kernels_gauge_fx.cu), or null to run in FP64
-size_t gauge_force_work(size_t V);
-cudaError_t launch_gauge_force(const int dims[4], const double2* U, void* work, double beta, double2* F,
+// what the split of the links found: one outside the fixed-point range, how many with one large entry per row
+struct GaugeFlags {
+    int bad, nweak, pad[2];
+};
+__host__ __device__ inline bool gauge_all_fp64(const GaugeFlags& f, size_t links) { return f.bad || (size_t)f.nweak * 64 > links; }
+// workspace of the fixed-point kernel (kernels_gauge_fx.cu): a mark per link, and the limbs, gauge_limb_bytes(V), or null to
+// split the links where they are used
+struct GaugeWork {
+    GaugeFlags* flags;
+    unsigned char* weak;
+    void* limbs;
+};
+size_t gauge_limb_bytes(size_t V);
+cudaError_t launch_gauge_force(const int dims[4], const double2* U, const GaugeWork& work, double beta, double2* F,
                                double* partials, double* retr_sum, cudaStream_t st);
 // lexicographic sites of the external gauge layout
 struct GaugeLex {
@@ -79,13 +90,8 @@ struct GaugeLex {
     size_t stride[4];
     size_t V;
 };
-// what the split of the links found: one outside the fixed-point range, how many with one large entry per row
-struct GaugeFlags {
-    int bad, nweak, pad[2];
-};
-__host__ __device__ inline bool gauge_all_fp64(const GaugeFlags& f, size_t links) { return f.bad || (size_t)f.nweak * 64 > links; }
-// its split and force kernels; work = 36 V int4 limbs, the flags and a mark (one byte) per link
-cudaError_t launch_gauge_force_fx(const GaugeLex& g, const double2* U, void* work, double beta, double2* F,
+// its split and force kernels
+cudaError_t launch_gauge_force_fx(const GaugeLex& g, const double2* U, const GaugeWork& work, double beta, double2* F,
                                   double* partials, cudaStream_t st);
 cudaError_t launch_link_update(size_t nlinks, double2* U, const double2* P, double a, cudaStream_t st);  // U <- exp(aP) U
 cudaError_t launch_axpy(size_t n, double2* y, const double2* x, double c, cudaStream_t st);              // y += c x

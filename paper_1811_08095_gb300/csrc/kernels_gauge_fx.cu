@@ -17,6 +17,10 @@
 // adding to its block's sum.  From one marked link in 64 the whole field goes to the FP64 kernel, since a warp that
 // holds one takes as long there as a full one: 0.50 ms at eps = 0.25, 0.58 at 0.1, 1.29 at 0.05, 2.07 from 0.03 down.
 //
+// Splitting the links where they are used instead of in a pass before gives the same bits and needs no
+// workspace for the limbs, but takes twice as long (16^3x32 1.03 ms; 8^4, where the chip is not full, 88 us
+// against 57): for calls that would have to allocate it first, see Engine::gauge_force.
+//
 // 16^3x32, action and force: 2.04 ms in FP64, 0.50 ms here (split 25 us, force 0.44 ms); bound by
 // the latency of the integer chains with the 8 warps per SM that 244 registers leave (three blocks per
 // SM spill 300 bytes: 0.50 ms, four 0.56 ms).
@@ -34,17 +38,39 @@ namespace {
 constexpr int kBSG = 128;
 constexpr int kWeakEntry = 0x3f900000;  // high word of 2^-6
 
-// element k of link (mu, s) as (re1, re0, im1, im0) at limbs[(k * 4 + mu) * V + s]
+// Element k of a link as (re1, re0, im1, im0).  Limbs: split by a pass before, element k of link (mu, s) at
+// p[(k * 4 + mu) * V + s].  Direct: the caller's FP64 links, split where they are used.
 struct FxM {
     int4 e[9];
 };
 
-__device__ __forceinline__ FxM fx_ld(const int4* __restrict__ U, size_t V, int mu, size_t s) {
-    FxM m;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) m.e[k] = __ldg(U + ((size_t)(k * 4 + mu) * V + s));
-    return m;
+__device__ __forceinline__ int4 fx_split_entry(double2 u) {  // |u| < 2 to 60 fraction bits
+    const FxLimbs r = fx_split(fx_from_double<8>(u.x, 1023)), q = fx_split(fx_from_double<8>(u.y, 1023));
+    return make_int4(r.hi, r.lo, q.hi, q.lo);
 }
+
+// loads are issued where they stand: rows are read again from L1 rather than held in registers
+struct Limbs {
+    const int4* p;
+    size_t st;  // between the elements of a link
+    __device__ __forceinline__ Limbs(const void* links, size_t V, int mu, size_t s)
+        : p((const int4*)links + (size_t)mu * V + s), st(4 * V) {}
+    __device__ __forceinline__ int4 at(int k) const {
+        int4 v;
+        asm volatile("ld.global.nc.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p + k * st));
+        return v;
+    }
+};
+struct Direct {
+    const double2* p;
+    __device__ __forceinline__ Direct(const void* links, size_t V, int mu, size_t s)
+        : p((const double2*)links + ((size_t)mu * V + s) * 9) {}
+    __device__ __forceinline__ int4 at(int k) const {
+        double2 v;
+        asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p + k));
+        return fx_split_entry(v);
+    }
+};
 
 // (A, B) += x y of the limb pairs: A the product of the leading limbs, B the cross terms
 __device__ __forceinline__ void fx_macc(int x1, int x0, int y1, int y0, long long& A, long long& B) {
@@ -84,29 +110,19 @@ __device__ __forceinline__ void fx_dot3(const int4 x[3], const int4 y0, const in
     if (CY) im = -im;
 }
 
-// a load that is issued where it stands: rows are read again from L1 rather than held in registers
-__device__ __forceinline__ int4 fx_ldv(const int4* p) {
-    int4 v;
-    asm volatile("ld.global.nc.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-    return v;
-}
-
 // One staple, row by row: T_i = a_i B^dag with a_i row i of A (LOWER: of A^dag), 58 fraction bits, and
 // S_i += T_i C^dag (LOWER: T_i C), 56 fraction bits.  Only a row of A and of T is held at a time.
-template <bool LOWER>
-__device__ __forceinline__ void fx_staple(const int4* __restrict__ U, size_t V, int ma, size_t sa, int mb, size_t sb,
-                                          int mc, size_t sc, long long S[18]) {
-    const int4 *pa = U + (size_t)ma * V + sa, *pb = U + (size_t)mb * V + sb, *pc = U + (size_t)mc * V + sc;
-    const size_t st = 4 * V;  // between the elements of a link
+template <bool LOWER, class SRC>
+__device__ __forceinline__ void fx_staple(const SRC A, const SRC B, const SRC C, long long S[18]) {
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         int4 a[3], t[3];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) a[k] = fx_ldv(pa + (LOWER ? 3 * k + i : 3 * i + k) * st);
+        for (int k = 0; k < 3; ++k) a[k] = A.at(LOWER ? 3 * k + i : 3 * i + k);
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
             long long re, im;
-            fx_dot3<LOWER, true>(a, fx_ldv(pb + 3 * j * st), fx_ldv(pb + (3 * j + 1) * st), fx_ldv(pb + (3 * j + 2) * st), re, im);
+            fx_dot3<LOWER, true>(a, B.at(3 * j), B.at(3 * j + 1), B.at(3 * j + 2), re, im);
             fx_limbs(re, t[j].x, t[j].y);
             fx_limbs(im, t[j].z, t[j].w);
         }
@@ -114,16 +130,16 @@ __device__ __forceinline__ void fx_staple(const int4* __restrict__ U, size_t V, 
         for (int j = 0; j < 3; ++j) {
             long long re, im;
             constexpr int sk = LOWER ? 3 : 1;
-            const int4* q = pc + (LOWER ? j : 3 * j) * st;
-            fx_dot3<false, !LOWER>(t, fx_ldv(q), fx_ldv(q + sk * st), fx_ldv(q + 2 * sk * st), re, im);
+            const int q = LOWER ? j : 3 * j;
+            fx_dot3<false, !LOWER>(t, C.at(q), C.at(q + sk), C.at(q + 2 * sk), re, im);
             S[2 * (3 * i + j)] += re;
             S[2 * (3 * i + j) + 1] += im;
         }
     }
 }
 
-// Links (external layout, n = 4 V of them) into limbs and their marks; flags->bad for a link outside the
-// fixed-point range
+// Links (external layout, n = 4 V of them) into limbs (unless out is null) and their marks; flags->bad for a
+// link outside the fixed-point range
 __global__ void __launch_bounds__(kBSG) split_links_kernel(const double2* __restrict__ U, size_t n, int4* __restrict__ out,
                                                            GaugeFlags* __restrict__ flags, unsigned char* __restrict__ weak) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -137,10 +153,9 @@ __global__ void __launch_bounds__(kBSG) split_links_kernel(const double2* __rest
             const int m = max(__double2hiint(u.x) & 0x7fffffff, __double2hiint(u.y) & 0x7fffffff);
             big = big || m >= 0x3ff80000;  // 1.5, and non-finite values
             large += m >= kWeakEntry;
-            const long long re = fx_from_double<8>(u.x, 1023), im = fx_from_double<8>(u.y, 1023);  // |u| < 2 to 60 bits
-            const FxLimbs r = fx_split(re), q = fx_split(im);
-            out[(size_t)k * n + i] = make_int4(r.hi, r.lo, q.hi, q.lo);
-            const float a = (float)r.hi * 0x1p-29f, b = (float)q.hi * 0x1p-29f;
+            const int4 q = fx_split_entry(u);
+            if (out) out[(size_t)k * n + i] = q;
+            const float a = (float)q.x * 0x1p-29f, b = (float)q.z * 0x1p-29f;
             const float t = fmaf(a, a, b * b);
             row[k / 3] += t;
             col[k % 3] += t;
@@ -151,12 +166,13 @@ __global__ void __launch_bounds__(kBSG) split_links_kernel(const double2* __rest
         if (big || !(worst < 0x1p-15f)) atomicOr(&flags->bad, 1);
         weak[i] = large <= 3;
     }
-    const int nweak = __syncthreads_count(i < n && large <= 3);
-    if (threadIdx.x == 0 && nweak) atomicAdd(&flags->nweak, nweak);
+    const unsigned marked = __ballot_sync(0xffffffffu, i < n && large <= 3);
+    if ((threadIdx.x & 31) == 0 && marked) atomicAdd(&flags->nweak, __popc(marked));
 }
 
 // One thread per unmarked link (mu, s), as gauge_force_kernel: Pi (optional) and per-block sums of Re tr(U Sigma)
-__global__ void __launch_bounds__(kBSG, 2) gauge_force_fx_kernel(GaugeLex g, const int4* __restrict__ U,
+template <class SRC>
+__global__ void __launch_bounds__(kBSG, 2) gauge_force_fx_kernel(GaugeLex g, const void* __restrict__ U,
                                                                  const GaugeFlags* __restrict__ flags,
                                                                  const unsigned char* __restrict__ weak, double beta,
                                                                  double2* __restrict__ F, double* __restrict__ part) {
@@ -183,8 +199,10 @@ __global__ void __launch_bounds__(kBSG, 2) gauge_force_fx_kernel(GaugeLex g, con
             int cb[4] = {c[0], c[1], c[2], c[3]};
             cb[nu] = c[nu] == 0 ? g.L[nu] - 1 : c[nu] - 1;
             const size_t xmb = gauge_shift(g, cb, xb, mu, +1);  // x + mu - nu
-            fx_staple<false>(U, g.V, nu, xm, mu, xn, nu, s, S);   // U_nu(x+mu) U_mu(x+nu)^+ U_nu(x)^+
-            fx_staple<true>(U, g.V, nu, xmb, mu, xb, nu, xb, S);  // U_nu(x+mu-nu)^+ U_mu(x-nu)^+ U_nu(x-nu)
+            const SRC a(U, g.V, nu, xm), b(U, g.V, mu, xn), c0(U, g.V, nu, s);
+            fx_staple<false>(a, b, c0, S);  // U_nu(x+mu) U_mu(x+nu)^+ U_nu(x)^+
+            const SRC al(U, g.V, nu, xmb), bl(U, g.V, mu, xb), cl(U, g.V, nu, xb);
+            fx_staple<true>(al, bl, cl, S);  // U_nu(x+mu-nu)^+ U_mu(x-nu)^+ U_nu(x-nu)
         }
         FxM Sm;
 #pragma unroll
@@ -193,7 +211,10 @@ __global__ void __launch_bounds__(kBSG, 2) gauge_force_fx_kernel(GaugeLex g, con
             fx_limbs(S[2 * k + 1] << 2, Sm.e[k].z, Sm.e[k].w);
         }
         // O = U Sigma with 56 fraction bits
-        const FxM u = fx_ld(U, g.V, mu, s);
+        const SRC own(U, g.V, mu, s);
+        FxM u;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) u.e[k] = own.at(k);
         long long O[18];
 #pragma unroll
         for (int k = 0; k < 9; ++k)
@@ -233,18 +254,16 @@ __global__ void __launch_bounds__(kBSG, 2) gauge_force_fx_kernel(GaugeLex g, con
 
 }  // namespace
 
-cudaError_t launch_gauge_force_fx(const GaugeLex& g, const double2* U, void* work, double beta, double2* F,
+cudaError_t launch_gauge_force_fx(const GaugeLex& g, const double2* U, const GaugeWork& w, double beta, double2* F,
                                   double* partials, cudaStream_t st) {
-    int4* limbs = (int4*)work;
-    GaugeFlags* flags = (GaugeFlags*)(limbs + 36 * g.V);
-    unsigned char* weak = (unsigned char*)(flags + 1);
-    cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(GaugeFlags), st);
+    cudaError_t e = cudaMemsetAsync(w.flags, 0, sizeof(GaugeFlags), st);
     if (e != cudaSuccess) return e;
     const unsigned nb = (unsigned)((4 * g.V + kBSG - 1) / kBSG);
     note_launch();
-    split_links_kernel<<<nb, kBSG, 0, st>>>(U, 4 * g.V, limbs, flags, weak);
+    split_links_kernel<<<nb, kBSG, 0, st>>>(U, 4 * g.V, (int4*)w.limbs, w.flags, w.weak);
     note_launch();
-    gauge_force_fx_kernel<<<nb, kBSG, 0, st>>>(g, limbs, flags, weak, beta, F, partials);
+    if (w.limbs) gauge_force_fx_kernel<Limbs><<<nb, kBSG, 0, st>>>(g, w.limbs, w.flags, w.weak, beta, F, partials);
+    else gauge_force_fx_kernel<Direct><<<nb, kBSG, 0, st>>>(g, U, w.flags, w.weak, beta, F, partials);
     return cudaGetLastError();
 }
 

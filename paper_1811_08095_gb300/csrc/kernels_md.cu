@@ -66,12 +66,12 @@ __device__ __forceinline__ Z3 mdm(const Z3& a, const Z3& b) {  // a^+ b
 }
 
 // one thread per link (mu, s): Pi (optional) and per-block sums of Re tr(U Sigma); for the fields and links
-// that the fixed-point kernel (kernels_gauge_fx.cu) does not take, or, without flags, for all
+// that the fixed-point kernel (kernels_gauge_fx.cu), launched before, does not take
 __global__ void __launch_bounds__(kBSM) gauge_force_kernel(GaugeLex g, const double2* __restrict__ U, double beta,
                                                            double2* __restrict__ F, double* __restrict__ part,
                                                            const GaugeFlags* __restrict__ flags,
                                                            const unsigned char* __restrict__ weak) {
-    const bool all = !flags || gauge_all_fp64(*flags, 4 * g.V);
+    const bool all = gauge_all_fp64(*flags, 4 * g.V);
     if (!all && flags->nweak == 0) return;
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     double retr = 0.0;
@@ -191,9 +191,9 @@ __global__ void axpy_kernel(size_t n, double2* __restrict__ y, const double2* __
 
 size_t gauge_force_blocks(size_t V) { return (4 * V + kBSM - 1) / kBSM; }
 
-size_t gauge_force_work(size_t V) { return 36 * V * sizeof(int4) + sizeof(GaugeFlags) + 4 * V; }
+size_t gauge_limb_bytes(size_t V) { return 36 * V * sizeof(int4); }
 
-cudaError_t launch_gauge_force(const int dims[4], const double2* U, void* work, double beta, double2* F,
+cudaError_t launch_gauge_force(const int dims[4], const double2* U, const GaugeWork& work, double beta, double2* F,
                                double* partials, double* retr_sum, cudaStream_t st) {
     GaugeLex g;
     size_t stride = 1;
@@ -204,15 +204,10 @@ cudaError_t launch_gauge_force(const int dims[4], const double2* U, void* work, 
     }
     g.V = stride;
     const size_t nb = gauge_force_blocks(g.V);
-    const GaugeFlags* flags = nullptr;  // with a workspace: the FP64 kernel takes what the other one leaves
-    if (work) {
-        const cudaError_t e = launch_gauge_force_fx(g, U, work, beta, F, partials, st);
-        if (e != cudaSuccess) return e;
-        flags = (const GaugeFlags*)((const int4*)work + 36 * g.V);
-    }
+    const cudaError_t e = launch_gauge_force_fx(g, U, work, beta, F, partials, st);
+    if (e != cudaSuccess) return e;
     note_launch();
-    gauge_force_kernel<<<(unsigned)nb, kBSM, 0, st>>>(g, U, beta, F, partials, flags,
-                                                     flags ? (const unsigned char*)(flags + 1) : nullptr);
+    gauge_force_kernel<<<(unsigned)nb, kBSM, 0, st>>>(g, U, beta, F, partials, work.flags, work.weak);
     return launch_sum_partials(partials, (int)nb, retr_sum, st);
 }
 

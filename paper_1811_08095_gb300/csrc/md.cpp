@@ -22,20 +22,34 @@ namespace odwf {
 
 namespace {
 constexpr double kOmelyanLambda = 0.1931833275037836;
+// An allocation of up to 1 MB comes from the 2 MB blocks that small allocations share; a larger one costs the call
+// that makes it 90 us.  Up to 16384 sites (9 MB of limbs) that call is faster splitting the links where they
+// are used, with the allocation beside its kernels: 8^4 154 -> 140 us, 8^3x16 165 -> 145, 8^2x16^2 200 -> 198;
+// 12^3x24 would take 390 instead of 290.
+constexpr size_t kDirectBytes = 1 << 20, kDirectSites = 16384;
 }
 
 int Engine::gauge_force(const double2* U, double beta, double* action, double2* F, cudaStream_t st) {
     int rc = 0;
     const size_t V = 2 * (size_t)vh();
     const size_t nb = gauge_force_blocks(V);
-    double* part = (double*)get_ws("md.gpart", (nb + 1) * sizeof(double), &rc);
+    // flags, partials and their sum, and a byte per link, in one small allocation
+    const size_t pb = (nb + 1) * sizeof(double);
+    char* p = (char*)get_ws("md.gpart", sizeof(GaugeFlags) + pb + 4 * V, &rc);
     if (rc) return rc;
-    // the fixed-point kernel's limbs; a device too full for them runs the FP64 kernel
-    void* work = get_ws("md.glimbs", gauge_force_work(V), &rc);
+    double* part = (double*)(p + sizeof(GaugeFlags));
+    GaugeWork work{(GaugeFlags*)p, (unsigned char*)p + sizeof(GaugeFlags) + pb, nullptr};
+    // The limbs stay with the handle.  The first call on a middle lattice splits the links where they are used
+    // (the same bits) and allocates while its kernels run; so does every call on a device too full for the limbs.
+    int nomem = 0;
+    const size_t lb = gauge_limb_bytes(V);
+    const bool direct = lb > kDirectBytes && V <= kDirectSites && ws["md.glimbs"].bytes == 0;
+    if (!direct) work.limbs = get_ws("md.glimbs", lb, &nomem);
     {
         ProfScope ps("md.gauge_force", (double)V * 4 * (144 + (F ? 144 : 0)), st);  // U in, F out
         ODWF_CK(launch_gauge_force(lat.dims, U, work, beta, F, part, part + nb, st));
     }
+    if (direct) get_ws("md.glimbs", lb, &nomem);
     if (action) {
         double retr = 0.0;
         ODWF_CK(cudaMemcpyAsync(&retr, part + nb, sizeof(double), cudaMemcpyDeviceToHost, st));
