@@ -10,7 +10,7 @@
 // the last unit kept).  The result resolves 2^-57 of the largest component of the neighbour, four
 // bits beyond FP64's own rounding of it.  Components more than 2^kFxSpread below the largest of
 // their 5D site, non-finite values and denormals keep their FP64 bits instead (exponent kFxRaw);
-// sites that read such a neighbour take the FP64 arithmetic (fx_hop_slow), so nothing is lost on
+// warps that read such a neighbour take the FP64 arithmetic (fx_hop_f64), so nothing is lost on
 // fields of extreme range and NaN and Inf propagate as in FP64.  (Components below 2^-1042 beside
 // one above 2^-958 count as zero.)
 //
@@ -64,27 +64,6 @@ __device__ __forceinline__ double fx_to_double(long long q, int e) {
     const double d = __ll2double_rn(q);
     const int hi = __double2hiint(d);
     return __hiloint2double(hi == 0 ? 0 : hi + (e << 20), __double2loint(d));
-}
-
-__device__ __forceinline__ void fx_load_double(const void* base, const int* ex, size_t h, int s, int ns, double v[24]) {
-    const int4* p = reinterpret_cast<const int4*>(base);
-    const int e = __ldg(ex + h * ns + s);
-    int4 q[12];
-#pragma unroll
-    for (int k = 0; k < 12; ++k) q[k] = __ldg(p + chunk_off(h, k, 12, ns, s));
-    if (e == kFxRaw) {
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            v[2 * k] = __hiloint2double(q[k].x, q[k].y);
-            v[2 * k + 1] = __hiloint2double(q[k].z, q[k].w);
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            v[2 * k] = fx_to_double(fx_join(q[k].x, q[k].y), e);
-            v[2 * k + 1] = fx_to_double(fx_join(q[k].z, q[k].w), e);
-        }
-    }
 }
 
 // 64-bit accumulation of a 32 x 32-bit product (one instruction)

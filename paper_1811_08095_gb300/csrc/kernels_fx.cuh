@@ -299,31 +299,99 @@ __device__ __forceinline__ void fx_dir(const int4* __restrict__ up, const int4* 
     }
 }
 
-// The stencil in FP64 for one 5D site, for neighbours or links outside the fixed-point range
-static __device__ __noinline__ void fx_hop_slow(const HopParams<double>& P, const void* in, const int* ex, int h, int s,
-                                         bool dag, double* y) {
-    for (int k = 0; k < 24; ++k) y[k] = 0.0;
-    const int* nb = P.nbr + ((size_t)P.p_out * P.g.Vh + h) * 8;
-#pragma unroll 1
-    for (int j = 0; j < 8; ++j) {
-        const int raw = nb[j], mu = j >> 1, hn = checked_index(raw & 0x7fffffff, P.g.Vh, P.bounds_flag, kBoundsNeighbour);
-        double v[24], hp[12], u[18], w[12];
-        fx_load_double(in, ex, (size_t)hn, s, P.ns, v);
-        const double sg = ((j & 1) == 0) == dag ? 1.0 : -1.0;
-        project(mu, sg, v, hp);
-        const size_t idx = (j & 1) == 0 ? ((size_t)(P.p_out * 4 + mu) * P.g.Vh + h)
-                                        : ((size_t)((1 - P.p_out) * 4 + mu) * P.g.Vh + hn);
-        LinkIO<LinkD18, double>::load(P.links_d, idx, u);
-        su3_mul(u, hp, w, (j & 1) != 0);
-        if (raw < 0)
-            for (int k = 0; k < 12; ++k) w[k] = -w[k];
-        accumulate(mu, sg, w, y);
+// d with its sign bit flipped where `mask` has bit 31
+__device__ __forceinline__ double fx_flip(double d, unsigned mask) {
+    return __hiloint2double((int)((unsigned)__double2hiint(d) ^ mask), __double2loint(d));
+}
+
+// fx_dir in FP64: the neighbour's stored exponent e (or kFxRaw), U the FP64 link, taken adjoint for a backward
+// hop and negated where `minus`
+template <int MU, bool PLUS>
+__device__ __forceinline__ void fx_dir_f64(const int4* __restrict__ up, const int4* __restrict__ dn, int e, int ns,
+                                           const double2* __restrict__ U, bool back, bool minus, double acc[18]) {
+    double h[3][2];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const int4 u = __ldg(up + c * ns), d = __ldg(dn + c * ns);
+        double ur, ui, dr, di;
+        if (e == kFxRaw) {
+            ur = __hiloint2double(u.x, u.y);
+            ui = __hiloint2double(u.z, u.w);
+            dr = __hiloint2double(d.x, d.y);
+            di = __hiloint2double(d.z, d.w);
+        } else {
+            ur = fx_to_double(fx_join(u.x, u.y), e);
+            ui = fx_to_double(fx_join(u.z, u.w), e);
+            dr = fx_to_double(fx_join(d.x, d.y), e);
+            di = fx_to_double(fx_join(d.z, d.w), e);
+        }
+        constexpr bool nr = (MU == 1) == PLUS, ni = (MU == 3) != PLUS, turn = MU == 0 || MU == 2;  // as fx_dir
+        h[c][0] = nr ? ur - (turn ? di : dr) : ur + (turn ? di : dr);
+        h[c][1] = ni ? ui - (turn ? dr : di) : ui + (turn ? dr : di);
+    }
+    double* lower = acc + (MU < 2 ? 6 : 12);
+    const unsigned fr = minus ? 0x80000000u : 0u, fi = fr ^ (back ? 0x80000000u : 0u);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        double wr = 0.0, wi = 0.0;
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const double2 u = __ldg(U + (back ? 3 * b + i : 3 * i + b));
+            const double ur = fx_flip(u.x, fr), ui = fx_flip(u.y, fi);
+            wr = fma(ur, h[b][0], wr);
+            wr = fma(-ui, h[b][1], wr);
+            wi = fma(ur, h[b][1], wi);
+            wi = fma(ui, h[b][0], wi);
+        }
+        acc[2 * i] += wr;
+        acc[2 * i + 1] += wi;
+        if (MU == 0 || MU == 2) {
+            lower[2 * i] = PLUS ? lower[2 * i] - wi : lower[2 * i] + wi;
+            lower[2 * i + 1] = PLUS ? lower[2 * i + 1] + wr : lower[2 * i + 1] - wr;
+        } else {
+            constexpr bool n = (MU == 1) == PLUS;
+            lower[2 * i] = n ? lower[2 * i] - wr : lower[2 * i] + wr;
+            lower[2 * i + 1] = n ? lower[2 * i + 1] - wi : lower[2 * i + 1] + wi;
+        }
     }
 }
 
 // index of the link of direction j at site h (parity p_out) with neighbour hn
 __device__ __forceinline__ size_t fx_link_index(const HopParams<double>& P, int j, int h, int hn) {
     return (j & 1) ? (size_t)((1 - P.p_out) * 4 + (j >> 1)) * P.g.Vh + hn : (size_t)(P.p_out * 4 + (j >> 1)) * P.g.Vh + h;
+}
+
+// The stencil in FP64, for warps that meet a neighbour or a link outside the fixed-point range: half a 5D site per
+// thread as the fixed-point one, 530 FP64 operations each with the conversions.  A warp takes one of the two, so
+// that a field of which every site goes here (S^dag S on 16^3x32x16: 7.9 ms) is still faster than with FP64 hops
+// throughout (12.7; with whole 5D sites by one thread, behind the integer stencil: 20.4).  All lanes of the warp call.
+template <bool DAG>
+static __device__ __noinline__ void fx_hop_f64(const HopParams<double>& P, const int4* in, const int* ex, int h, int s, int a,
+                                               int partner, double* v) {
+    const int ns = P.ns, cross = (9 - 6 * a) * ns, same = 6 * ns;
+    const int* nb = P.nbr + ((size_t)P.p_out * P.g.Vh + h) * 8;
+    double acc[18];
+#pragma unroll
+    for (int k = 0; k < 18; ++k) acc[k] = 0.0;
+#define ODWF_FX_DIR64(MU_, DIR_)                                                                                     \
+    {                                                                                                                \
+        const int j_ = (MU_ == 1 || MU_ == 2) ? ((2 * MU_ + DIR_) ^ a) : 2 * MU_ + DIR_;                             \
+        const int raw_ = __ldg(nb + j_), n_ = checked_index(raw_ & 0x7fffffff, P.g.Vh, P.bounds_flag, kBoundsNeighbour); \
+        const int4* p_ = in + (size_t)n_ * (12 * ns);                                                                \
+        fx_dir_f64<MU_, (DIR_ == 0) == DAG>(p_, p_ + (MU_ < 2 ? cross : same), __ldg(ex + (size_t)n_ * ns + s), ns,   \
+                                            static_cast<const double2*>(P.links_d) + fx_link_index(P, j_, h, n_) * 9, \
+                                            j_ & 1, raw_ >= 0, acc);                                                 \
+    }
+    ODWF_FX_DIR64(0, 0) ODWF_FX_DIR64(0, 1)
+    ODWF_FX_DIR64(1, 0) ODWF_FX_DIR64(1, 1)
+    ODWF_FX_DIR64(2, 0) ODWF_FX_DIR64(2, 1)
+    ODWF_FX_DIR64(3, 0) ODWF_FX_DIR64(3, 1)
+#undef ODWF_FX_DIR64
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        v[k] = 0.5 * acc[k];
+        v[6 + k] = 0.5 * (acc[12 + k] + __shfl_xor_sync(0xffffffffu, acc[6 + k], partner));
+    }
 }
 
 template <int F>
@@ -393,10 +461,18 @@ __global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) hop_fx_kernel(const 
         M = max(M, e[j]);
     }
     __syncthreads();  // a site's threads may lie in two warps (Ns = 32)
-    long long acc[18];
+    double v[12];
+    slow = slow || ((M < kFxMinExp || M >= kFxMaxExp) && M > kFxZero / 2);
+    if (__any_sync(0xffffffffu, slow)) {
+        double y[12];
+        fx_hop_f64<DAG>(P, in, ex, h, s, a, t.partner, y);
 #pragma unroll
-    for (int k = 0; k < 18; ++k) acc[k] = 0;
-    const int cross = (9 - 6 * a) * ns, same = 6 * ns;  // from upper spin a to lower spin 1 - a, to lower spin a
+        for (int k = 0; k < 12; ++k) v[k] = y[k];
+    } else {
+        long long acc[18];
+#pragma unroll
+        for (int k = 0; k < 18; ++k) acc[k] = 0;
+        const int cross = (9 - 6 * a) * ns, same = 6 * ns;  // from upper spin a to lower spin 1 - a, to lower spin a
 #define ODWF_FX_DIR(MU_, DIR_)                                                                                      \
     {                                                                                                               \
         constexpr int j_ = 2 * MU_ + DIR_;                                                                          \
@@ -406,23 +482,17 @@ __global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) hop_fx_kernel(const 
         fx_dir<MU_, (DIR_ == 0) == DAG>(p_, p_ + (MU_ < 2 ? cross : same), ns,                                      \
                                         my_links + 9 * (swap_ ? (j_ ^ a) : j_), min(M - e_, 63), acc);              \
     }
-    ODWF_FX_DIR(0, 0) ODWF_FX_DIR(0, 1)
-    ODWF_FX_DIR(1, 0) ODWF_FX_DIR(1, 1)
-    ODWF_FX_DIR(2, 0) ODWF_FX_DIR(2, 1)
-    ODWF_FX_DIR(3, 0) ODWF_FX_DIR(3, 1)
+        ODWF_FX_DIR(0, 0) ODWF_FX_DIR(0, 1)
+        ODWF_FX_DIR(1, 0) ODWF_FX_DIR(1, 1)
+        ODWF_FX_DIR(2, 0) ODWF_FX_DIR(2, 1)
+        ODWF_FX_DIR(3, 0) ODWF_FX_DIR(3, 1)
 #undef ODWF_FX_DIR
-    // -1/2 W psi (or -1/2 W^dag psi) = acc 2^(M + 2) / 2, the lower spin with the other thread's part
-    double v[12];
+        // -1/2 W psi (or -1/2 W^dag psi) = acc 2^(M + 2) / 2, the lower spin with the other thread's part
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        v[k] = fx_to_double(acc[k], M + 1);
-        v[6 + k] = fx_to_double(acc[12 + k] + __shfl_xor_sync(0xffffffffu, acc[6 + k], t.partner), M + 1);
-    }
-    if (slow || ((M < kFxMinExp || M >= kFxMaxExp) && M > kFxZero / 2)) {
-        double y[24];
-        fx_hop_slow(P, P.in.d(sys), ex, h, s, DAG, y);
-#pragma unroll
-        for (int k = 0; k < 12; ++k) v[k] = -0.5 * (a ? y[6 + k + (k < 6 ? 0 : 6)] : y[k + (k < 6 ? 0 : 6)]);
+        for (int k = 0; k < 6; ++k) {
+            v[k] = fx_to_double(acc[k], M + 1);
+            v[6 + k] = fx_to_double(acc[12 + k] + __shfl_xor_sync(0xffffffffu, acc[6 + k], t.partner), M + 1);
+        }
     }
 
     // the links are read: their shared memory now holds the columns of fx_columns
