@@ -207,12 +207,18 @@ __device__ __forceinline__ void fx_store(void* base, int* ex, size_t h, const Fx
                                          const double v[12]) {
     const int s = t.s, a = t.a;
     int mx = 0;
-    unsigned mn = 0xffffffffu;  // smallest high word of a nonzero component, less one
+    unsigned mn = 0xffffffffu;  // smallest high word of a nonzero group (fx.cuh), less one
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        const int hi = __double2hiint(v[k]) & 0x7fffffff;
-        mx = max(mx, hi);
-        mn = min(mn, (unsigned)(hi - 1));
+    for (int c = 0; c < 3; ++c) {
+        int up = 0, dn = 0;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            up = max(up, __double2hiint(v[2 * c + k]) & 0x7fffffff);
+            dn = max(dn, __double2hiint(v[6 + 2 * c + k]) & 0x7fffffff);
+        }
+        const int other = __shfl_xor_sync(0xffffffffu, dn, t.partner);
+        mx = max(mx, max(up, dn));
+        mn = min(mn, min((unsigned)(max(up, dn) - 1), (unsigned)(max(up, other) - 1)));
     }
     mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, t.partner));
     mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, t.partner));
@@ -235,7 +241,7 @@ __device__ __forceinline__ void fx_store(void* base, int* ex, size_t h, const Fx
             q = make_int4(__double2hiint(v[2 * k]), __double2loint(v[2 * k]), __double2hiint(v[2 * k + 1]),
                           __double2loint(v[2 * k + 1]));
         } else {
-            const FxLimbs re = fx_split(fx_from_double<6>(v[2 * k], e)), im = fx_split(fx_from_double<6>(v[2 * k + 1], e));
+            const FxLimbs re = fx_round(v[2 * k], e), im = fx_round(v[2 * k + 1], e);
             q = make_int4(re.hi, re.lo, im.hi, im.lo);
         }
         p[fx_chunk(h, a, k / 3, k % 3, ns, s)] = q;
@@ -250,9 +256,11 @@ __device__ __forceinline__ void fx_store(void* base, int* ex, size_t h, const Fx
 // and w_a = U h_a returns to that lower spin with the conjugate factor.  Where the factor's sign differs
 // between the two threads of a site, thread 1 takes the opposite direction (whose sg has the other
 // sign), so both run the same code.  acc: upper spin a, lower spin 1 - a (mu 0, 1), lower spin a (mu 2, 3).
+// size: |w| of each colour, leading words (see kFxWeak), the real part of one direction and the imaginary part of
+// the other, so that neither real nor imaginary fields look small.
 template <int MU, bool PLUS>
 __device__ __forceinline__ void fx_dir(const int4* __restrict__ up, const int4* __restrict__ dn, int ns, const int4* U,
-                                       int sh, long long acc[18]) {
+                                       int sh, long long acc[18], unsigned size[3]) {
     FxLimbs h[3][2];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -287,6 +295,7 @@ __device__ __forceinline__ void fx_dir(const int4* __restrict__ up, const int4* 
         const long long wr = (A[0] + ((B[0] + C[0]) >> 31)) >> sh, wi = (A[1] + ((B[1] + C[1]) >> 31)) >> sh;
         acc[2 * i] += wr;
         acc[2 * i + 1] += wi;
+        size[i] += (unsigned)abs((int)((PLUS ? wr : wi) >> 32));
         // sg G^dag w: i w for mu 0, 2; -w for mu 1; w for mu 3
         if (MU == 0 || MU == 2) {
             lower[2 * i] = PLUS ? lower[2 * i] - wi : lower[2 * i] + wi;
@@ -361,7 +370,8 @@ __device__ __forceinline__ size_t fx_link_index(const HopParams<double>& P, int 
     return (j & 1) ? (size_t)((1 - P.p_out) * 4 + (j >> 1)) * P.g.Vh + hn : (size_t)(P.p_out * 4 + (j >> 1)) * P.g.Vh + h;
 }
 
-// The stencil in FP64, for warps that meet a neighbour or a link outside the fixed-point range: half a 5D site per
+// The stencil in FP64, for warps that meet a neighbour or a link outside the fixed-point range or whose sums
+// hold a small one: half a 5D site per
 // thread as the fixed-point one, 530 FP64 operations each with the conversions.  A warp takes one of the two, so
 // that a field of which every site goes here (S^dag S on 16^3x32x16: 7.9 ms) is still faster than with FP64 hops
 // throughout (12.7; with whole 5D sites by one thread, behind the integer stencil: 20.4).  All lanes of the warp call.
@@ -462,16 +472,14 @@ __global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) hop_fx_kernel(const 
     }
     __syncthreads();  // a site's threads may lie in two warps (Ns = 32)
     double v[12];
-    slow = slow || ((M < kFxMinExp || M >= kFxMaxExp) && M > kFxZero / 2);
-    if (__any_sync(0xffffffffu, slow)) {
-        double y[12];
-        fx_hop_f64<DAG>(P, in, ex, h, s, a, t.partner, y);
-#pragma unroll
-        for (int k = 0; k < 12; ++k) v[k] = y[k];
-    } else {
+    bool redo = __any_sync(0xffffffffu, slow || ((M < kFxMinExp || M >= kFxMaxExp) && M > kFxZero / 2));
+    if (!redo) {
         long long acc[18];
+        unsigned size[2][3];  // mu = 0, 1 and mu = 2, 3
 #pragma unroll
         for (int k = 0; k < 18; ++k) acc[k] = 0;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) size[k / 3][k % 3] = 0;
         const int cross = (9 - 6 * a) * ns, same = 6 * ns;  // from upper spin a to lower spin 1 - a, to lower spin a
 #define ODWF_FX_DIR(MU_, DIR_)                                                                                      \
     {                                                                                                               \
@@ -480,7 +488,7 @@ __global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) hop_fx_kernel(const 
         const int n_ = swap_ && a ? nb[j_ ^ 1] : nb[j_], e_ = swap_ && a ? e[j_ ^ 1] : e[j_];                       \
         const int4* p_ = in + (size_t)n_ * (12 * ns);                                                               \
         fx_dir<MU_, (DIR_ == 0) == DAG>(p_, p_ + (MU_ < 2 ? cross : same), ns,                                      \
-                                        my_links + 9 * (swap_ ? (j_ ^ a) : j_), min(M - e_, 63), acc);              \
+                                        my_links + 9 * (swap_ ? (j_ ^ a) : j_), min(M - e_, 63), acc, size[MU_ / 2]); \
     }
         ODWF_FX_DIR(0, 0) ODWF_FX_DIR(0, 1)
         ODWF_FX_DIR(1, 0) ODWF_FX_DIR(1, 1)
@@ -493,6 +501,19 @@ __global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) hop_fx_kernel(const 
             v[k] = fx_to_double(acc[k], M + 1);
             v[6 + k] = fx_to_double(acc[12 + k] + __shfl_xor_sync(0xffffffffu, acc[6 + k], t.partner), M + 1);
         }
+        unsigned least = 0xffffffffu;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const unsigned other = __shfl_xor_sync(0xffffffffu, size[0][c], t.partner);
+            least = min(least, size[1][c] + min(size[0][c], other));
+        }
+        redo = __any_sync(0xffffffffu, least < kFxWeak && M > kFxZero / 2);
+    }
+    if (redo) {
+        double y[12];
+        fx_hop_f64<DAG>(P, in, ex, h, s, a, t.partner, y);
+#pragma unroll
+        for (int k = 0; k < 12; ++k) v[k] = y[k];
     }
 
     // the links are read: their shared memory now holds the columns of fx_columns
