@@ -418,8 +418,10 @@ int odwf_md_trajectory(odwf_handle* h, void* U, void* P, int nterms, const void*
  * hops K1..K4 (see odwf_mixed_cg_step; K1 is the plain Dslash chi_t = B M^-1 (-1/2 W chi_p)),
  * 5 = the p update.  nsys systems (1..64) share the handle's links; every input field of every
  * system is filled from `fill` (an even-site field, host or device; any finite values) and
- * every system runs.  After one warm-up launch, `reps` launches are timed with two CUDA events
- * on `stream`; out receives the kernel class name, the launch counts, the total time and the
+ * every system runs.  After one warm-up pass, `reps` launches are timed with two CUDA events
+ * on `stream`, each with the sums over its iteration's block partials as the solver makes them:
+ * kind 3 forms alpha, kind 4 is followed by the launch that forms beta or, on small lattices, kinds
+ * 5 and 1 form it; out receives the kernel class name, the launch counts, the total time and the
  * algorithmic bytes (each field read or written once per system, links once per launch).
  * Results are meaningful as bandwidth when one system's fields exceed the L2 cache.
  * Allocates its workspaces on the handle (freed by odwf_destroy).

@@ -180,6 +180,7 @@ int BatchCG::init(Engine* e, int capacity, const odwf_solve_params& prm, cudaStr
             kbytes_launch[k] = k < 4 ? links : 0.0;
             pcls[k] = prof_class(kname[k], kbytes_sys[k], kbytes_launch[k]);
         }
+        pcls[5] = prof_class(p2 + ".beta_sum", 0.0, 8.0 * hop_blocks(E->ns, low, 4, E->vh(), 1));
     } else {
     pcls[0] = prof_class(pre + ".K1_minv", n5 * 2 * sp, links);
     pcls[1] = prof_class(pre + ".K2_schur_norm_mdinv", n5 * 3 * sp, links);
@@ -427,10 +428,9 @@ int BatchCG::launch_iterations(int k, int lo, int n, cudaStream_t s) {
     return ODWF_OK;
 }
 
-// The four hops K1..K4 of one second-generation mixed iteration over slots lo..lo+n-1 (the
-// non-dagger hops read chi = B psi): the launches the solver replays every iteration.
-int BatchCG::launch_v2_kernel(int kind, int lo, int n, cudaStream_t s) {
-    if (kind == 5) return launch_v2_pupdate(1, lo, n, 1, kRunning, s);
+// One of the hops K1..K4 of a second-generation mixed iteration over slots lo..lo+n-1 (the non-dagger hops
+// read chi = B psi).  K3 also forms alpha from K2's partials, K1 beta from nb_prev of K4's.
+int BatchCG::launch_v2_hop(int kind, int lo, int n, cudaStream_t s, int nb_prev) {
     auto P = params<float>(1);
     P.gate = 1;
     P.need_status = kRunning;
@@ -448,40 +448,38 @@ int BatchCG::launch_v2_kernel(int kind, int lo, int n, cudaStream_t s) {
         P.cg_x = Xin.ref();
         P.cg_p = Pl.ref();
     }
-    ODWF_CK(launch_hop_prod(P, kind, low, lk, n, s));
+    P.nb_prev = k == 2 ? hop_blocks(E->ns, low, 2, E->vh(), n) : k == 0 ? nb_prev : 0;
+    auto pb_ = prof_begin(pcls[k], s);
+    P.prof_count = pb_.dev_count;
+    const cudaError_t e_ = launch_hop_prod(P, kind, low, lk, n, s);
+    prof_end(pb_, s);
+    ODWF_CK(e_);
     return ODWF_OK;
 }
 
-int BatchCG::launch_v2_hops(int lo, int n, cudaStream_t s, bool prev_beta, bool last_beta) {
-    auto P = params<float>(1);
-    P.gate = 1;
-    P.need_status = kRunning;
-    P.sys_base = lo;
-    const FieldRef ins[4] = {Chil.ref(), Tl.ref(), Al.ref(), Cl.ref()};
-    const FieldRef outs[4] = {Tl.ref(), Al.ref(), Cl.ref(), FieldRef{}};
-    const FieldRef zs[4] = {FieldRef{}, Pl.ref(), FieldRef{}, Al.ref()};
-    for (int k = 0; k < 4; ++k) {
-        P.p_out = (k & 1) ? 0 : 1;
-        P.in = ins[k];
-        P.out = outs[k];
-        P.z = zs[k];
-        if (k == 3) {
-            P.cg_r = Rin.ref();
-            P.cg_x = Xin.ref();
-            P.cg_p = Pl.ref();
-        }
-        // K3 also forms alpha from K2's partials, K1 beta from the last K4's
-        P.nb_prev = k == 2 ? hop_blocks(E->ns, low, 2, E->vh(), n)
-                  : k == 0 && prev_beta ? hop_blocks(E->ns, low, 4, E->vh(), n) : 0;
-        auto pb_ = prof_begin(pcls[k], s);
-        P.prof_count = pb_.dev_count;
-        const cudaError_t e_ = launch_hop_prod(P, k + 1, low, lk, n, s);
-        prof_end(pb_, s);
-        P.prof_count = nullptr;
-        ODWF_CK(e_);
-    }
-    if (last_beta) ODWF_CK(launch_beta(partials, hop_blocks(E->ns, low, 4, E->vh(), n), nblk, st, kRunning, lo, n, s));
+// beta of every running system from K4's partials
+int BatchCG::launch_v2_beta(int lo, int n, cudaStream_t s) {
+    auto pb_ = prof_begin(pcls[5], s);
+    const cudaError_t e_ = launch_beta(partials, hop_blocks(E->ns, low, 4, E->vh(), n), nblk, st, kRunning, lo, n, s);
+    prof_end(pb_, s);
+    ODWF_CK(e_);
     return ODWF_OK;
+}
+
+// A kernel of the iteration as the solver replays it, with the sums over partials that it or a launch of its own makes
+int BatchCG::launch_v2_kernel(int kind, int lo, int n, cudaStream_t s) {
+    const int nb = hop_blocks(E->ns, low, 4, E->vh(), n);
+    const bool in_update = nb * n <= kBetaInUpdate;
+    if (kind == 5) return launch_v2_pupdate(1, lo, n, 1, kRunning, s, in_update ? nb : 0);
+    const int rc = launch_v2_hop(kind, lo, n, s, in_update ? nb : 0);
+    return rc || kind != 4 || in_update ? rc : launch_v2_beta(lo, n, s);
+}
+
+int BatchCG::launch_v2_hops(int lo, int n, cudaStream_t s, bool prev_beta, bool last_beta) {
+    const int nb = prev_beta ? hop_blocks(E->ns, low, 4, E->vh(), n) : 0;
+    for (int kind = 1; kind <= 4; ++kind)
+        if (const int rc = launch_v2_hop(kind, lo, n, s, nb)) return rc;
+    return last_beta ? launch_v2_beta(lo, n, s) : ODWF_OK;
 }
 
 // p = r + beta p (mode 1) or p = r (mode 0), chi_p = B p, for the slots whose status is `need`.

@@ -81,7 +81,7 @@ struct BatchCG {
     CgHost* H = nullptr;
     std::unique_ptr<CgHost> own;   // when the engine's is in use
     bool idle = true;              // nothing of this batch is in flight on the iteration stream
-    int pcls[5] = {-1, -1, -1, -1, -1};  // profiler classes: K1..K4, p update
+    int pcls[6] = {-1, -1, -1, -1, -1, -1};  // profiler classes: K1..K4, p update, beta's sum
     std::string kname[5];                 // (second-generation kernels) class names and
     double kbytes_sys[5] = {0}, kbytes_launch[5] = {0};  // algorithmic bytes per system / launch
     int pcls_rel[4] = {-1, -1, -1, -1};  // FP64 residual hops of the reliable update
@@ -112,6 +112,8 @@ struct BatchCG {
     // nb > 0: the update forms beta from the nb partials of K4
     int launch_v2_pupdate(int mode, int lo, int n, int gate, int need, cudaStream_t s, int nb = 0);
     int launch_v2_kernel(int kind, int lo, int n, cudaStream_t s);  // kind 1..4: K1..K4 alone, 5: P
+    int launch_v2_hop(int kind, int lo, int n, cudaStream_t s, int nb_prev);
+    int launch_v2_beta(int lo, int n, cudaStream_t s);
     // write a slot's scalars (and r = m_q / (2 m0)) directly; synchronizes s
     int set_state(int slot, const SysState& init, double r, cudaStream_t s);
     bool slot_running(int i) const;

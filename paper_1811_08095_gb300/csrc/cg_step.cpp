@@ -159,6 +159,15 @@ int Engine::time_kernel(int kind, int prec, int recon, int link_prec, int nsys, 
         ODWF_CK(launch_pack(Sp::F32, fd, bc.Xin.ref_sys(i), g, 0, ns, 1, st));
         if ((rc = bc.set_state(i, s0, mq / (2.0 * m0), st))) return rc;
     }
+    // the four hops leave the partials that the timed kernel may sum; with rr = 2 |r|^2 beta is 1/2
+    if ((rc = bc.launch_v2_hops(0, nsys, st))) return rc;
+    ODWF_CK(cudaMemcpyAsync(bc.st_host, bc.st, sizeof(SysState) * nsys, cudaMemcpyDeviceToHost, st));
+    ODWF_CK(cudaStreamSynchronize(st));
+    for (int i = 0; i < nsys; ++i) {
+        const double rr = bc.st_host[i].rr_new;
+        s0.rr = rr > 0.0 && std::isfinite(rr) ? 2.0 * rr : 1.0;
+        if ((rc = bc.set_state(i, s0, mq / (2.0 * m0), st))) return rc;
+    }
     if ((rc = bc.launch_v2_kernel(kind, 0, nsys, st))) return rc;  // warm-up launch
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     ODWF_CK(cudaEventCreate(&e0));
