@@ -40,6 +40,9 @@ __global__ void __launch_bounds__(DEEP ? kBS2Deep : kBS2, DEEP ? 4 : 3) hop2_ker
     constexpr int kSL = 8 * kLS + 4;   // floats per site (padding spreads banks)
     constexpr bool DAG = (KIND == K3 || KIND == K4);
     const int sys = blockIdx.y + P.sys_base;
+    // In K1 and K3 the extra block below may park this system while other warps read its status here (one load
+    // per warp), and either value will do: these kernels use nothing else that it writes, have no block barrier, and
+    // their output is not read once the system is parked (the launches behind find it so).
     if (P.gate && P.st[sys].status != P.need_status) return;
     if (P.prof_count && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(P.prof_count, 1ull);
 

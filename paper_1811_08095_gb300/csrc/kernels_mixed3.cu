@@ -213,6 +213,7 @@ __global__ void __launch_bounds__(kBS3, hop3_min_blocks<KIND>()) hop3_kernel(con
     static_assert(KIND == K1 || KIND == K2 || KIND == K3, "hop3 implements the hops K1, K2 and K3");
     constexpr bool DAG = (KIND == K3);
     const int sys = blockIdx.y + P.sys_base;
+    // K1, K3: read beside the extra block's write, see hop2_kernel
     if (P.gate && P.st[sys].status != P.need_status) return;
     if (P.prof_count && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(P.prof_count, 1ull);
 
