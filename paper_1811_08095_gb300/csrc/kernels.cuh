@@ -78,7 +78,6 @@ struct HopParams {
     int ns;
     int lg_ns;
     int p_out;           // parity of the output sites
-    int preshifted;      // non-dagger hops: `in` already holds chi = B psi (skip B per neighbour)
     FieldRef in, z, out;
     FieldRef cg_r, cg_x, cg_p;  // F_CG: r and x (accumulator format), p (input format)
     FieldRef b;                 // F_RESID: right-hand side (accumulator format)
@@ -409,7 +408,7 @@ __global__ void __launch_bounds__(256) hop_kernel(const HopParams<R> P) {
 #pragma unroll
                 for (int k = 0; k < 24; ++k) v[k] = 0;
             }
-            if (!DAG && !P.preshifted) bidiag_apply(v, P.cf.rho[s], P.cf.sigma[s], r, s, ns, false);  // chi = B psi
+            if (!DAG) bidiag_apply(v, P.cf.rho[s], P.cf.sigma[s], r, s, ns, false);  // chi = B psi
 
             // forward hop uses (1 - gamma) for D and (1 + gamma) for D^dag; backward the opposite
             const R sg = DAG ? (dir == 0 ? (R)1 : (R)-1) : (dir == 0 ? (R)-1 : (R)1);
