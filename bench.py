@@ -209,9 +209,7 @@ def ncu_traffic(kernel_class):
     return None
 
 
-def update_arith_name(updates):
-    """The reliable-update arithmetic of a mixed solve: every setting runs the same operator."""
-    return "FP64-accurate fixed point"
+UPDATE_ARITH = "FP64-accurate fixed point"  # every --updates setting runs the same operator
 
 
 def aggregate(t_local_s: float, solves_local: int, dist=None, device=None):
@@ -494,7 +492,7 @@ def run_ours(args, world, rank, local):
                        "omega": "shifted (R5) Zolotarev on [0.05, 6.2]", "tol": TOL,
                        "precision": "%s storage (per-site FP32 scale), FP32 links (%d reals), FP32 arithmetic, "
                                     "%s reliable updates (delta %g), FP64 reductions" % (
-                                        args.prec, args.link_recon, update_arith_name(args.updates),
+                                        args.prec, args.link_recon, UPDATE_ARITH,
                                         args.delta),
                        "solver": "batched even-odd CG on S^dag S, 3 systems per launch",
                        "l2": "flushed between steps (512 MB write); per-system working set > 1 GB",
@@ -801,7 +799,7 @@ def run_hmc(args, world, rank, local):
             "value": round(value, 4), "unit": "MD steps/s", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": round(ms_avg, 2), "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "%s solves (%s reliable updates), FP64 forces and MD updates" % (
-                args.prec, update_arith_name(args.updates)), "data": "synthetic",
+                args.prec, UPDATE_ARITH), "data": "synthetic",
             "config": {"workload": HMC_WORKLOAD, "lattice": "16^3x32", "Ns": ns, "m0": M0, "beta": HMC_BETA,
                        "mass_chain": list(HMC_CHAIN), "tau": HMC_TAU, "md_steps_per_bench_step": HMC_NSTEPS,
                        "integrator": "Omelyan, Sexton-Weingarten with %d gauge steps per outer drift" % HMC_INNER,
@@ -1029,7 +1027,7 @@ def run_batched_c3(args, world, rank, local):
             "config": {"lattice": "24^3x48", "Ns": NS, "m0": M0, "masses": list(MASSES),
                        "sources": "12 spin-colour point sources at even site %s, wall placement" % (site,),
                        "gauge": "U = exp(0.25 i H) (seed 3)", "prec": args.prec, "link_recon": args.link_recon,
-                       "delta": args.delta, "updates": update_arith_name(args.updates), "tol": TOL,
+                       "delta": args.delta, "updates": UPDATE_ARITH, "tol": TOL,
                        "omega": "shifted (R5) Zolotarev on [0.05, 6.2]"}}
     print(json.dumps(line), flush=True)
     h.close()
@@ -1086,7 +1084,7 @@ def run_paper_scale_c5(args, world, rank, local):
             "device_memory": {"used_gb": round((total - free) / 1e9, 2), "total_gb": round(total / 1e9, 2)},
             "config": {"lattice": "64^4", "Ns": NS, "m0": M0, "mq": mq, "gauge": "U = exp(0.2 i H) (seed 5)",
                        "links": "FP32, 12 reals", "prec": prec, "delta": args.delta,
-                       "updates": update_arith_name(args.updates), "tol": TOL,
+                       "updates": UPDATE_ARITH, "tol": TOL,
                        "rhs": "unit Gaussian (torch seed 5)"}}
     print(json.dumps(line), flush=True)
     h.close()
@@ -1229,7 +1227,7 @@ def main():
     ap.add_argument("--delta", type=float, default=0.01, help="reliable-update threshold")
     ap.add_argument("--link-recon", type=int, default=12, choices=[12, 18])
     ap.add_argument("--updates", default="auto", choices=["auto", "f64", "ff"],
-                    help="arithmetic of the reliable updates (auto: the library's choice)")
+                    help="arithmetic of the reliable updates; the settings are kept for callers and run the same operator")
     ap.add_argument("--check-every", type=int, default=8, help="iterations between host polls of the solver state")
     ap.add_argument("--workload", default="c2", choices=["c2", "c3", "c5", "serve", "profile", "mres", "dslash", "flow", "hmc"],
                     help="c2: the default line; c3: 36-system batch on 24^3x48; c5: one 64^4 solve; serve; "
