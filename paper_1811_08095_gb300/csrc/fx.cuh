@@ -15,26 +15,27 @@
 // arithmetic:
 //   * a term of the stencil adds an upper and a lower spin of one colour.  A 5D site where the larger
 //     of such a pair is more than 2^kFxSpread below the largest component of the site, for any of the twelve pairs
-//     (two upper spins, two lower spins, three colours), keeps its FP64 bits (exponent kFxRaw).  A pair that
+//     (two upper spins, two lower spins, three colours), keeps its FP64 bits (exponent + kFxRaw).  A pair that
 //     is stored in fixed point resolves 2^-52 of itself or better.  One chirality alone may be smaller, as it is on
-//     the domain walls.  Share of 5D sites that keep their FP64 bits at kFxSpread = 6 / 7 / 8, 16^3x32x16,
-//     m_q = 0.002: solution for a Gaussian source 5e-6 / 0 / 0, for a point source 5e-3 / 5e-4 / 5e-5; S^dag S of a
-//     Gaussian field 2.01 ms at 6 and 1.97 at 7.
+//     the domain walls.  Warps that read FP64 bits convert them (fx_hop_conv): nothing is lost for the next test.
+//     Share of such 5D sites at kFxSpread = 6 / 7 / 8, 16^3x32x16, m_q = 0.002: solution for a Gaussian source
+//     5e-6 / 0 / 0, for a point source 5e-3 / 5e-4 / 5e-5.  On diagonal links a colour 2^-7 below the others errs by
+//     1.1e-16 of itself at 7, as in FP64, and by 1.4e-16 at 8.
 //   * the stencil adds up |w| of its terms for each complex component.  A sum of leading words below kFxWeak,
 //     3/32 to 3/16 of the largest neighbour component, or twice that beside links with an entry of
 //     modulus 1, means that the component is made of small terms only (links that do not mix colours, a large
-//     neighbour in other spins).  Above it the stencil errs by 2^-51.6 (rms) of the component's terms or less, as
-//     FP64 does.  In a Gaussian field the sum is 10 to 20 times that line; S^dag S takes 1.5% longer for the sums.
+//     neighbour in other spins), and the warp repeats the stencil in FP64 (fx_hop_f64).  Above it the stencil errs
+//     by 2^-51.6 (rms) of the component's terms or less, as FP64 does.  In a Gaussian field the sum is 10 to 20 times
+//     that line; S^dag S takes 1.5% longer for the sums.
 // Measured against extended precision, the error of a component is that of the FP64 hops or below for links from
 // 1 to exp(0.7 i H), for fields that fall by e^-0.7 per s and per chirality or by e^-1.2 per site, and for a colour
 // 1 to 2^-30 of the others on diagonal links (1.1e-16 rms at every ratio, FP64 1.1e-16; without the tests 8e-16 at
 // 2^-7 and 4e-10 at 2^-30).
-// Non-finite values and denormals keep their FP64 bits too.  Warps that read such a neighbour, or find such a sum, take
-// the FP64 stencil (fx_hop_f64), so NaN and Inf propagate as in FP64.  (Components below 2^-1042 beside one above
-// 2^-958 count as zero.)
+// Non-finite values, denormals and sums near the ends of the exponent range take the FP64 stencil at once (exponent
+// kFxHard), so NaN and Inf propagate as in FP64.  (Components below 2^-1042 beside one above 2^-958 count as zero.)
 //
 // A link array holds nine (re1, re0, im1, im0) records per link, rows first, in the order of the FP64
-// links ((p * 4 + mu) * Vh + h), and one exponent each behind them (kFxRaw: a non-finite link).
+// links ((p * 4 + mu) * Vh + h), and one exponent each behind them (kFxHard: a non-finite link).
 //
 // Storage of a field: the 16-byte chunks of the FP64 layout (SpF64), each a complex number as
 // (re1, re0, im1, im0), and one int32 exponent per 5D site at ex[h * Ns + s].  Limbs of a sum of two
@@ -45,7 +46,9 @@
 
 namespace odwf {
 
-constexpr int kFxRaw = 1 << 28;      // exponent marking FP64 bits
+constexpr int kFxRaw = 1 << 28;      // added to the exponent of a site that keeps its FP64 bits
+constexpr int kFxHard = 1 << 29;     // exponent of one that only FP64 arithmetic can take
+constexpr int kFxBias = 1081;        // 1023 + 52 + 6: exponent of a site from its largest component's exponent field
 constexpr int kFxZero = -(1 << 24);  // exponent of an all-zero site (never the largest)
 constexpr int kFxSpread = 7;         // largest exponent range of a site's nonzero pairs of spins
 constexpr unsigned kFxWeak = 3u << 20;  // smallest sum of |w|, high words of the stencil's 64-bit terms
@@ -89,6 +92,13 @@ __device__ __forceinline__ FxLimbs fx_round(double d, int emax) {
     l.hi = (int)((p + (1ll << 31)) >> 32);
     return l;
 }
+
+// a complex number in FP64 bits into limbs
+__device__ __forceinline__ int4 fx_convert(int4 q, int emax) {
+    const FxLimbs re = fx_round(__hiloint2double(q.x, q.y), emax), im = fx_round(__hiloint2double(q.z, q.w), emax);
+    return make_int4(re.hi, re.lo, im.hi, im.lo);
+}
+__device__ __forceinline__ bool fx_is_raw(int e) { return e >= kFxRaw / 2; }
 
 __device__ __forceinline__ long long fx_join(int hi, int lo) { return ((long long)hi << 31) + lo; }
 

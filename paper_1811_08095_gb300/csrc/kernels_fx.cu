@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(128) links_fx_kernel(const double2* __restrict
         const FxLimbs re = fx_split(q[2 * k] >> more), im = fx_split(q[2 * k + 1] >> more);
         out[i * 9 + k] = make_int4(re.hi, re.lo, im.hi, im.lo);
     }
-    ex[i] = raw ? kFxRaw : emax < kFxMinField ? kFxZero : emax - 1022 + more;
+    ex[i] = raw ? kFxHard : emax < kFxMinField ? kFxZero : emax - 1022 + more;
 }
 
 cudaError_t launch_links_fx(const void* d18, void* fx, size_t n_links, cudaStream_t st) {

@@ -198,8 +198,8 @@ __device__ __forceinline__ void fx_load_fx(const void* base, const int* ex, size
     for (int k = 0; k < 6; ++k) q[k] = __ldg(p + fx_chunk(h, a, k / 3, k % 3, ns, s));
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-        v[2 * k] = e == kFxRaw ? __hiloint2double(q[k].x, q[k].y) : fx_to_double(fx_join(q[k].x, q[k].y), e);
-        v[2 * k + 1] = e == kFxRaw ? __hiloint2double(q[k].z, q[k].w) : fx_to_double(fx_join(q[k].z, q[k].w), e);
+        v[2 * k] = fx_is_raw(e) ? __hiloint2double(q[k].x, q[k].y) : fx_to_double(fx_join(q[k].x, q[k].y), e);
+        v[2 * k + 1] = fx_is_raw(e) ? __hiloint2double(q[k].z, q[k].w) : fx_to_double(fx_join(q[k].z, q[k].w), e);
     }
 }
 // Both threads of a 5D site call; `valid` is the same for both.
@@ -223,7 +223,7 @@ __device__ __forceinline__ void fx_store(void* base, int* ex, size_t h, const Fx
     mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, t.partner));
     mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, t.partner));
     const int emax = mx >> 20, emin = (int)((mn + 1) >> 20);
-    const bool odd = emax == 0x7ff || emax < kFxMinField || (mn != 0xffffffffu && emax - emin > kFxSpread);
+    const bool wide = mn != 0xffffffffu && emax - emin > kFxSpread, odd = emax == 0x7ff || emax < kFxMinField;
     bool zero = false;
     if (__any_sync(0xffffffffu, odd)) {
         zero = odd;
@@ -232,7 +232,7 @@ __device__ __forceinline__ void fx_store(void* base, int* ex, size_t h, const Fx
     }
     if (!valid) return;
     int4* p = reinterpret_cast<int4*>(base);
-    const bool raw = odd && !zero;
+    const bool hard = odd && !zero, raw = hard || (wide && !zero);
     const int e = zero ? 2046 : emax;  // an all-zero site: every significand shifted out
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
@@ -246,7 +246,7 @@ __device__ __forceinline__ void fx_store(void* base, int* ex, size_t h, const Fx
         }
         p[fx_chunk(h, a, k / 3, k % 3, ns, s)] = q;
     }
-    if (a == 0) ex[h * ns + s] = raw ? kFxRaw : zero ? kFxZero : emax - 1081;  // 1023 + 52 + 6
+    if (a == 0) ex[h * ns + s] = hard ? kFxHard : zero ? kFxZero : emax - kFxBias + (raw ? kFxRaw : 0);
 }
 
 // ---------------------------------------------------------------- the stencil
@@ -258,13 +258,18 @@ __device__ __forceinline__ void fx_store(void* base, int* ex, size_t h, const Fx
 // sign), so both run the same code.  acc: upper spin a, lower spin 1 - a (mu 0, 1), lower spin a (mu 2, 3).
 // size: |w| of each colour, leading words (see kFxWeak), the real part of one direction and the imaginary part of
 // the other, so that neither real nor imaginary fields look small.
-template <int MU, bool PLUS>
+// CONV: a neighbour with en >= kFxRaw / 2 holds FP64 bits.
+template <int MU, bool PLUS, bool CONV>
 __device__ __forceinline__ void fx_dir(const int4* __restrict__ up, const int4* __restrict__ dn, int ns, const int4* U,
-                                       int sh, long long acc[18], unsigned size[3]) {
+                                       int sh, long long acc[18], unsigned size[3], int en = 0) {
     FxLimbs h[3][2];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const int4 u = __ldg(up + c * ns), d = __ldg(dn + c * ns);
+        int4 u = __ldg(up + c * ns), d = __ldg(dn + c * ns);
+        if (CONV && fx_is_raw(en)) {
+            u = fx_convert(u, en - kFxRaw + kFxBias);
+            d = fx_convert(d, en - kFxRaw + kFxBias);
+        }
         // G d as (re, im): -i d = (im, -re) for mu 0, 2; -d for mu 1; d for mu 3
         const FxLimbs gr = (MU == 0 || MU == 2) ? FxLimbs{d.z, d.w} : FxLimbs{d.x, d.y};
         const FxLimbs gi = (MU == 0 || MU == 2) ? FxLimbs{d.x, d.y} : FxLimbs{d.z, d.w};
@@ -313,7 +318,7 @@ __device__ __forceinline__ double fx_flip(double d, unsigned mask) {
     return __hiloint2double((int)((unsigned)__double2hiint(d) ^ mask), __double2loint(d));
 }
 
-// fx_dir in FP64: the neighbour's stored exponent e (or kFxRaw), U the FP64 link, taken adjoint for a backward
+// fx_dir in FP64: the neighbour's stored exponent e, U the FP64 link, taken adjoint for a backward
 // hop and negated where `minus`
 template <int MU, bool PLUS>
 __device__ __forceinline__ void fx_dir_f64(const int4* __restrict__ up, const int4* __restrict__ dn, int e, int ns,
@@ -323,7 +328,7 @@ __device__ __forceinline__ void fx_dir_f64(const int4* __restrict__ up, const in
     for (int c = 0; c < 3; ++c) {
         const int4 u = __ldg(up + c * ns), d = __ldg(dn + c * ns);
         double ur, ui, dr, di;
-        if (e == kFxRaw) {
+        if (fx_is_raw(e)) {
             ur = __hiloint2double(u.x, u.y);
             ui = __hiloint2double(u.z, u.w);
             dr = __hiloint2double(d.x, d.y);
@@ -370,11 +375,46 @@ __device__ __forceinline__ size_t fx_link_index(const HopParams<double>& P, int 
     return (j & 1) ? (size_t)((1 - P.p_out) * 4 + (j >> 1)) * P.g.Vh + hn : (size_t)(P.p_out * 4 + (j >> 1)) * P.g.Vh + h;
 }
 
+// The fixed-point stencil for warps that meet neighbours with FP64 bits: those are converted where they are read.
+// Such sites are rare in most fields, and a warp that went to the FP64 stencil for one finished 4 us after the
+// others, which a small launch waits for: FP64 CG on 8^3x16x8 52.3 -> 49.8 ms, S^dag S on 16^3x32x16 of a field
+// with one colour 1e-15 of the others on rough links 3.8 -> 2.5 ms.
+template <bool DAG>
+static __device__ __noinline__ void fx_hop_conv(const HopParams<double>& P, const int4* in, const int* ex, int h, int s, int a,
+                                                const int4* my_links, int M, long long* acc_out, unsigned* size_out) {
+    const int ns = P.ns, cross = (9 - 6 * a) * ns, same = 6 * ns;
+    const int* nb = P.nbr + ((size_t)P.p_out * P.g.Vh + h) * 8;
+    long long acc[18];
+    unsigned size[2][3];
+#pragma unroll
+    for (int k = 0; k < 18; ++k) acc[k] = 0;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) size[k / 3][k % 3] = 0;
+#define ODWF_FX_DIRC(MU_, DIR_)                                                                                      \
+    {                                                                                                                \
+        const int j_ = (MU_ == 1 || MU_ == 2) ? ((2 * MU_ + DIR_) ^ a) : 2 * MU_ + DIR_;                             \
+        const int n_ = checked_index(__ldg(nb + j_) & 0x7fffffff, P.g.Vh, P.bounds_flag, kBoundsNeighbour);          \
+        const int en_ = __ldg(ex + (size_t)n_ * ns + s), eu_ = __ldg(P.link_ex + fx_link_index(P, j_, h, n_));       \
+        const int4* p_ = in + (size_t)n_ * (12 * ns);                                                                \
+        fx_dir<MU_, (DIR_ == 0) == DAG, true>(p_, p_ + (MU_ < 2 ? cross : same), ns, my_links + 9 * j_,               \
+                                              min(M - (en_ - (fx_is_raw(en_) ? kFxRaw : 0) + eu_), 63), acc,         \
+                                              size[MU_ / 2], en_);                                                   \
+    }
+    ODWF_FX_DIRC(0, 0) ODWF_FX_DIRC(0, 1)
+    ODWF_FX_DIRC(1, 0) ODWF_FX_DIRC(1, 1)
+    ODWF_FX_DIRC(2, 0) ODWF_FX_DIRC(2, 1)
+    ODWF_FX_DIRC(3, 0) ODWF_FX_DIRC(3, 1)
+#undef ODWF_FX_DIRC
+#pragma unroll
+    for (int k = 0; k < 18; ++k) acc_out[k] = acc[k];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) size_out[k] = size[k / 3][k % 3];
+}
+
 // The stencil in FP64, for warps that meet a neighbour or a link outside the fixed-point range or whose sums
-// hold a small one: half a 5D site per
-// thread as the fixed-point one, 530 FP64 operations each with the conversions.  A warp takes one of the two, so
-// that a field of which every site goes here (S^dag S on 16^3x32x16: 7.9 ms) is still faster than with FP64 hops
-// throughout (12.7; with whole 5D sites by one thread, behind the integer stencil: 20.4).  All lanes of the warp call.
+// hold a small one: half a 5D site per thread as the fixed-point one, 530 FP64 operations each with the
+// conversions.  S^dag S on 16^3x32x16: fields of which every warp runs both stencils 8.7 ms (a small colour) or 9.8
+// (a zero colour on unit links), FP64 hops throughout 12.7, others 1.97.  All lanes of the warp call.
 template <bool DAG>
 static __device__ __noinline__ void fx_hop_f64(const HopParams<double>& P, const int4* in, const int* ex, int h, int s, int a,
                                                int partner, double* v) {
@@ -462,12 +502,13 @@ __global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) hop_fx_kernel(const 
     const int4* in = reinterpret_cast<const int4*>(P.in.d(sys)) + chunk_slot(s, ns) + 3 * a * ns;
     const int* ex = reinterpret_cast<const int*>(P.in.n(sys));
     int e[8], M = kFxZero;
-    bool slow = false;
+    bool slow = false, conv = false;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         const int en = __ldg(ex + (size_t)nb[j] * ns + s), eu = __ldg(P.link_ex + fx_link_index(P, j, h, nb[j]));
-        slow |= en == kFxRaw || eu == kFxRaw;
-        e[j] = en + eu;
+        slow |= max(en, eu) >= kFxHard;
+        conv |= fx_is_raw(en);
+        e[j] = en - (fx_is_raw(en) ? kFxRaw : 0) + eu;
         M = max(M, e[j]);
     }
     __syncthreads();  // a site's threads may lie in two warps (Ns = 32)
@@ -480,21 +521,32 @@ __global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) hop_fx_kernel(const 
         for (int k = 0; k < 18; ++k) acc[k] = 0;
 #pragma unroll
         for (int k = 0; k < 6; ++k) size[k / 3][k % 3] = 0;
-        const int cross = (9 - 6 * a) * ns, same = 6 * ns;  // from upper spin a to lower spin 1 - a, to lower spin a
+        if (__any_sync(0xffffffffu, conv)) {
+            long long t_acc[18];
+            unsigned t_size[6];
+            fx_hop_conv<DAG>(P, in, ex, h, s, a, my_links, M, t_acc, t_size);
+#pragma unroll
+            for (int k = 0; k < 18; ++k) acc[k] = t_acc[k];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) size[k / 3][k % 3] = t_size[k];
+        } else {
+            const int cross = (9 - 6 * a) * ns, same = 6 * ns;  // from upper spin a to lower spin 1 - a, to lower spin a
 #define ODWF_FX_DIR(MU_, DIR_)                                                                                      \
     {                                                                                                               \
         constexpr int j_ = 2 * MU_ + DIR_;                                                                          \
         constexpr bool swap_ = MU_ == 1 || MU_ == 2; /* thread 1 takes the opposite direction */                    \
         const int n_ = swap_ && a ? nb[j_ ^ 1] : nb[j_], e_ = swap_ && a ? e[j_ ^ 1] : e[j_];                       \
         const int4* p_ = in + (size_t)n_ * (12 * ns);                                                               \
-        fx_dir<MU_, (DIR_ == 0) == DAG>(p_, p_ + (MU_ < 2 ? cross : same), ns,                                      \
-                                        my_links + 9 * (swap_ ? (j_ ^ a) : j_), min(M - e_, 63), acc, size[MU_ / 2]); \
+        fx_dir<MU_, (DIR_ == 0) == DAG, false>(p_, p_ + (MU_ < 2 ? cross : same), ns,                               \
+                                               my_links + 9 * (swap_ ? (j_ ^ a) : j_), min(M - e_, 63), acc,        \
+                                               size[MU_ / 2]);                                                      \
     }
-        ODWF_FX_DIR(0, 0) ODWF_FX_DIR(0, 1)
-        ODWF_FX_DIR(1, 0) ODWF_FX_DIR(1, 1)
-        ODWF_FX_DIR(2, 0) ODWF_FX_DIR(2, 1)
-        ODWF_FX_DIR(3, 0) ODWF_FX_DIR(3, 1)
+            ODWF_FX_DIR(0, 0) ODWF_FX_DIR(0, 1)
+            ODWF_FX_DIR(1, 0) ODWF_FX_DIR(1, 1)
+            ODWF_FX_DIR(2, 0) ODWF_FX_DIR(2, 1)
+            ODWF_FX_DIR(3, 0) ODWF_FX_DIR(3, 1)
 #undef ODWF_FX_DIR
+        }
         // -1/2 W psi (or -1/2 W^dag psi) = acc 2^(M + 2) / 2, the lower spin with the other thread's part
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
