@@ -70,8 +70,9 @@ enum {
 };
 
 /* ODWF_FF (odwf_apply_normal_prec only): the operator of the mixed-precision CG's reliable updates.
- * It is the FP64 operator: its stencil runs in block fixed point on the integer pipe, which resolves
- * more than FP64 and is faster on this GPU than FP64 or pairs of FP32 (the name's origin). */
+ * It is the FP64 operator: its stencil runs in block fixed point on the integer pipe, which is faster
+ * on this GPU than FP64 or pairs of FP32 (the name's origin), and in FP64 where fixed point would lose
+ * bits that FP64 keeps (a component far below the others that does not mix with them). */
 typedef enum { ODWF_F64 = 0, ODWF_F32 = 1, ODWF_F16 = 2, ODWF_BF16 = 3, ODWF_FF = 4 } odwf_prec;
 
 enum { ODWF_MODE_FULL = 0, ODWF_MODE_SCHUR_EVEN = 1 };

@@ -3,13 +3,14 @@
 // a non-dagger hop reads (1 + L) psi, written by the kernel that produced it.
 //
 // What bounds it: three pipes at about half each, 5 blocks of 128 threads per SM overlapping phases.
-// Per 5D site a hop takes 1728 integer multiply-adds at 32 per clock and SM (54 clocks) and, at 2 per
+// Per 5D site a hop takes 1728 integer multiply-adds at about 28 per clock and SM (62 clocks) and, at 2 per
 // clock and SM, 120 to 190 FP64 operations (60 to 95 clocks): conversions of the 24 sums, 3 per real for
 // a solve along s, 1 to 2 for a bidiagonal operator.  16^3x32x16, one system, the four hops of S^dag S:
-// 0.44 / 0.55 / 0.46 / 0.53 ms at 50 to 62% FP64 pipe (FP64 stencil, 1334 to 1700 FP64 operations: 2.6 to
+// 0.42 / 0.53 / 0.44 / 0.54 ms at 52 to 72% FP64 pipe (FP64 stencil, 1334 to 1700 FP64 operations: 2.6 to
 // 3.0 ms; one thread per 5D site at 168 registers: 0.57 / 0.69 / 0.61 / 0.49 ms; with the two threads in
 // adjacent lanes a quarter warp touched four lines: 0.47 / 0.57 / 0.51 / 0.54 ms).  Four blocks per SM
-// take 10% longer, six spill.
+// take 10% longer, six spill.  Warps that meet what fixed point cannot hold take other routes, fx_hop_conv and
+// fx_hop_f64.
 #pragma once
 
 #include "fx.cuh"

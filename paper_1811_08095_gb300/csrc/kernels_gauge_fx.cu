@@ -2,7 +2,7 @@
 // integer pipe.
 //
 // Thirteen SU(3) products per link are 1400 FP64 operations on a pipe of 2 per clock and SM; as 31-bit
-// limbs (fx.cuh) they are 4212 integer multiply-adds at 32 per clock and SM.  Entries of SU(3) matrices
+// limbs (fx.cuh) they are 4212 integer multiply-adds at about 28 per clock and SM.  Entries of SU(3) matrices
 // are at most 1, so every link has 60 fraction bits and no exponent; products are kept to 2^-58, staples
 // and U Sigma to 2^-56, against 2^-53 of each FP64 operation.  Fields whose rows or columns are not of
 // unit length to 2^-16 (the entry points take any matrices) raise a flag in the pass that splits the
@@ -12,17 +12,18 @@
 // Where the links have one large entry per row (near the unit field, or an abelian one) the force comes from
 // the small entries, whose products FP64 keeps to 2^-53 of themselves and limbs to 2^-58 of 1.  With links
 // exp(i eps H) both err by 1.4e-16 of the force (rms, FP64 at every eps) at eps = 0.035, where the off-diagonal
-// entries are about 2^-6; the limbs by 1.0e-16 at 0.25, 2.1e-16 at 0.02 and 3.7e-15 at 0.001.  The pass that splits the links marks those
-// whose other six entries are below 2^-6; the FP64 kernel takes the marked ones and this one the others, each
-// adding to its block's sum.  From one marked link in 64 the whole field goes to the FP64 kernel, since a warp that
-// holds one takes as long there as a full one: 0.50 ms at eps = 0.25, 0.58 at 0.1, 1.29 at 0.05, 2.07 from 0.03 down.
+// entries are about 2^-6; the limbs by 1.0e-16 at 0.25, 2.1e-16 at 0.02 and 3.7e-15 at 0.001.  The pass that
+// splits the links marks those whose other six entries are below 2^-6; the FP64 kernel takes the marked ones
+// and this one the others, each adding to its block's sum.  From one marked link in 64 the whole field goes to
+// the FP64 kernel, since a warp that holds one takes as long there as a full one.  16^3x32: 0.50 ms at eps =
+// 0.25, 0.58 at 0.1, 1.29 at 0.05, 2.07 from 0.03 down.
 //
 // Splitting the links where they are used instead of in a pass before gives the same bits and needs no
 // workspace for the limbs, but takes twice as long (16^3x32 1.03 ms; 8^4, where the chip is not full, 88 us
 // against 57): for calls that would have to allocate it first, see Engine::gauge_force.
 //
-// 16^3x32, action and force: 2.04 ms in FP64, 0.50 ms here (split 25 us, force 0.44 ms); bound by
-// the latency of the integer chains with the 8 warps per SM that 244 registers leave (three blocks per
+// 16^3x32, action and force: 2.04 ms in FP64, 0.50 ms here (split 27 us, force 0.44 ms); bound by
+// the latency of the integer chains with the 8 warps per SM that 252 registers leave (three blocks per
 // SM spill 300 bytes: 0.50 ms, four 0.56 ms).
 //
 // Bounds: entries of a product of unit-row matrices are at most 1, of a staple sqrt(3), of six 10.4

@@ -24,7 +24,7 @@ namespace {
 constexpr double kOmelyanLambda = 0.1931833275037836;
 // An allocation of up to 1 MB comes from the 2 MB blocks that small allocations share; a larger one costs the call
 // that makes it 90 us.  Up to 16384 sites (9 MB of limbs) that call is faster splitting the links where they
-// are used, with the allocation beside its kernels: 8^4 154 -> 140 us, 8^3x16 165 -> 145, 8^2x16^2 200 -> 198;
+// are used, with the allocation beside its kernels: 8^4 154 -> 125-140 us, 8^3x16 165 -> 130-140, 8^2x16^2 200 -> 196;
 // 12^3x24 would take 390 instead of 290.
 constexpr size_t kDirectBytes = 1 << 20, kDirectSites = 16384;
 }
