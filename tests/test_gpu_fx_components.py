@@ -121,6 +121,19 @@ def test_spins_of_different_size(torch, ratio):
             assert size < 1e3 * ratio and err <= 1e-13 * size
 
 
+@pytest.mark.parametrize("ns", [2, 16, 32])
+@pytest.mark.parametrize("ratio", [2.0 ** -7, 1e-3, 1e-12, 1e-40])
+def test_small_colours_on_dense_links(torch, ratio, ns):
+    """Links that mix colours: sites keep FP64 bits, and the fixed-point stencil converts them where it reads them.
+    Every other site, so that both kinds of neighbours meet."""
+    dims = (4, 2, 6, 4)
+    U, w = make_case(dims, ns, MQ, eps=0.7, seed=6)
+    psi = syn.gaussian_spinor(ns, dims, 14)
+    psi[:, :, ::2, :, :, :, 1:] *= ratio
+    for got, ref in _ops(torch, dims, ns, U, w, psi, True):
+        _check_colours(got, ref)
+
+
 def test_noise_off_the_diagonal(torch):
     """A free field as an eigendecomposition makes it: 1e-15 off the diagonal, a colour at that level."""
     dims, ns = (4, 4, 2, 6), 16
