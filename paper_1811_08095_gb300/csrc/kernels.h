@@ -103,7 +103,9 @@ cudaError_t launch_hop_mixed(const HopParams<float>& P, Epi e, Sp low, Lk lk, in
 // Launches of at most 16384 half-precision 5D sites (all systems) take the one-s-per-lane kernels with
 // every neighbour fetched up front: they are bound by the chain of memory latencies of one block.  One
 // GB300, FP16: 4^4x8 (1024 sites) K1 6.2 -> 4.2 us, K2 10.2 -> 8.3; 8^4x8 (16384) K2 10.4 -> 8.3, K4
-// 11.5 -> 10.3; 8^4x16 (32768) K2 10.6 -> 12.4.
+// 11.5 -> 10.3; 8^4x16 (32768) K2 10.6 -> 12.4.  Whole iterations with these kernels / the others, one system of 8^3
+// x Lt: 16384 sites 28.7 / 33.7 us, 20480 32.0 / 34.9, 32768 33.9 / 35.5, 40960 to 57344 equal, 65536 52.7 / 44.2; the two
+// are equal near 40960, so the line is on the safe side of it by a factor of 2.5.
 bool hop_deep(Sp low, size_t n5);
 bool hop2_supported(int ns, Sp low, size_t vh);
 cudaError_t launch_hop2(const HopParams<float>& P, int kind, Sp low, Lk lk, int nsys, cudaStream_t st);
@@ -126,7 +128,8 @@ cudaError_t launch_p_update2(Sp low, int ns, const FieldRef& r, const FieldRef& 
 // K4 partials of all systems of a launch up to which the p update forms beta itself (launch_p_update2 with
 // nb > 0).  It saves a launch but every block waits for the sum and the division: per iteration 23.4 -> 22.2
 // us on 4^4x8 (16 partials), 38.2 -> 37.2 on 8^3x16x16 (256), but 61.2 -> 63.9 for eight systems on 8^4x8
-// (512) and 118 -> 124 on 12^3x24x16 (1296).
+// (512) and 118 -> 124 on 12^3x24x16 (1296).  Between, with it / without, one system of Ns = 16: 320 partials 54.6 / 55.7
+// us, 400 56.6 / 58.0, 480 69.6 / 68.8, 600 75.6 / 74.7: the two are equal near 450, the line is on the safe side.
 constexpr int kBetaInUpdate = 256;
 
 // Site-local M, M^dag, M^-1, M^-dag (op 0..3); op 4 = B (the chiral shift rho + sigma L)
