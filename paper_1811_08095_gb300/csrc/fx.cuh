@@ -31,8 +31,8 @@
 // 1 to exp(0.7 i H), for fields that fall by e^-0.7 per s and per chirality or by e^-1.2 per site, and for a colour
 // 1 to 2^-30 of the others on diagonal links (1.1e-16 rms at every ratio, FP64 1.1e-16; without the tests 8e-16 at
 // 2^-7 and 4e-10 at 2^-30).
-// Non-finite values, denormals and sums near the ends of the exponent range take the FP64 stencil at once (exponent
-// kFxHard), so NaN and Inf propagate as in FP64.  (Components below 2^-1042 beside one above 2^-958 count as zero.)
+// Non-finite values, sites below 2^-958 (both with exponent kFxHard) and sums near the ends of the exponent range take
+// the FP64 stencil at once, so NaN and Inf propagate as in FP64.  (Components below 2^-1042 beside one above 2^-958 count as zero.)
 //
 // A link array holds nine (re1, re0, im1, im0) records per link, rows first, in the order of the FP64
 // links ((p * 4 + mu) * Vh + h), and one exponent each behind them (kFxHard: a non-finite link).
